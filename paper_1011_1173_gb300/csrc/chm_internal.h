@@ -160,8 +160,8 @@ int pass_enqueue(void *L, long long n, long long ld, const void *V, long long ld
                  const int8_t *sigma, int sign, int dtype, cudaStream_t stream, long long *d_info,
                  const PassChoice &ch, const Scratch &sc, PassSpace &ps, void *B = nullptr, long long ldb = 0,
                  long long nrhs = 0);
-// The solve's scratch for a factor of order n (chm_solve.cu).
-ScratchNeed solve_need(long long n);
+// The scratch of a solve of nrhs right-hand sides with a factor of order n (chm_solve.cu).
+ScratchNeed solve_need(long long n, long long nrhs);
 // chm_solve's forward and back substitution on `sc` (which holds solve_need).
 int solve_enqueue(const void *L, long long n, long long ld, void *B, long long ldb, long long nrhs, int dtype,
                   const Scratch &sc, cudaStream_t stream);

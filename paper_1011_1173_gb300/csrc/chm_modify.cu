@@ -505,7 +505,7 @@ static int modify_solve_dispatch(void *L, long long n, long long ld, const void 
     if (ch.path == 2) {
         // the solve's scratch first (the stream's workspace, grown under its
         // own hold of the lock), then the passes on the same workspace
-        if ((rc = with_stream_scratch(stream, solve_need(n), [](const Scratch &) { return (int)CHM_OK; })) != CHM_OK)
+        if ((rc = with_stream_scratch(stream, solve_need(n, nrhs), [](const Scratch &) { return (int)CHM_OK; })) != CHM_OK)
             return rc;
         return with_pass_workspace(stream, pass_workspace_bytes(n, dtype, ch.seg), n, dtype,
                                    [&](const Scratch &sc, PassSpace &ps) {

@@ -1,23 +1,34 @@
 // Solve with a factor: B <- (L^T L)^{-1} B, the use a maintained Cholesky
 // factor serves (Sec. 1).  A forward substitution with L^T (lower) followed
 // by a back substitution with L (upper), both blocked by kW = 32 rows, in
-// one persistent launch per group of up to four right-hand sides.
+// one persistent launch per group of right-hand sides.
 //
-// Tasks, taken in order from a launch-wide counter by blocks of four warps:
-//   t <  nb: forward task for block b = t:  y_b = D_b^{-T} (b_b - sum_{p<b} L_{p,b}^T y_p)
-//   t >= nb: backward task for b = 2nb-1-t: x_b = D_b^{-1} (y_b - sum_{q>b} L_{b,q} x_q)
-// where D_b is the diagonal block and L_{p,b} the 32 x 32 tile in row block
-// p and column block b.  A task waits only on tasks taken before it, so the
-// launch cannot deadlock whatever the number of resident blocks.
+// A launch runs C chains of R right-hand sides each.  Tasks are taken in
+// order from a launch-wide counter by blocks of four warps:
+//   t < nb: prepare block b = t: U_b = D_b^{-1}, G_b = U_b^T L_{b-1,b}^T and
+//     H_b = U_b L_{b,b+1} (D_b the diagonal block, L_{p,b} the 32 x 32 tile in
+//     row block p and column block b), shared by every chain;
+//   then, dealt round-robin to the chains, step s = 0 .. 2 nb - 1 of each:
+//     s <  nb: y_b = D_b^{-T} (b_b - sum_{p<b} L_{p,b}^T y_p), b = s
+//     s >= nb: x_b = D_b^{-1} (y_b - sum_{q>b} L_{b,q} x_q), b = 2 nb - 1 - s
+// A task waits only on tasks taken before it, so the launch cannot deadlock
+// whatever the number of resident blocks.
 //
-// Each forward task inverts its diagonal block (U_b = D_b^{-1}, one column
-// per lane) and forms G_b = U_b^T L_{b-1,b}^T while its warps accumulate the
-// tiles whose y is already published, and z_b = U_b^T (b_b - sum over
-// p <= b-2) once y_{b-2} is in; then y_b = z_b - G_b y_{b-1}.  The backward
-// task reuses U_b and forms H_b = U_b L_{b,b+1}: x_b = z'_b - H_b x_{b+1}.
-// Between one block's result and the next block's there is one 32 x 32
-// product (eight FMAs per warp), one barrier and a four-way sum.  Results
-// pass between blocks as epoch-tagged doubles (no fence, no flag).
+// A forward step sums the tiles whose y is already published, forms
+// z_b = U_b^T (b_b - sum over p <= b-2) once y_{b-2} is in, and then
+// y_b = z_b - G_b y_{b-1}; a backward step mirrors it with H_b.  Between one
+// block's result and the next block's there is one 32 x 32 product (eight
+// FMAs per warp and right-hand side), one barrier and a four-way sum.
+// Results pass between blocks as epoch-tagged doubles (no fence, no flag).
+//
+// Why chains: right-hand sides do not depend on each other, and a step is
+// bound by FP64 issue (one FP64 instruction per 64 cycles and warp), so a
+// step of four right-hand sides takes three times a step of one.  C chains
+// side by side fill the SMs that one chain leaves idle; the tiles they share
+// meet in L2, and U, G and H are formed once instead of once per four
+// right-hand sides.  n = 5000, float64, 16 right-hand sides: 1.13 ms in 16
+// chains against 6.96 ms as four launches of four right-hand sides each; the
+// FP64 rate allows 0.76 ms (400 M FMAs).
 #include <float.h>
 
 #include <algorithm>
@@ -32,8 +43,10 @@ namespace {
 
 constexpr int kSolveThreads = 128;
 constexpr int kSolveWarps = kSolveThreads / 32;
-constexpr int kSolveRhs = 4;                       // right-hand sides per launch (largest)
+constexpr int kSolveRhs = 4;                       // right-hand sides per chain (largest)
+constexpr int kSolveChains = 16;                   // chains per launch (largest)
 constexpr int kRowsPerWarp = kW / kSolveWarps;     // rows (or columns) of a split tile per warp
+constexpr int kPrepMats = 3;                       // U_b, G_b and H_b
 constexpr unsigned kFull = 0xffffffffu;
 
 template <typename T>
@@ -43,20 +56,22 @@ struct SolveArgs {
     T *B;
     long long ldb;
     int nb;           // blocks of kW rows
-    int nr;           // right-hand sides of this launch (1 .. R)
+    int nr;           // right-hand sides of this launch (1 .. C R)
+    int chains;       // C: chain c takes right-hand sides c R .. c R + R - 1
     // back substitution only: y = L^{-T} b is given, row i of right-hand
     // side r at Y[i * ys + r * cs] (chm_modify_solve's pass forms it)
     const T *Y;
     long long ys, cs;
     int back_only;
-    double *inv;      // [nb][kW][kW]: U_b = D_b^{-1}, row i at i * kW
-    int *yflag;       // [nb]: y_b and U_b published (== epoch)
-    long long *ytag;  // [nb][kW][R][2]: y_b as tagged doubles
-    long long *xtag;  // [nb][kW][R][2]: x_b as tagged doubles
+    double *inv;      // [nb][kPrepMats][kW][kW]: U_b = D_b^{-1} (row i at i * kW), G_b and H_b
+                      // (transposed: element (i, j) at j * kW + i)
+    int *uflag;       // [nb]: U_b, G_b and H_b published (== epoch)
+    long long *ytag;  // [C][nb][kW][R][2]: y_b as tagged doubles
+    long long *xtag;  // [C][nb][kW][R][2]: x_b as tagged doubles
     int *ctl;
     long long *status;
     long long timeout_ns;
-    // the workspace allocations inv, yflag and ytag / xtag are carved from (bounds-checked builds)
+    // the workspace allocations inv, uflag and ytag / xtag are carved from (bounds-checked builds)
     const char *ws_data;
     size_t ws_data_bytes;
     const int *ws_iflags;
@@ -66,13 +81,21 @@ struct SolveArgs {
     long long chk_cut;
 };
 
-template <int R>
-struct SolveSmem {
+// Shared memory of a block: a preparation task's matrices or a step's
+// partial sums.
+struct PrepSmem {
     double D[kW][kW + 1];  // diagonal block (row, column); identity beyond the order
     double U[kW][kW + 1];  // its inverse
-    double T[kW][kW + 1];  // the tile next to the diagonal block (see the tasks)
-    double part[2][kSolveWarps][R][kW];
+    double T[kW][kW + 1];  // the tile above it, then the tile to its right
+    double M[kW / 2][kW / 2 + 1];
     double rd[kW];         // 1 / D_ii
+};
+template <int R>
+struct SolveSmem {
+    union {
+        PrepSmem prep;
+        double part[2][kSolveWarps][R][kW];
+    };
 };
 
 template <int R>
@@ -131,15 +154,19 @@ __device__ __forceinline__ double part_sum(const SolveSmem<R> &S, int buf, int r
     return (S.part[buf][0][r][lane] + S.part[buf][1][r][lane]) + (S.part[buf][2][r][lane] + S.part[buf][3][r][lane]);
 }
 
-template <typename T, int R>
-__device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int b, SolveSmem<R> &S)
+// U_b, G_b and H_b of block b.  The inverse goes by halves: with
+// D = [[D1, B], [0, D2]], U = [[U1, -U1 B U2], [0, U2]]; the two 16 x 16
+// inverses take one warp (a column per lane, 136 dependent FMAs instead of
+// the 528 of a whole column each) and the products all four.
+template <typename T>
+__device__ void prep_task(const SolveArgs<T> &a, const SyncArgs &sy, int b, PrepSmem &S)
 {
+    constexpr int kH = kW / 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long ld = a.ld;
+    const long long n = a.n, ld = a.ld;
     const long long c0 = (long long)b * kW;
-    const int nc = (int)min((long long)kW, a.n - c0);
-    const bool active = lane < nc;
-    const long long who = b;
+    const int nc = (int)min((long long)kW, n - c0);
+    const bool above = b >= 1 && !a.back_only;  // G_b serves the forward steps only
 
     // the diagonal block (identity beyond the order) and the tile above it,
     // S.T[j][m] = L[(b-1) kW + j, c0 + m]
@@ -147,28 +174,16 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
         const int i = e & (kW - 1), j = e / kW;
         double v = 0.0;
         if (j < nc) {
-            if (i <= j && CHK_TRI(sy, c0 + i + (c0 + j) * ld, a.n, ld)) v = (double)__ldg(a.L + c0 + i + (c0 + j) * ld);
+            if (i <= j && CHK_TRI(sy, c0 + i + (c0 + j) * ld, n, ld)) v = (double)__ldg(a.L + c0 + i + (c0 + j) * ld);
         } else if (i == j) {
             v = 1.0;
         }
         S.D[i][j] = v;
-        if (b >= 1)
-            S.T[i][j] = (j < nc && CHK_TRI(sy, c0 - kW + i + (c0 + j) * ld, a.n, ld))
+        if (above)
+            S.T[i][j] = (j < nc && CHK_TRI(sy, c0 - kW + i + (c0 + j) * ld, n, ld))
                             ? (double)__ldg(a.L + c0 - kW + i + (c0 + j) * ld) : 0.0;
     }
-    double rhs[R];
-    if (a.back_only) {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            rhs[r] = (active && r < a.nr) ? (double)__ldcg(a.Y + (c0 + lane) * a.ys + r * a.cs) : 0.0;
-    } else {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            rhs[r] = (active && r < a.nr && CHK_RECT(sy, c0 + lane + r * a.ldb, a.n, a.nr, a.ldb))
-                         ? (double)a.B[c0 + lane + r * a.ldb] : 0.0;
-    }
     __syncthreads();
-
     if (warp == 0) {
         double d = S.D[lane][lane];
         if (!(d > 0.0 && d <= DBL_MAX)) {  // not a Cholesky factor
@@ -177,49 +192,111 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
         }
         S.rd[lane] = 1.0 / d;
         __syncwarp();
-        // column `lane` of U = D^{-1}: back substitution on D u = e_lane
-        double u[kW];
+        // column `col` of the inverse of diagonal half h: back substitution on D_h u = e_col
+        const int h = lane & kH, col = lane & (kH - 1);
+        double u[kH];
 #pragma unroll
-        for (int i = kW - 1; i >= 0; --i) {
-            double s = (i == lane) ? 1.0 : 0.0;
+        for (int i = kH - 1; i >= 0; --i) {
+            double s = (i == col) ? 1.0 : 0.0;
 #pragma unroll
-            for (int m = i + 1; m < kW; ++m) s = fma(-S.D[i][m], u[m], s);
-            u[i] = s * S.rd[i];
+            for (int m = i + 1; m < kH; ++m) s = fma(-S.D[h + i][h + m], u[m], s);
+            u[i] = s * S.rd[h + i];
         }
-        double *inv = a.inv + (size_t)b * kW * kW;
 #pragma unroll
-        for (int i = 0; i < kW; ++i) {
-            S.U[i][lane] = u[i];
-            __stcg(inv + i * kW + lane, u[i]);
-        }
-    }
-
-    __syncthreads();  // U in shared memory
-
-    if (a.back_only) {
-        // y_b is given: publish it with U_b for this block's backward task
-        if (warp == 0) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) put_tagged(a.ytag + tag_at<R>(b, lane, r), rhs[r], ep64);
-            __syncwarp();
-            if (lane == 0) st_release_gpu(a.yflag + b, sy.epoch);
-        }
-        return;
-    }
-
-    // G = U^T S.T^T, the rows j of S.T split over the warps:
-    // g[jj] = G[lane][warp * 8 + jj] = sum_m U[m][lane] S.T[warp * 8 + jj][m]
-    double g[kRowsPerWarp];
-#pragma unroll
-    for (int jj = 0; jj < kRowsPerWarp; ++jj) g[jj] = 0.0;
-    if (b >= 1) {
-#pragma unroll
-        for (int m = 0; m < kW; ++m) {
-            const double um = S.U[m][lane];
-#pragma unroll
-            for (int jj = 0; jj < kRowsPerWarp; ++jj) g[jj] = fma(um, S.T[warp * kRowsPerWarp + jj][m], g[jj]);
+        for (int i = 0; i < kH; ++i) {
+            S.U[h + i][h + col] = u[i];
+            if (h) S.U[h + i][col] = 0.0;
         }
     }
+    __syncthreads();
+    // M = B U2, then U12 = -U1 M: two outputs a thread, a row pair per half warp
+    const int mi = threadIdx.x / kH, mj = threadIdx.x & (kH - 1);
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        const int i = mi + 8 * v;
+        double s = 0.0;
+#pragma unroll
+        for (int m = 0; m < kH; ++m) s = fma(S.D[i][kH + m], S.U[kH + m][kH + mj], s);
+        S.M[i][mj] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        const int i = mi + 8 * v;
+        double s = 0.0;
+#pragma unroll
+        for (int m = 0; m < kH; ++m) s = fma(S.U[i][m], S.M[m][mj], s);
+        S.U[i][kH + mj] = -s;
+    }
+    __syncthreads();
+    double *inv = a.inv + (size_t)b * kPrepMats * kW * kW;
+    for (int e = threadIdx.x; e < kW * kW; e += kSolveThreads) __stcg(inv + e, S.U[e / kW][e & (kW - 1)]);
+    // G: G[i][j] = sum_{m<=i} U[m][i] T[j][m]; rows i = warp, warp + 4, ... (so
+    // that the four warps' triangles weigh the same), lane = j
+    if (above) {
+        for (int ii = 0; ii < kRowsPerWarp; ++ii) {
+            const int i = ii * kSolveWarps + warp;
+            double s0 = 0.0, s1 = 0.0;
+            for (int m = 0; m <= i; m += 2) {
+                s0 = fma(S.U[m][i], S.T[lane][m], s0);
+                if (m < i) s1 = fma(S.U[m + 1][i], S.T[lane][m + 1], s1);
+            }
+            __stcg(inv + kW * kW + (size_t)lane * kW + i, s0 + s1);
+        }
+    }
+    // H: H[i][j] = sum_{m>=i} U[i][m] T[m][j], T the tile to the right of the diagonal block
+    if (b + 1 < a.nb) {
+        __syncthreads();
+        const long long q1 = c0 + kW;
+        const int nc1 = (int)min((long long)kW, n - q1);
+        for (int e = threadIdx.x; e < kW * kW; e += kSolveThreads) {
+            const int i = e & (kW - 1), j = e / kW;
+            S.T[i][j] = (j < nc1 && CHK_TRI(sy, c0 + i + (q1 + j) * ld, n, ld)) ? (double)__ldg(a.L + c0 + i + (q1 + j) * ld)
+                                                                                : 0.0;
+        }
+        __syncthreads();
+        for (int ii = 0; ii < kRowsPerWarp; ++ii) {
+            const int i = ii * kSolveWarps + warp;
+            double s0 = 0.0, s1 = 0.0;
+            for (int m = kW - 1; m >= i; m -= 2) {
+                s0 = fma(S.U[i][m], S.T[m][lane], s0);
+                if (m > i) s1 = fma(S.U[i][m - 1], S.T[m - 1][lane], s1);
+            }
+            __stcg(inv + 2 * kW * kW + (size_t)lane * kW + i, s0 + s1);
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) st_release_gpu(a.uflag + b, sy.epoch);
+}
+
+// The block's four warps wait for U_b, G_b and H_b; false if the wait gave up.
+template <typename T>
+__device__ __forceinline__ bool wait_prep(const SolveArgs<T> &a, const SyncArgs &sy, int b)
+{
+    const bool ok = __all_sync(kFull, wait_eq(sy, a.uflag + b, sy.epoch, b));
+    __syncwarp();
+    return ok;
+}
+
+// Chain c's step at block b, forward.
+template <typename T, int R>
+__device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int c, int b, SolveSmem<R> &S)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long ld = a.ld;
+    const long long c0 = (long long)b * kW;
+    const int nc = (int)min((long long)kW, a.n - c0);
+    const bool active = lane < nc;
+    const long long who = b;
+    const int r0 = c * R;  // this chain's first right-hand side
+    long long *ytag = a.ytag + (size_t)c * a.nb * kW * R * 2;
+
+    double rhs[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        rhs[r] = (active && r0 + r < a.nr && CHK_RECT(sy, c0 + lane + (r0 + r) * a.ldb, a.n, a.nr, a.ldb))
+                     ? (double)a.B[c0 + lane + (r0 + r) * a.ldb] : 0.0;
     // tiles p <= b - 3 of column block b, dealt round-robin to the warps (a
     // fixed order of the sums: results do not depend on timing); lane =
     // column of the block, the tile's 32 rows read down the column
@@ -235,11 +312,21 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
         for (int j = 0; j < kW; ++j)
             t[j] = (active && CHK_TRI(sy, colo + (long long)p * kW + j, a.n, ld)) ? (double)__ldg(src + j) : 0.0;
         double yv[R];
-        wait_block<R>(sy, a.ytag, ep64, p, who, yv);
+        wait_block<R>(sy, ytag, ep64, p, who, yv);
 #pragma unroll
         for (int j = 0; j < kW; ++j)
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = fma(t[j], __shfl_sync(kFull, yv[r], j), acc[r]);
+    }
+    // this warp's rows of U_b and columns of G_b (see the products below)
+    const bool ok = wait_prep(a, sy, b);
+    const double *inv = a.inv + (size_t)b * kPrepMats * kW * kW;
+    double u[kRowsPerWarp], g[kRowsPerWarp];
+#pragma unroll
+    for (int jj = 0; jj < kRowsPerWarp; ++jj) {
+        const int j = warp * kRowsPerWarp + jj;
+        u[jj] = ok ? __ldcg(inv + j * kW + lane) : 0.0;
+        g[jj] = (ok && b >= 1) ? __ldcg(inv + kW * kW + j * kW + lane) : 0.0;
     }
     // tile b - 2: its rows split over the warps
     if (b >= 2) {
@@ -248,7 +335,7 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
 #pragma unroll
         for (int jj = 0; jj < kRowsPerWarp; ++jj) t[jj] = active ? (double)__ldg(src + jj) : 0.0;
         double yv[R];
-        wait_block<R>(sy, a.ytag, ep64, b - 2, who, yv);
+        wait_block<R>(sy, ytag, ep64, b - 2, who, yv);
 #pragma unroll
         for (int jj = 0; jj < kRowsPerWarp; ++jj)
 #pragma unroll
@@ -268,9 +355,8 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
 #pragma unroll
     for (int jj = 0; jj < kRowsPerWarp; ++jj) {
         const int j = warp * kRowsPerWarp + jj;
-        const double uji = S.U[j][lane];
 #pragma unroll
-        for (int r = 0; r < R; ++r) pz[r] = fma(uji, __shfl_sync(kFull, rv[r], j), pz[r]);
+        for (int r = 0; r < R; ++r) pz[r] = fma(u[jj], __shfl_sync(kFull, rv[r], j), pz[r]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) S.part[1][warp][r][lane] = pz[r];
@@ -278,14 +364,14 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
     double z[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) z[r] = part_sum(S, 1, r, lane);
-    __syncthreads();  // part[0] free again
+    // (part[0] is free again: every warp read it before the barrier above)
     // y_b = z_b - G_b y_{b-1}: the step that waits on the previous block
     double py[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) py[r] = 0.0;
     if (b >= 1) {
         double yv[R];
-        wait_block<R>(sy, a.ytag, ep64, b - 1, who, yv, true);
+        wait_block<R>(sy, ytag, ep64, b - 1, who, yv, true);
 #pragma unroll
         for (int jj = 0; jj < kRowsPerWarp; ++jj)
 #pragma unroll
@@ -297,15 +383,13 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) put_tagged(a.ytag + tag_at<R>(b, lane, r), z[r] - part_sum(S, 0, r, lane), ep64);
-        __syncwarp();
-        // U_b and y_b for this block's backward task
-        if (lane == 0) st_release_gpu(a.yflag + b, sy.epoch);
+        for (int r = 0; r < R; ++r) put_tagged(ytag + tag_at<R>(b, lane, r), z[r] - part_sum(S, 0, r, lane), ep64);
     }
 }
 
+// Chain c's step at block b, backward.
 template <typename T, int R>
-__device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int b,
+__device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int c, int b,
                               SolveSmem<R> &S)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -315,36 +399,23 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
     const bool active = lane < nc;
     const long long who = b;
     const bool has_next = b + 1 < a.nb;
+    const int r0 = c * R;
+    long long *xtag = a.xtag + (size_t)c * a.nb * kW * R * 2;
 
-    (void)__all_sync(kFull, wait_eq(sy, a.yflag + b, sy.epoch, who));
-    __syncwarp();
-    // U_b, and the tile to its right, S.T[m][j] = L[c0 + m, (b+1) kW + j]
-    const double *inv = a.inv + (size_t)b * kW * kW;
-    const long long q1 = (long long)(b + 1) * kW;
-    const int nc1 = has_next ? (int)min((long long)kW, n - q1) : 0;
-    for (int e = threadIdx.x; e < kW * kW; e += kSolveThreads) {
-        const int i = e / kW, j = e & (kW - 1);
-        S.U[i][j] = __ldcg(inv + e);
-        S.T[j][i] = (has_next && j < nc && i < nc1 && CHK_TRI(sy, c0 + j + (q1 + i) * ld, n, ld))
-                        ? (double)__ldg(a.L + c0 + j + (q1 + i) * ld) : 0.0;
+    // this warp's columns of U_b and H_b (see the products below)
+    const bool ok = wait_prep(a, sy, b);
+    const double *inv = a.inv + (size_t)b * kPrepMats * kW * kW;
+    double u[kRowsPerWarp], h[kRowsPerWarp];
+#pragma unroll
+    for (int jj = 0; jj < kRowsPerWarp; jj += 2) {
+        const int j = warp * kRowsPerWarp + jj;
+        const double2 v = ok ? __ldcg(reinterpret_cast<const double2 *>(inv + lane * kW + j)) : make_double2(0.0, 0.0);
+        u[jj] = v.x;
+        u[jj + 1] = v.y;
     }
-    double yv[R];
-    wait_block<R>(sy, a.ytag, ep64, b, who, yv);
-    __syncthreads();
-
-    // H = U S.T, the columns j of S.T split over the warps:
-    // h[jj] = H[lane][warp * 8 + jj] = sum_m U[lane][m] S.T[m][warp * 8 + jj]
-    double h[kRowsPerWarp];
 #pragma unroll
-    for (int jj = 0; jj < kRowsPerWarp; ++jj) h[jj] = 0.0;
-    if (has_next) {
-#pragma unroll
-        for (int m = 0; m < kW; ++m) {
-            const double um = S.U[lane][m];
-#pragma unroll
-            for (int jj = 0; jj < kRowsPerWarp; ++jj) h[jj] = fma(um, S.T[m][warp * kRowsPerWarp + jj], h[jj]);
-        }
-    }
+    for (int jj = 0; jj < kRowsPerWarp; ++jj)
+        h[jj] = (ok && has_next) ? __ldcg(inv + 2 * kW * kW + (warp * kRowsPerWarp + jj) * kW + lane) : 0.0;
 
     // tiles q >= b + 3 of row block b, from the last one up, dealt
     // round-robin to the warps; lane = row of the block, so each column of a
@@ -359,14 +430,14 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
         const int ncq = (int)min((long long)kW, n - q0);
         double t[kW];
 #pragma unroll
-        for (int c = 0; c < kW; ++c)
-            t[c] = (active && c < ncq && CHK_TRI(sy, rowo + (q0 + c) * ld, n, ld)) ? (double)__ldg(row + (q0 + c) * ld) : 0.0;
+        for (int i = 0; i < kW; ++i)
+            t[i] = (active && i < ncq && CHK_TRI(sy, rowo + (q0 + i) * ld, n, ld)) ? (double)__ldg(row + (q0 + i) * ld) : 0.0;
         double xv[R];
-        wait_block<R>(sy, a.xtag, ep64, q, who, xv);
+        wait_block<R>(sy, xtag, ep64, q, who, xv);
 #pragma unroll
-        for (int c = 0; c < kW; ++c)
+        for (int i = 0; i < kW; ++i)
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] = fma(t[c], __shfl_sync(kFull, xv[r], c), acc[r]);
+            for (int r = 0; r < R; ++r) acc[r] = fma(t[i], __shfl_sync(kFull, xv[r], i), acc[r]);
     }
     // tile b + 2: its columns split over the warps
     if (b + 2 < a.nb) {
@@ -375,16 +446,25 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
         double t[kRowsPerWarp];
 #pragma unroll
         for (int cc = 0; cc < kRowsPerWarp; ++cc) {
-            const int c = warp * kRowsPerWarp + cc;
-            t[cc] = (active && c < ncq && CHK_TRI(sy, rowo + (q0 + c) * ld, n, ld)) ? (double)__ldg(row + (q0 + c) * ld) : 0.0;
+            const int i = warp * kRowsPerWarp + cc;
+            t[cc] = (active && i < ncq && CHK_TRI(sy, rowo + (q0 + i) * ld, n, ld)) ? (double)__ldg(row + (q0 + i) * ld) : 0.0;
         }
         double xv[R];
-        wait_block<R>(sy, a.xtag, ep64, b + 2, who, xv);
+        wait_block<R>(sy, xtag, ep64, b + 2, who, xv);
 #pragma unroll
         for (int cc = 0; cc < kRowsPerWarp; ++cc)
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 acc[r] = fma(t[cc], __shfl_sync(kFull, xv[r], warp * kRowsPerWarp + cc), acc[r]);
+    }
+    // y_b: this chain's forward result, or the caller's
+    double yv[R];
+    if (a.back_only) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            yv[r] = (active && r0 + r < a.nr) ? (double)__ldcg(a.Y + (c0 + lane) * a.ys + (r0 + r) * a.cs) : 0.0;
+    } else {
+        wait_block<R>(sy, a.ytag + (size_t)c * a.nb * kW * R * 2, ep64, b, who, yv);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) S.part[0][warp][r][lane] = acc[r];
@@ -399,9 +479,8 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
 #pragma unroll
     for (int jj = 0; jj < kRowsPerWarp; ++jj) {
         const int j = warp * kRowsPerWarp + jj;
-        const double uij = S.U[lane][j];
 #pragma unroll
-        for (int r = 0; r < R; ++r) pz[r] = fma(uij, __shfl_sync(kFull, rv[r], j), pz[r]);
+        for (int r = 0; r < R; ++r) pz[r] = fma(u[jj], __shfl_sync(kFull, rv[r], j), pz[r]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) S.part[1][warp][r][lane] = pz[r];
@@ -409,14 +488,13 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
     double z[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) z[r] = part_sum(S, 1, r, lane);
-    __syncthreads();  // part[0] free again
     // x_b = z'_b - H_b x_{b+1}: the step that waits on the previous block
     double px[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) px[r] = 0.0;
     if (has_next) {
         double xv[R];
-        wait_block<R>(sy, a.xtag, ep64, b + 1, who, xv, true);
+        wait_block<R>(sy, xtag, ep64, b + 1, who, xv, true);
 #pragma unroll
         for (int jj = 0; jj < kRowsPerWarp; ++jj)
 #pragma unroll
@@ -430,8 +508,9 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const double x = z[r] - part_sum(S, 0, r, lane);
-            put_tagged(a.xtag + tag_at<R>(b, lane, r), x, ep64);
-            if (active && r < a.nr && CHK_RECT(sy, c0 + lane + r * a.ldb, a.n, a.nr, a.ldb)) a.B[c0 + lane + r * a.ldb] = (T)x;
+            put_tagged(xtag + tag_at<R>(b, lane, r), x, ep64);
+            if (active && r0 + r < a.nr && CHK_RECT(sy, c0 + lane + (r0 + r) * a.ldb, a.n, a.nr, a.ldb))
+                a.B[c0 + lane + (r0 + r) * a.ldb] = (T)x;
         }
     }
 }
@@ -449,21 +528,28 @@ __global__ void __launch_bounds__(kSolveThreads) solve_kernel(SolveArgs<T> a)
     sy.timeout_ns = a.timeout_ns;
     sy.chk_cut = a.chk_cut;
     const long long ep64 = (long long)sy.epoch << 32;
+    const size_t tags = (size_t)a.chains * a.nb * kW * R * 2;
     // bounds-checked builds: the workspace regions inside their allocations
-    const bool ws_in = CHK_REGION(sy, a.inv, (size_t)a.nb * kW * kW * sizeof(double), a.ws_data, a.ws_data_bytes) &&
-                       CHK_REGION(sy, a.yflag, (size_t)a.nb * sizeof(int), a.ws_iflags, a.ws_iflags_n * sizeof(int)) &&
-                       CHK_REGION(sy, a.ytag, (size_t)a.nb * kW * R * 2 * sizeof(long long), a.ws_progress,
-                                  a.ws_progress_n * sizeof(long long)) &&
-                       CHK_REGION(sy, a.xtag, (size_t)a.nb * kW * R * 2 * sizeof(long long), a.ws_progress,
-                                  a.ws_progress_n * sizeof(long long));
+    const bool ws_in = CHK_REGION(sy, a.inv, (size_t)a.nb * kPrepMats * kW * kW * sizeof(double), a.ws_data, a.ws_data_bytes) &&
+                       CHK_REGION(sy, a.uflag, (size_t)a.nb * sizeof(int), a.ws_iflags, a.ws_iflags_n * sizeof(int)) &&
+                       CHK_REGION(sy, a.ytag, tags * sizeof(long long), a.ws_progress, a.ws_progress_n * sizeof(long long)) &&
+                       CHK_REGION(sy, a.xtag, tags * sizeof(long long), a.ws_progress, a.ws_progress_n * sizeof(long long));
+    (void)tags;
 
+    const int nb = a.nb, steps = a.back_only ? nb : 2 * nb;
     for (;;) {
         if (threadIdx.x == 0) s_task = (!ws_in || aborted(sy)) ? -1 : atomicAdd(a.ctl + kCtlPairNext, 1);
         __syncthreads();
         const int t = s_task;
-        if (t < 0 || t >= 2 * a.nb) break;
-        if (t < a.nb) forward_task<T, R>(a, sy, ep64, t, S);
-        else backward_task<T, R>(a, sy, ep64, 2 * a.nb - 1 - t, S);
+        if (t < 0 || t >= nb + a.chains * steps) break;
+        if (t < nb) {
+            // a back substitution starts at the last block
+            prep_task<T>(a, sy, a.back_only ? nb - 1 - t : t, S.prep);
+        } else {
+            const int c = (t - nb) % a.chains, s = (t - nb) / a.chains + (a.back_only ? nb : 0);
+            if (s < nb) forward_task<T, R>(a, sy, ep64, c, s, S);
+            else backward_task<T, R>(a, sy, ep64, c, 2 * nb - 1 - s, S);
+        }
         __syncthreads();
     }
 
@@ -487,9 +573,17 @@ __global__ void __launch_bounds__(kSolveThreads) solve_kernel(SolveArgs<T> a)
     }
 }
 
+// Right-hand sides of one launch, at most: 64 (their tagged words take
+// 2 KB per row block and right-hand side), 16 above order 8192, where 16
+// chains of one already keep the FP64 pipes busy.
+int solve_group(long long n) { return n > 8192 ? kSolveChains : kSolveChains * kSolveRhs; }
+// Right-hand sides per chain: one while the chains suffice for all (a step
+// is shortest then), else as few as do.
+int solve_rhs(int nr) { return nr <= kSolveChains ? 1 : nr <= 2 * kSolveChains ? 2 : kSolveRhs; }
+
 template <typename T, int R>
 int launch_solve(const void *L, long long n, long long ld, void *B, long long ldb, int nr, const Scratch &sc,
-                 cudaStream_t stream, const T *Y = nullptr, long long ys = 0, long long cs = 0)
+                 cudaStream_t stream, const T *Y, long long ys, long long cs)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return CHM_ERR_CUDA;
@@ -511,14 +605,15 @@ int launch_solve(const void *L, long long n, long long ld, void *B, long long ld
     a.ldb = ldb;
     a.nb = nb;
     a.nr = nr;
+    a.chains = (nr + R - 1) / R;
     a.Y = Y;
     a.ys = ys;
     a.cs = cs;
     a.back_only = Y != nullptr;
     a.inv = reinterpret_cast<double *>(sc.data);
-    a.yflag = sc.iflags;
+    a.uflag = sc.iflags;
     a.ytag = sc.progress;
-    a.xtag = sc.progress + (size_t)nb * kW * R * 2;
+    a.xtag = sc.progress + (size_t)a.chains * nb * kW * R * 2;
     a.ctl = sc.ctl;
     a.status = sc.status;
     a.timeout_ns = timeout_ns();
@@ -529,20 +624,26 @@ int launch_solve(const void *L, long long n, long long ld, void *B, long long ld
     a.ws_progress = sc.progress;
     a.ws_progress_n = sc.progress_cap;
     a.chk_cut = check_cut();
-    const int grid = (int)std::min<long long>(2ll * nb, (long long)sm_count(dev) * occ[dev]);
+    const long long tasks = nb + (long long)a.chains * (a.back_only ? nb : 2 * nb);
+    const int grid = (int)std::min<long long>(tasks, (long long)sm_count(dev) * occ[dev]);
     solve_kernel<T, R><<<grid, kSolveThreads, 0, stream>>>(a);
     return cudaGetLastError() == cudaSuccess ? CHM_OK : CHM_ERR_CUDA;
 }
 
+// Both substitutions, or (Y given) the back substitution alone.
 template <typename T>
 int solve_all(const void *L, long long n, long long ld, void *B, long long ldb, long long nrhs, const Scratch &sc,
-              cudaStream_t stream)
+              cudaStream_t stream, const T *Y = nullptr, long long ys = 0, long long cs = 0)
 {
     T *b = static_cast<T *>(B);
-    for (long long r0 = 0; r0 < nrhs; r0 += kSolveRhs) {
-        const int nr = (int)std::min<long long>(kSolveRhs, nrhs - r0);
-        const int rc = nr == 1 ? launch_solve<T, 1>(L, n, ld, b + r0 * ldb, ldb, 1, sc, stream)
-                               : launch_solve<T, kSolveRhs>(L, n, ld, b + r0 * ldb, ldb, nr, sc, stream);
+    const int most = solve_group(n);
+    for (long long r0 = 0; r0 < nrhs; r0 += most) {
+        const int nr = (int)std::min<long long>(most, nrhs - r0);
+        const T *y = Y ? Y + r0 * cs : nullptr;
+        const int R = solve_rhs(nr);
+        const int rc = R == 1   ? launch_solve<T, 1>(L, n, ld, b + r0 * ldb, ldb, nr, sc, stream, y, ys, cs)
+                       : R == 2 ? launch_solve<T, 2>(L, n, ld, b + r0 * ldb, ldb, nr, sc, stream, y, ys, cs)
+                                : launch_solve<T, kSolveRhs>(L, n, ld, b + r0 * ldb, ldb, nr, sc, stream, y, ys, cs);
         if (rc != CHM_OK) return rc;
     }
     return CHM_OK;
@@ -550,32 +651,17 @@ int solve_all(const void *L, long long n, long long ld, void *B, long long ldb, 
 
 }  // namespace
 
-ScratchNeed solve_need(long long n)
+ScratchNeed solve_need(long long n, long long nrhs)
 {
     const size_t nb = (size_t)((n + kW - 1) / kW);
+    const size_t nr = (size_t)std::min<long long>(std::max(1ll, nrhs), solve_group(n));
+    const size_t R = (size_t)solve_rhs((int)nr), cols = (nr + R - 1) / R * R;
     ScratchNeed need;
     need.iflags = (nb + 63) & ~(size_t)63;
-    need.progress = 2 * nb * kW * kSolveRhs * 2;
-    need.data = nb * kW * kW * sizeof(double);
+    need.progress = 2 * nb * kW * cols * 2;
+    need.data = nb * kPrepMats * kW * kW * sizeof(double);
     return need;
 }
-
-namespace {
-template <typename T>
-int solve_back_t(const void *L, long long n, long long ld, void *B, long long ldb, long long nrhs, const T *Y,
-                 long long ys, long long cs, const Scratch &sc, cudaStream_t stream)
-{
-    T *b = static_cast<T *>(B);
-    for (long long r0 = 0; r0 < nrhs; r0 += kSolveRhs) {
-        const int nr = (int)std::min<long long>(kSolveRhs, nrhs - r0);
-        const T *y = Y + r0 * cs;
-        const int rc = nr == 1 ? launch_solve<T, 1>(L, n, ld, b + r0 * ldb, ldb, 1, sc, stream, y, ys, cs)
-                               : launch_solve<T, kSolveRhs>(L, n, ld, b + r0 * ldb, ldb, nr, sc, stream, y, ys, cs);
-        if (rc != CHM_OK) return rc;
-    }
-    return CHM_OK;
-}
-}  // namespace
 
 int solve_enqueue(const void *L, long long n, long long ld, void *B, long long ldb, long long nrhs, int dtype,
                   const Scratch &sc, cudaStream_t stream)
@@ -590,8 +676,8 @@ int solve_back_enqueue(const void *L, long long n, long long ld, void *B, long l
 {
     if (n <= 0 || nrhs <= 0) return CHM_OK;
     return dtype == CHM_F64
-               ? solve_back_t<double>(L, n, ld, B, ldb, nrhs, static_cast<const double *>(Y), ys, cs, sc, stream)
-               : solve_back_t<float>(L, n, ld, B, ldb, nrhs, static_cast<const float *>(Y), ys, cs, sc, stream);
+               ? solve_all<double>(L, n, ld, B, ldb, nrhs, sc, stream, static_cast<const double *>(Y), ys, cs)
+               : solve_all<float>(L, n, ld, B, ldb, nrhs, sc, stream, static_cast<const float *>(Y), ys, cs);
 }
 
 namespace {
@@ -609,7 +695,7 @@ int solve_dispatch(const void *L, long long n, long long ld, void *B, long long 
     int rc = check_reachable(L);
     if (rc == CHM_OK) rc = check_reachable(B);
     if (rc != CHM_OK) return rc;
-    return with_stream_scratch(stream, solve_need(n), [&](const Scratch &sc) {
+    return with_stream_scratch(stream, solve_need(n, nrhs), [&](const Scratch &sc) {
         return dtype == CHM_F64 ? solve_all<double>(L, n, ld, B, ldb, nrhs, sc, stream)
                                 : solve_all<float>(L, n, ld, B, ldb, nrhs, sc, stream);
     });
