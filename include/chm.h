@@ -35,8 +35,8 @@
  *   - Precision.  CHM_F64: L and V are double; all arithmetic in double.
  *     CHM_F32_MIXED: L and V are float; the Apply sweep runs in float while
  *     every Compute step runs in double on the promoted float values.  The
- *     vectors are taken in groups (those of one launch of the wave kernel,
- *     or one pass of the pass kernels): within a group each diagonal entry
+ *     vectors are taken in groups (those of one launch of the team or the wave
+ *     kernel, or one pass of the pass kernels): within a group each diagonal entry
  *     is carried in double from vector to vector and rounded to float once,
  *     after the group's last vector; the ratios that enter Apply (c and s,
  *     or the pass kernels' sweep coefficients) are rounded to float.  The
@@ -68,8 +68,9 @@
  *     and ends the launch's waits; nothing traps.  chm_config_get("checked")
  *     says which build is loaded (1 checked, 0 not).
  *   - Memory.  The library keeps a workspace per (device, stream): per
- *     vector of a launch (at most 64 per launch) rotation panels, ratio
- *     tiles and flags of about 19 KB per 32 rows, and the status word
+ *     vector of a launch (at most 64 per launch) coefficients, residuals,
+ *     matrices and flags of at most about 42 KB per 32 rows, and the status
+ *     word
  *     (chm_workspace_bytes gives the total).  It is allocated on the first
  *     call that needs a larger one; later calls of the same or smaller size
  *     allocate nothing.
@@ -180,7 +181,7 @@ int chm_modify_noalloc(void *L, int64_t n, int64_t ld, const void *V, int64_t ld
  * Batched up/downdate of many independent factors (a systems form of the
  * method; Sec. 4.1's rank-k blocking applied to each factor).  A plan fixes
  * the shapes; each execution takes the factors' and update blocks' device
- * addresses and runs every factor in ONE launch of the wave kernel, replayed
+ * addresses and runs every factor in ONE launch of the team kernel, replayed
  * from a CUDA graph captured by the plan (a copy of the problem table from
  * pinned host memory, a reset of the per-factor status words, the launch).
  *
@@ -194,13 +195,13 @@ int chm_modify_noalloc(void *L, int64_t n, int64_t ld, const void *V, int64_t ld
  *   plan    receives the plan
  * Factors with n_i == 0 or k_i == 0 are no-ops.  V_i is n_i x k_i
  * column-major with leading dimension n_i.  The plan owns all device scratch
- * (about n_i * 19 KB per vector of every factor) and pinned staging memory;
+ * (at most about 42 KB per vector and 32 rows of every factor) and pinned staging memory;
  * nothing is allocated by chm_batch_execute.  The current device at creation
  * is the plan's device.  Returns CHM_OK, CHM_ERR_ARG, CHM_ERR_NOMEM or
  * CHM_ERR_CUDA.
  *
- * chm_batch_autotune: times candidate launch configurations (SM groups,
- * blocks per SM, largest-work-first or caller order) on synthetic factors of
+ * chm_batch_autotune: times candidate launch configurations (teams of thread
+ * blocks that share a factor, blocks per SM, largest-work-first or caller order) on synthetic factors of
  * the plan's shapes (L = I, V = 1e-3, allocated for the duration of the call)
  * and keeps the fastest.  Synchronises `stream`.  The plan's status words
  * are reset.  Returns CHM_OK, CHM_ERR_NOMEM (no room for the synthetic
@@ -239,7 +240,7 @@ int chm_batch_plan_destroy(void *plan);
  * systems form of the method; each request is Algorithm 1 with its own V
  * and sign).  A worker thread keeps one FIFO per factor; whenever one of
  * its launch slots is free it packs the oldest ready request of every idle
- * factor into one launch of the wave kernel on that slot's stream.  Each
+ * factor into one launch of the team kernel on that slot's stream.  Each
  * slot launches with 1/max_inflight of the GPU's resident blocks, so a
  * launch formed from requests that arrived while another was running
  * overlaps it on the device.  Requests on one factor run one after another
@@ -416,7 +417,7 @@ int chm_microbench(int which, double *out, int nout);
  * Library-wide settings of the single-factor entry points (chm_update,
  * chm_downdate, chm_modify_ex), for tuning and tests; they take effect on
  * the next call and may be changed at any time from one thread.
- *   "path"     0 automatic (default), 1 the wave kernel, 2 the pass kernels
+ *   "path"     0 automatic (default), 1 the wave path, 2 the pass kernels
  *   "pass_kb"  update vectors per pass of the pass kernels, 1..16 (0: by
  *              type, 8 float, 4 double)
  *   "pass_d"   lookahead of the pass kernels' forward-substitution chain in
@@ -433,9 +434,13 @@ int chm_microbench(int which, double *out, int nout);
  *              and the Compute kernels run after the substitution
  * The two paths compute the same factor by the same method (Algorithm 1's
  * rotations, restated exactly) with different work splits:
- *   wave  one persistent launch per 64 vectors; each vector is a wave that
- *         sweeps the factor, its forward-substitution chain driven by the
- *         sweep's carries.  Fastest while the factor stays in L2.
+ *   wave  one persistent launch per 64 vectors, on one of two kernels.  The
+ *         team kernel (orders up to 8192; in double above 6144 only up to 16
+ *         vectors) substitutes every vector through the factor as it enters
+ *         a pass of up to 8 vectors, each vector a chain of its own, and
+ *         sweeps each tile once per pass.  The wave kernel (the rest): each
+ *         vector is a wave that sweeps the factor, its forward-substitution
+ *         chain driven by the sweep's carries.
  *   pass  per block of up to 16 vectors (Sec. 4.1's blocking): a forward
  *         substitution P = L^{-T} V run by one chain block with lookahead,
  *         every rotation's coefficients from prefix Grams of P (the Compute,
@@ -459,7 +464,7 @@ int chm_config_set(const char *key, int64_t value);
 int chm_config_get(const char *key, int64_t *value);
 
 /*
- * The path (1 wave kernel, 2 pass kernels) a single-factor modification of
+ * The path (1 wave path, 2 pass kernels) a single-factor modification of
  * order n by k vectors takes under the current settings and tuning cache.
  * Host only.  Returns CHM_OK or CHM_ERR_ARG.
  */
@@ -528,9 +533,10 @@ int chm_selftest_reciprocals(const double *x, int64_t count, double *out);
 /*
  * Diagnostics.  When the environment variable CHM_TRACE is set to 1 before
  * the first call, every launch of the plain entry points records 16 int64
- * stamps of the device's %globaltimer (ns) at fixed points per (wave, column
- * block): first the sweep tasks' records, then the wave blocks'
- * ([2][waves][blocks][16]).  chm_trace_dump synchronises the device and
+ * stamps of the device's %globaltimer (ns) at fixed points: on the wave
+ * kernel per (wave, column block), first the sweep tasks' records, then the
+ * wave blocks' ([2][waves][blocks][16]); on the team kernel per (vector,
+ * column block), [vectors][blocks][16].  chm_trace_dump synchronises the device and
  * writes the last launch's records (native endianness) to the file `path`.
  * Returns CHM_OK, CHM_ERR_STATE if tracing is off, CHM_ERR_ARG if the file
  * cannot be written, or CHM_ERR_CUDA.  Not for production use.
@@ -540,11 +546,15 @@ int chm_selftest_reciprocals(const double *x, int64_t count, double *out);
  *                          (default 4e9); a wait that runs out ends the
  *                          launch with CHM_ERR_TIMEOUT and the context stays
  *                          usable
- *   CHM_GROUPS             SM groups (concurrent waves) of a launch
+ *   CHM_GROUPS             wave kernel: SM groups (concurrent waves) of a
+ *                          launch; team kernel: teams of blocks of a batch or
+ *                          server launch (factors worked on at once)
  *   CHM_MAX_CTAS_PER_SM    cap on resident blocks per SM
  *   CHM_TEST_SKIP_PUBLISH  test hook: the next launch of the plain entry
  *                          points leaves the given block's rotation panel
- *                          unreleased, so the waits on it run out
+ *                          (wave kernel) or its first vector's substitution
+ *                          step (team kernel) unreleased, so the waits on it
+ *                          run out
  */
 int chm_trace_dump(const char *path);
 

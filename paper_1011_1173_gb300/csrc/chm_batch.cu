@@ -29,11 +29,10 @@ struct Plan {
     // problems with work, in launch order: order[p] = caller's factor index
     std::vector<int> order;
     bool lpt = true;  // launch order: largest work first (else caller's order)
-    int npairs = 0, nbmax = 0;
+    long long ntasks = 0;
     std::vector<Prob> tmpl;  // carved records without L and V
     Scratch sc;
     Prob *d_probs = nullptr;
-    int *d_pair_prob = nullptr;
     long long *d_info = nullptr;  // [count][2], caller's order
     Prob *h_probs[kStaging] = {nullptr, nullptr};
     cudaGraphExec_t exec[kStaging] = {nullptr, nullptr};
@@ -61,13 +60,11 @@ int relayout(Plan *p)
     p->order = act;
     std::vector<ProbShape> shapes;
     for (int i : act) shapes.push_back(ProbShape{p->n[i], p->k[i]});
-    const ScratchNeed need = scratch_need(shapes.data(), (int)shapes.size());
-    p->npairs = need.npairs;
-    p->nbmax = need.nbmax;
+    p->ntasks = 0;
     p->tmpl.assign(act.size(), Prob());
     for (Prob &pr : p->tmpl) memset(&pr, 0, sizeof(pr));
     if (act.empty()) return CHM_OK;
-    const std::vector<int> pair_prob = carve(shapes.data(), (int)shapes.size(), p->sc, p->tmpl.data());
+    team_carve(shapes.data(), (int)shapes.size(), p->sc, p->tmpl.data());
     for (size_t q = 0; q < act.size(); ++q) {
         const int i = act[q];
         Prob &pr = p->tmpl[q];
@@ -76,10 +73,8 @@ int relayout(Plan *p)
         pr.ldv = std::max(1ll, p->n[i]);
         pr.down_mask = p->sign[i] < 0 ? (p->k[i] >= 64 ? ~0ull : ((1ull << p->k[i]) - 1)) : 0ull;
         pr.info = p->d_info + 2 * (size_t)i;
+        p->ntasks += pr.ntasks;
     }
-    if (cudaMemcpy(p->d_pair_prob, pair_prob.data(), pair_prob.size() * sizeof(int), cudaMemcpyHostToDevice) !=
-        cudaSuccess)
-        return CHM_ERR_CUDA;
     return CHM_OK;
 }
 
@@ -107,7 +102,6 @@ void destroy(Plan *p)
     }
     if (p->last) cudaEventDestroy(p->last);
     cudaFree(p->d_probs);
-    cudaFree(p->d_pair_prob);
     cudaFree(p->d_info);
     scratch_free(&p->sc);
     if (cur >= 0) cudaSetDevice(cur);
@@ -131,8 +125,7 @@ int capture(Plan *p, int s)
         rc = CHM_ERR_CUDA;
     if (rc == CHM_OK) rc = info_init(p->d_info, p->count, cs);
     if (rc == CHM_OK)
-        rc = launch_wave(p->dtype, nullptr, p->d_probs, p->d_pair_prob, (int)np, p->npairs, p->nbmax, p->sc,
-                         p->cfg, nullptr, cs);
+        rc = launch_team(p->dtype, nullptr, p->d_probs, (int)np, p->ntasks, p->sc, p->cfg, nullptr, cs);
     const cudaError_t ec = cudaStreamEndCapture(cs, &g);
     if (rc == CHM_OK && ec != cudaSuccess) rc = CHM_ERR_CUDA;
     if (rc == CHM_OK && cudaGraphInstantiate(&p->exec[s], g, 0) != cudaSuccess) rc = CHM_ERR_CUDA;
@@ -266,11 +259,11 @@ int autotune(Plan *p, cudaStream_t stream)
     if (rc != CHM_OK) return rc;
     const int nsm = sm_count(p->device);
     int occ = 0;
-    rc = wave_occupancy(p->dtype, p->device, &occ);
+    rc = team_occupancy(p->dtype, p->device, &occ);
     if (rc != CHM_OK) return rc;
     std::vector<int> groups;
-    for (int d : {16, 12, 9, 7, 6, 5, 4, 3, 2}) {
-        const int g = std::max(1, std::min(std::min(p->npairs, kMaxGroups), nsm / d));
+    for (int d : {24, 16, 12, 8, 6, 4, 3, 2, 1}) {
+        const int g = std::max(1, std::min(std::min((int)p->order.size(), kMaxTeams), nsm * occ / d));
         if (std::find(groups.begin(), groups.end(), g) == groups.end()) groups.push_back(g);
     }
     const LaunchCfg keep = p->cfg;
@@ -341,12 +334,10 @@ int chm_batch_plan_create(int count, const int64_t *n, const int64_t *ld, const 
         p->sign[i] = sigma ? sigma[i] : 1;
         if (n[i] > 0 && k[i] > 0) shapes.push_back(ProbShape{n[i], (int)k[i]});
     }
-    const ScratchNeed need = scratch_need(shapes.data(), (int)shapes.size());
+    const ScratchNeed need = team_need(shapes.data(), (int)shapes.size());
     int rc = CHM_OK;
     if (cudaMalloc(&p->d_info, 2 * sizeof(long long) * std::max(1, count)) != cudaSuccess) rc = CHM_ERR_NOMEM;
     if (rc == CHM_OK && cudaMalloc(&p->d_probs, sizeof(Prob) * std::max<size_t>(1, shapes.size())) != cudaSuccess)
-        rc = CHM_ERR_NOMEM;
-    if (rc == CHM_OK && cudaMalloc(&p->d_pair_prob, sizeof(int) * std::max(1, need.npairs)) != cudaSuccess)
         rc = CHM_ERR_NOMEM;
     if (rc == CHM_OK) rc = scratch_alloc(&p->sc, need.iflags, need.progress, std::max<size_t>(need.data, 256));
     for (int s = 0; s < kStaging && rc == CHM_OK; ++s) {
@@ -359,7 +350,7 @@ int chm_batch_plan_create(int count, const int64_t *n, const int64_t *ld, const 
     if (rc == CHM_OK) rc = relayout(p);
     // the kernel's one-time set-up happens here, outside any stream capture
     int occ = 0;
-    if (rc == CHM_OK) rc = wave_occupancy(dtype, p->device, &occ);
+    if (rc == CHM_OK) rc = team_occupancy(dtype, p->device, &occ);
     if (rc == CHM_OK) rc = info_init(p->d_info, count, nullptr);
     if (rc == CHM_OK && cudaDeviceSynchronize() != cudaSuccess) rc = CHM_ERR_CUDA;
     if (rc != CHM_OK) {

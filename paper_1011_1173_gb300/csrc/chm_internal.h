@@ -70,6 +70,20 @@ int launch_wave(int dtype, const Prob *single, const Prob *d_probs, const int *d
                 int nprobs, int npairs, int nbmax, const Scratch &sc, const LaunchCfg &cfg,
                 long long *trace, cudaStream_t stream);
 
+// The team kernel (chm_team.cu): scratch needed by a list of problems laid
+// out one after another; the scratch pointers, nb, k and task counts of
+// problems[0..count) for that layout; blocks per SM; and one launch of
+// either one problem (`single`) or `nprobs` whose records are in device
+// memory, with `tasks` tasks in all.  cfg.groups is the number of teams.
+// `trace` is null or a device array of k * nb * kTracePoints words.
+ScratchNeed team_need(const ProbShape *shapes, int count);
+void team_carve(const ProbShape *shapes, int count, const Scratch &sc, Prob *problems);
+int team_occupancy(int dtype, int dev, int *ctas_per_sm);
+int launch_team(int dtype, const Prob *single, const Prob *d_probs, int nprobs, long long tasks, const Scratch &sc,
+                const LaunchCfg &cfg, long long *trace, cudaStream_t stream);
+// True if a single-factor modification on path 1 takes the team kernel (else the wave kernel).
+bool use_team(long long n, long long k, int dtype);
+
 // Set count {status, row} words to {0, -1} on `stream`.
 int info_init(long long *d_info, int count, cudaStream_t stream);
 
@@ -81,7 +95,7 @@ int scratch_alloc(Scratch *sc, size_t iflags, size_t progress, size_t data);
 // device's memory, an unknown address).
 int check_reachable(const void *p);
 // Device bytes the single-factor entry points hold for order n, k vectors.
-size_t single_workspace_bytes(long long n, long long k);
+size_t single_workspace_bytes(long long n, long long k, int dtype);
 // Runs fn on the current device's workspace for `stream` (the one the plain
 // entry points use, whose status word chm_status_sync reads), grown first to
 // at least `need`, under the workspaces' lock.

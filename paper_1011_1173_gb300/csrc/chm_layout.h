@@ -94,6 +94,7 @@ struct Prob {
     int k;                         // waves of this problem in the launch (<= kMaxWaves)
     int nb;                        // column blocks of kW columns
     int pair0;                     // index of its first pair (k waves, then the final pass)
+    int ntasks;                    // team kernel: its tasks
     unsigned long long down_mask;  // bit q set: wave q is a downdate
     char *data;                    // prob_data_bytes(nb, k), 256-byte aligned
     int *iflags;                   // prob_iflags(nb, k) ints
@@ -110,6 +111,8 @@ constexpr int kCtlStarted = 3;    // blocks started
 constexpr int kCtlExited = 4;     // blocks finished
 constexpr int kCtlEpoch = 8;      // launch counter; flags of this launch equal it
 constexpr int kCtlAbort = 32;     // non-zero once a wait has timed out
+constexpr int kCtlTeam = 64;      // team kernel: [kMaxTeams] the team's problem + 1 (the wave kernel's groups' place)
+constexpr int kMaxTeams = 256;
 constexpr int kCtlGroupTicket = 64;                                  // u64 [kMaxGroups]: (current pair + 1) << 32
 constexpr int kCtlGroupSweepers = kCtlGroupTicket + 2 * kMaxGroups;  // [kMaxGroups] sweep SMs per group
 constexpr int kCtlSmSlot = kCtlGroupSweepers + kMaxGroups;           // [kMaxSm] arrivals per SM

@@ -13,6 +13,7 @@
 
 #include "chm.h"
 #include "chm_internal.h"
+#include "chm_team_layout.h"
 #include "chm_wave.cuh"
 
 namespace chm {
@@ -241,11 +242,31 @@ int check_reachable(const void *p)
     }
 }
 
-size_t single_workspace_bytes(long long n, long long k)
+// Path 1's two kernels.  The team kernel spends three FMAs per element and
+// vector where the wave kernel spends two, but does not sweep the factor
+// vector after vector: it is ahead until a large factor and many vectors in
+// double keep the wave kernel at the FP64 rate.  Measured, ms per modification
+// (team / wave), double: n = 512 k = 1 0.10 / 0.15, k = 16 0.27 / 0.38; n = 5000
+// k = 1 0.42 / 1.10, k = 16 1.70 / 1.98, k = 64 6.18 / 6.61; n = 8192 k = 16
+// 3.82 / 3.97, k = 64 14.5 / 13.8; float: n = 2000 k = 1 0.14 / 0.41, k = 16
+// 0.28 / 0.65; n = 8192 k = 64 5.5 / 8.6.
+bool use_team(long long n, long long k, int dtype)
+{
+    if (n > 8192) return false;
+    return dtype != CHM_F64 || n <= 6144 || k <= 16;
+}
+
+// The scratch of path 1 for one launch.
+static ScratchNeed single_need(const ProbShape &sh, int dtype)
+{
+    return use_team(sh.n, sh.k, dtype) ? team_need(&sh, 1) : scratch_need(&sh, 1);
+}
+
+size_t single_workspace_bytes(long long n, long long k, int dtype)
 {
     if (n <= 0 || k <= 0) return 0;
     const ProbShape sh{n, (int)std::min<long long>(k, kMaxWaves)};
-    const ScratchNeed need = scratch_need(&sh, 1);
+    const ScratchNeed need = single_need(sh, dtype);
     return kCtlInts * sizeof(int) + 2 * sizeof(long long) + std::max(need.iflags, (size_t)4096) * sizeof(int) +
            std::max(need.progress, (size_t)1024) * sizeof(long long) + need.data;
 }
@@ -392,7 +413,7 @@ static unsigned long long down_mask(const int8_t *sigma, int sign, long long q0,
 // scratch `sc` (already large enough for kw_max waves).
 static int enqueue_single(void *L, long long n, long long ld, const void *V, long long ldv, long long k,
                           const int8_t *sigma, int sign, int dtype, cudaStream_t stream, long long *d_info,
-                          const Scratch &sc, int kw_max, bool allow_trace)
+                          const Scratch &sc, int kw_max, bool allow_trace, bool team)
 {
     const size_t elt = dtype == CHM_F64 ? 8 : 4;
     const int nb = (int)((n + kW - 1) / kW);
@@ -403,7 +424,8 @@ static int enqueue_single(void *L, long long n, long long ld, const void *V, lon
         Prob pr;
         memset(&pr, 0, sizeof(pr));
         const ProbShape sh{n, kw};
-        carve(&sh, 1, sc, &pr);
+        if (team) team_carve(&sh, 1, sc, &pr);
+        else carve(&sh, 1, sc, &pr);
         pr.L = L;
         pr.V = static_cast<const char *>(V) + (size_t)q0 * ldv * elt;
         pr.n = n;
@@ -413,7 +435,7 @@ static int enqueue_single(void *L, long long n, long long ld, const void *V, lon
         pr.info = d_info;
         long long *trace = nullptr;
         if (allow_trace && trace_on()) {
-            const size_t need = (size_t)2 * (kw + 1) * nb * kTracePoints;
+            const size_t need = (team ? (size_t)kw : (size_t)2 * (kw + 1)) * nb * kTracePoints;
             if (g_trace_cap < need) {
                 cudaFree(g_trace);
                 g_trace = nullptr;
@@ -428,7 +450,8 @@ static int enqueue_single(void *L, long long n, long long ld, const void *V, lon
         }
         LaunchCfg cfg;
         cfg.skip_publish = take_test_skip();
-        rc = launch_wave(dtype, &pr, nullptr, nullptr, 1, kw + 1, nb, sc, cfg, trace, stream);
+        rc = team ? launch_team(dtype, &pr, nullptr, 1, pr.ntasks, sc, cfg, trace, stream)
+                  : launch_wave(dtype, &pr, nullptr, nullptr, 1, kw + 1, nb, sc, cfg, trace, stream);
         if (rc != CHM_OK) return rc;
     }
     return CHM_OK;
@@ -471,9 +494,9 @@ static int modify_dispatch(void *L, long long n, long long ld, const void *V, lo
     }
     const int kw_max = (int)std::min<long long>(k, kMaxWaves);
     const ProbShape sh{n, kw_max};
-    const ScratchNeed need = scratch_need(&sh, 1);
-    return with_stream_scratch(stream, need, [&](const Scratch &sc) {
-        return enqueue_single(L, n, ld, V, ldv, k, sigma, sign, dtype, stream, d_info, sc, kw_max, true);
+    return with_stream_scratch(stream, single_need(sh, dtype), [&](const Scratch &sc) {
+        return enqueue_single(L, n, ld, V, ldv, k, sigma, sign, dtype, stream, d_info, sc, kw_max, true,
+                              use_team(n, kw_max, dtype));
     });
 }
 
@@ -625,12 +648,15 @@ static int noalloc_setup(int dev, NoAllocState **out)
     return CHM_OK;
 }
 
-// Waves per launch that fit the array for order n (0: none).
-static int noalloc_waves(long long n)
+// Vectors per launch that fit the array, of the k asked for (0: none).  The
+// team kernel's launches hold whole passes, so that the passes, and with
+// them the result, are those of one launch.
+static int noalloc_vectors(long long n, int k, bool team)
 {
-    for (int kw = kMaxWaves; kw >= 1; --kw) {
+    for (int kw = k; kw >= 1; --kw) {
         const ProbShape sh{n, kw};
-        const ScratchNeed need = scratch_need(&sh, 1);
+        const ScratchNeed need = team ? team_need(&sh, 1) : scratch_need(&sh, 1);
+        if (team && kw < k && kw % team::kTeamKb != 0) continue;
         if (need.iflags <= kNoAllocIflags && need.progress <= kNoAllocProgress &&
             need.data <= kNoAllocBytes - kNoAllocDataOff)
             return kw;
@@ -650,7 +676,9 @@ static int modify_noalloc(void *L, long long n, long long ld, const void *V, lon
     if (n > kNoAllocMaxN) return CHM_ERR_BUDGET;
     if (n == 0 || k == 0) return info_init(d_info, 1, stream);
     if ((rc = check_reachable(L)) != CHM_OK || (rc = check_reachable(V)) != CHM_OK) return rc;
-    const int kw_max = std::min<int>(noalloc_waves(n), (int)std::min<long long>(k, kMaxWaves));
+    const int kw = (int)std::min<long long>(k, kMaxWaves);
+    const bool team = use_team(n, kw, dtype);
+    const int kw_max = noalloc_vectors(n, kw, team);
     if (kw_max < 1) return CHM_ERR_BUDGET;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return CHM_ERR_CUDA;
@@ -659,7 +687,7 @@ static int modify_noalloc(void *L, long long n, long long ld, const void *V, lon
     NoAllocState *st = nullptr;
     rc = noalloc_setup(dev, &st);
     if (rc != CHM_OK) return rc;
-    return enqueue_single(L, n, ld, V, ldv, k, sigma, sign, dtype, stream, d_info, st->sc, kw_max, false);
+    return enqueue_single(L, n, ld, V, ldv, k, sigma, sign, dtype, stream, d_info, st->sc, kw_max, false, team);
 }
 
 }  // namespace chm
@@ -705,7 +733,7 @@ int chm_workspace_bytes(int64_t n, int64_t k, int dtype, size_t *bytes)
 {
     if (!bytes || n < 0 || k < 0 || n > (1ll << 26)) return CHM_ERR_ARG;
     if (dtype != CHM_F64 && dtype != CHM_F32_MIXED) return CHM_ERR_ARG;
-    const size_t wave = chm::single_workspace_bytes(n, k);
+    const size_t wave = chm::single_workspace_bytes(n, k, dtype);
     const chm::PassChoice ch = chm::choose_path(n, k, dtype, false);
     const size_t pass = (n > 0 && k > 0) ? chm::kCtlInts * sizeof(int) + 2 * sizeof(long long) +
                                                chm::pass_workspace_bytes(n, dtype, ch.seg)

@@ -65,10 +65,8 @@ struct Slot {
     Scratch sc;
     size_t scratch_bytes = 0;
     Prob *h_probs = nullptr;
-    int *h_pair = nullptr;
     long long *h_info = nullptr;
     Prob *d_probs = nullptr;
-    int *d_pair = nullptr;
     long long *d_info = nullptr;
     cudaEvent_t done = nullptr;
     std::vector<Request *> reqs;
@@ -104,7 +102,7 @@ size_t elt_size(int dtype) { return dtype == CHM_F64 ? 8 : 4; }
 ScratchNeed need_of(long long n, int k)
 {
     const ProbShape sh{n, k};
-    return scratch_need(&sh, 1);
+    return team_need(&sh, 1);
 }
 
 // Complete the launch of a slot (its event has fired); called with the lock held.
@@ -180,8 +178,8 @@ int launch_slot(Server *s, Slot &sl)
     const int np = (int)sl.reqs.size();
     std::vector<Prob> probs(np);
     for (Prob &p : probs) memset(&p, 0, sizeof(p));
-    const std::vector<int> pair_prob = carve(shapes.data(), np, sl.sc, probs.data());
-    int nbmax = 0;
+    team_carve(shapes.data(), np, sl.sc, probs.data());
+    long long ntasks = 0;
     for (int i = 0; i < np; ++i) {
         Request *r = sl.reqs[i];
         const Factor &f = s->factors[r->fid];
@@ -193,23 +191,18 @@ int launch_slot(Server *s, Slot &sl)
         p.ldv = f.n;
         p.down_mask = r->sigma < 0 ? (r->k >= 64 ? ~0ull : ((1ull << r->k) - 1)) : 0ull;
         p.info = sl.d_info + 2 * (size_t)i;
-        nbmax = std::max(nbmax, p.nb);
+        ntasks += p.ntasks;
         sl.h_probs[i] = p;
     }
-    memcpy(sl.h_pair, pair_prob.data(), pair_prob.size() * sizeof(int));
     for (Request *r : sl.reqs)
         if (cudaStreamWaitEvent(sl.stream, r->v_ready, 0) != cudaSuccess) return CHM_ERR_CUDA;
     if (cudaMemcpyAsync(sl.d_probs, sl.h_probs, np * sizeof(Prob), cudaMemcpyHostToDevice, sl.stream) != cudaSuccess)
-        return CHM_ERR_CUDA;
-    if (cudaMemcpyAsync(sl.d_pair, sl.h_pair, pair_prob.size() * sizeof(int), cudaMemcpyHostToDevice, sl.stream) !=
-        cudaSuccess)
         return CHM_ERR_CUDA;
     int rc = info_init(sl.d_info, np, sl.stream);
     if (rc != CHM_OK) return rc;
     LaunchCfg cfg;
     cfg.grid = s->grid;
-    rc = launch_wave(s->dtype, nullptr, sl.d_probs, sl.d_pair, np, (int)pair_prob.size(), nbmax, sl.sc, cfg,
-                     nullptr, sl.stream);
+    rc = launch_team(s->dtype, nullptr, sl.d_probs, np, ntasks, sl.sc, cfg, nullptr, sl.stream);
     if (rc != CHM_OK) return rc;
     if (cudaMemcpyAsync(sl.h_info, sl.d_info, 2 * np * sizeof(long long), cudaMemcpyDeviceToHost, sl.stream) !=
         cudaSuccess)
@@ -285,10 +278,8 @@ void destroy(Server *s)
         }
         scratch_free(&sl.sc);
         cudaFreeHost(sl.h_probs);
-        cudaFreeHost(sl.h_pair);
         cudaFreeHost(sl.h_info);
         cudaFree(sl.d_probs);
-        cudaFree(sl.d_pair);
         cudaFree(sl.d_info);
         if (sl.done) cudaEventDestroy(sl.done);
         if (sl.stream) cudaStreamDestroy(sl.stream);
@@ -317,7 +308,7 @@ int create(size_t budget, int dtype, int max_inflight, Server **out)
     s->budget = budget;
     s->nslots = std::max(1, std::min(kMaxSlots, max_inflight <= 0 ? 2 : max_inflight));
     int occ = 0;
-    int rc = wave_occupancy(dtype, s->device, &occ);
+    int rc = team_occupancy(dtype, s->device, &occ);
     if (rc != CHM_OK) {
         delete s;
         return rc;
@@ -333,8 +324,9 @@ int create(size_t budget, int dtype, int max_inflight, Server **out)
     for (int i = 0; i < s->nslots && rc == CHM_OK; ++i) {
         Slot &sl = s->slots[i];
         // flag and tagged-word regions in proportion to the data region: per
-        // 32 columns and wave, ~18 KB of data against 3 int flags and 129 tags
-        const size_t iflags = per / 4096, progress = per / 128;
+        // 32 columns and pass of 8 vectors, 20 KB of data or more against 2
+        // int flags and 584 tagged words
+        const size_t iflags = per / 4096, progress = per / 40;
         const size_t data = per - iflags * sizeof(int) - progress * sizeof(long long);
         rc = scratch_alloc(&sl.sc, iflags, progress, data);
         sl.scratch_bytes = per;
@@ -342,10 +334,8 @@ int create(size_t budget, int dtype, int max_inflight, Server **out)
         if (cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming) != cudaSuccess ||
             cudaMallocHost(&sl.h_probs, kMaxProbsPerLaunch * sizeof(Prob)) != cudaSuccess ||
-            cudaMallocHost(&sl.h_pair, kMaxProbsPerLaunch * (kMaxWaves + 1) * sizeof(int)) != cudaSuccess ||
             cudaMallocHost(&sl.h_info, 2 * kMaxProbsPerLaunch * sizeof(long long)) != cudaSuccess ||
             cudaMalloc(&sl.d_probs, kMaxProbsPerLaunch * sizeof(Prob)) != cudaSuccess ||
-            cudaMalloc(&sl.d_pair, kMaxProbsPerLaunch * (kMaxWaves + 1) * sizeof(int)) != cudaSuccess ||
             cudaMalloc(&sl.d_info, 2 * kMaxProbsPerLaunch * sizeof(long long)) != cudaSuccess)
             rc = CHM_ERR_NOMEM;
     }

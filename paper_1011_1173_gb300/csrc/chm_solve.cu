@@ -126,17 +126,12 @@ __device__ __forceinline__ void wait_block(const SyncArgs &sy, const long long *
 #pragma unroll
         for (int r = 0; r < R; ++r) ok = get_tagged(w + 2 * r, ep64, &v[r]) && ok;
         if (__all_sync(kFull, ok)) return;
+        // (looked at by all lanes alike: a branch of lane 0 alone would leave
+        // the warp split, and every later shuffle would wait for the halves)
         if ((it & 15u) == 15u) {
-            int stop = 0;
-            if (lane == 0) {
-                if (aborted(sy)) {
-                    stop = 1;
-                } else if (global_ns() - t0 > sy.timeout_ns || it > (1u << 28)) {
-                    record_error(sy, kStatusTimeout, who);
-                    stop = 1;
-                }
-            }
-            if (__shfl_sync(kFull, stop, 0)) {
+            const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 28);
+            if (__any_sync(kFull, late || aborted(sy))) {
+                if (lane == 0 && late) record_error(sy, kStatusTimeout, who);
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[r] = 0.0;
                 return;

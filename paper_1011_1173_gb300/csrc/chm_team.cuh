@@ -1,0 +1,1227 @@
+// Team kernel of the rank-k up/downdate (Walder 2010, Algorithm 1): one
+// persistent launch that carries one or many independent factors, for
+// factors that stay in L2.  It evaluates the same exact identities as the
+// pass kernels (chm_pass.cuh), in passes of up to kTeamKb = 8 vectors:
+//   P = F^{-T} V;  the prefix Grams H_r = Sigma + sum_{i<r} p_i p_i^T and
+//   their factors L |D| Sigma L^T, which fix every rotation's coefficients
+//   (Compute);  and the scaled Apply sweep, two FMAs per element and vector.
+//
+// Work split.  Every piece of a pass is a task of one thread block (four
+// warps), and the tasks of a factor are numbered in an order in which each
+// waits only on tasks before it, so that a launch of any number of resident
+// blocks progresses.  Blocks take a factor's tasks from its ticket word; a
+// factor is worked on by a team of blocks, and the launch holds G teams.
+//   PREP(b)   U_b = D_b^{-1} and G1_b = U_b^T F_{b-1,b}^T of diagonal block b
+//   PREP2(b)  G2_b = U_b^T F_{b-2,b}^T
+//   SUB(c, b) step b of the forward substitution of vector c:
+//               p_b = U_b^T (v_b - sum_{r<=b-3} F_{r,b}^T p_r) - G2_b p_{b-2} - G1_b p_{b-1}.
+//             The tiles above are summed as their p arrive, and what is left
+//             of v at the start of every sweep segment is kept.  After
+//             p_{b-1} there is one 32 x 32 product, eight FMAs a warp.
+//   COEF(b)   the prefix Grams of row block b's rows, their LDL^T and the
+//             rows' sweep coefficients
+//   SWEEP(b, s) segments of column block b (`seg` row blocks each): the
+//             carries restart from the kept residual, and every tile is
+//             read, rotated and written once per pass
+// A column is swept only after its substitution step, which is the last
+// reader of its tiles as they entered the pass, so no tile needs a flag of
+// its own; the next pass of a factor enters column b once b's sweep is done.
+//
+// What bounds it.  A vector's substitution is the serial chain: nb steps of
+// about 1.7 us (a flag through L2, 8 FMAs at one FP64 instruction per 64
+// cycles and warp, a barrier, a four-way sum).  Vectors do not wait for each
+// other, and nothing else is on the chain: the sweep trails it by one
+// segment, whatever the number of vectors.  With many vectors or factors the
+// FP64 rate binds (three FMAs per element and vector: one in the
+// substitution, two in the sweep).
+//
+// Precision: CHM_F64 is double throughout.  CHM_F32_MIXED substitutes in
+// double (P, U, G) with the far sums in pairs of floats (48 bits), forms the
+// coefficients in double, and sweeps in float; the diagonal is carried in
+// double through all passes of the launch and rounded to float at the end of
+// each.
+#pragma once
+
+#include "chm_device.cuh"
+#include "chm_pass.cuh"
+#include "chm_team_layout.h"
+
+namespace chm {
+namespace team {
+
+constexpr int kThreads = 128;
+constexpr int kWarps = 4;
+constexpr int kPer = kW / kWarps;  // rows of a split 32 x 32 product per warp
+
+template <typename T>
+struct Launch {
+    const Prob *probs;  // device array [nprobs]; null: the one problem is prob0
+    Prob prob0;
+    int nprobs, nteams;
+    int *ctl;           // kCtlInts control words
+    long long *status;  // sticky {status, row} of the scratch owner
+    long long *trace;   // optional timestamps of the one problem, [k][nb][kTracePoints]
+    long long timeout_ns;
+    int skip_publish;   // test hook: vector 0's step at this block is never published (-1: none)
+    // the workspace allocations the problems' regions are carved from (bounds-checked builds)
+    const char *ws_data;
+    size_t ws_data_bytes;
+    const int *ws_iflags;
+    size_t ws_iflags_n;
+    const long long *ws_progress;
+    size_t ws_progress_n;
+    long long chk_cut;  // bounds-checked build: columns taken off each factor's declared extent
+};
+
+// One pass of one problem, in shared memory: written by thread 0 when the
+// block takes up the problem or its next pass.
+template <typename T>
+struct View {
+    T *L;
+    const T *V;  // the pass's first vector
+    long long n, ld, ldv;
+    int nb, pass, npass, kb, KB, seg, nbound, look, units;
+    unsigned down_mask;  // bit q: vector q of the pass is a downdate
+    bool vec;            // 16-byte column segments
+    double *ug;          // [nb][3][kW][kW]: U_b (row i at i * kW), G1_b and G2_b (element (i, j) at j * kW + i)
+    T *coef;             // [nb * kW][2 KB]
+    T *escale;           // [nb * kW]
+    double *dfac;        // [nb * kW]
+    T *snap;             // [nbound][nb * kW][KB]
+    double *rst;         // [nbound][KB (KB + 1) / 2]: packed unit lower factor, 1 / |D_q| on the diagonal
+    double *dcar;        // [nb * kW]: the diagonal, carried in double from pass to pass
+    long long *ptag;     // [kb][nb][kW][2]
+    long long *htag;     // [nb][KB (KB + 1) / 2][2]
+    int *uflag, *gflag, *g2flag, *cflag;  // [nb] each: U, G1, G2, coefficients published (== epoch)
+    long long *sdone;    // [nb]: sweep tasks of a column finished, all passes (epoch-tagged count)
+    SyncArgs sync;
+};
+
+// A block's cursor in the list of a pass's tasks.
+struct Stage {
+    int t;        // stage
+    int first;    // its first task
+    int passes;   // tasks of the passes before
+};
+
+struct PrepSmem {
+    double D[kW][kW + 1];
+    double U[kW][kW + 1];
+    double F[kW][kW + 1];
+    double M[kW / 2][kW / 2 + 1];
+    double rd[kW];
+};
+template <typename T>
+struct SubSmem {
+    T tile[kWarps][2][kW * pass::Stride<T>::value];
+    double y[kWarps][kW];   // the p a warp works with (double), or its float pairs
+    double part[2][kWarps][kW];
+    double z[kW];           // what is left of v
+};
+struct CoefSmem {
+    static constexpr int ne = kTeamKb * (kTeamKb + 1) / 2;
+    static constexpr int hs = ne | 1;
+    double H[kW][hs];       // row r: its prefix Gram, then its factor
+    double g[8][ne];        // the Grams of the threads' shares of the rows
+    double p[kW][kTeamKb + 1];
+    double z[kW][kTeamKb + 1];
+};
+// A sweep task's segments: NV warps pass a tile on, so NV + 1 tiles are in
+// flight per segment.
+template <typename T, int KB, int NV>
+struct SweepSmem {
+    static constexpr int NS = NV + 1, UNITS = kWarps / NV;
+    struct Unit {
+        T tile[NS][kW * pass::Stride<T>::value];
+        T cf[NS][kW * 2 * KB];
+        T e[NS][kW];
+    } unit[UNITS];
+};
+template <typename T>
+union TaskSmem {
+    PrepSmem prep;
+    SubSmem<T> sub;
+    CoefSmem coef;
+    SweepSmem<T, 1, 1> sweep1;
+    SweepSmem<T, 2, 2> sweep2;
+    SweepSmem<T, 4, 4> sweep4;
+    SweepSmem<T, 8, 4> sweep8;
+    __device__ TaskSmem() {}
+};
+
+constexpr unsigned kFull = 0xffffffffu;
+
+// Stamp `pt` of column block b of vector c (diagnostics): 0 SUB taken, 1 its
+// tiles summed, 2 what is left multiplied by U, 3 the previous step seen, 4
+// its result put; for the pass's first vector 5 COEF's inputs in, 6 its
+// results out, 7 the column's last segment swept.
+#define TEAM_TRACE(c, b, pt)                                                                                     \
+    do {                                                                                                         \
+        if (P.trace && threadIdx.x == 0)                                                                         \
+            P.trace[((size_t)(v.pass * kTeamKb + (c)) * v.nb + (b)) * kTracePoints + (pt)] = global_ns();        \
+    } while (0)
+
+// Stage the 32 x 32 tile at row r0, column c0 into dst[column][Stride], read
+// through L2 (an earlier pass of the launch may have written it on another
+// SM): 16-byte asynchronous copies if `vec`, else loads of one element,
+// eight in flight per lane (a 4-byte cp.async would go through L1).  `diag`:
+// the diagonal tile, rows <= column only; the rest is zero.
+template <typename T>
+__device__ __forceinline__ void stage_tile(const SyncArgs &sy, T *dst, const T *L, long long ld, long long r0,
+                                           long long c0, long long n, bool vec, bool diag, int lane)
+{
+    constexpr int SD = pass::Stride<T>::value;
+    if (vec) {
+        pass::stage_tile(sy, dst, L, ld, r0, c0, n, kW, true, lane);
+        return;
+    }
+#pragma unroll 1
+    for (int c = 0; c < kW; c += 8) {
+        T x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long o = (r0 + lane) + (c0 + c + i) * ld;
+            x[i] = (c0 + c + i < n && (!diag || lane <= c + i) && CHK_TRI(sy, o, n, ld)) ? __ldcg(L + o) : T(0);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) dst[(c + i) * SD + lane] = x[i];
+    }
+}
+
+// ---------------------------------------------------------------- PREP
+
+// The next pass may enter column block b once the last one has swept it
+// (every pass but the last has kTeamKb vectors, one column per task).
+template <typename T>
+__device__ __forceinline__ bool wait_column(const View<T> &v, int b)
+{
+    if (v.pass == 0) return true;
+    const long long want = ((long long)v.sync.epoch << 32) + (long long)v.pass * segs_of(b, seg_of(v.nb, kTeamKb));
+    const bool ok = __all_sync(kFull, wait_ge(v.sync, v.sdone + b, want, b));
+    __syncwarp();
+    return ok;
+}
+
+// out[j kW + i] = G[i][j] = sum_{m<=i} U[m][i] F[j][m]; rows i = warp,
+// warp + 4, ... (so that the four warps' triangles weigh the same: 144
+// FMAs each, with U's zeros in the rows' last groups of four), lane = j.
+__device__ __forceinline__ void form_g(const PrepSmem &S, double *out)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double acc[kPer];
+#pragma unroll
+    for (int ii = 0; ii < kPer; ++ii) acc[ii] = 0.0;
+#pragma unroll
+    for (int m = 0; m < kW; ++m) {
+        const double f = S.F[lane][m];
+#pragma unroll
+        for (int ii = m / kWarps; ii < kPer; ++ii) acc[ii] = fma(S.U[m][ii * kWarps + warp], f, acc[ii]);
+    }
+#pragma unroll
+    for (int ii = 0; ii < kPer; ++ii) __stcg(out + (size_t)lane * kW + ii * kWarps + warp, acc[ii]);
+}
+// The tile `up` blocks above diagonal block b: F[j][m] = L[(b - up) kW + j, b kW + m].
+template <typename T>
+__device__ __forceinline__ void load_above(const View<T> &v, int b, int up, PrepSmem &S)
+{
+    const long long c0 = (long long)b * kW;
+    const int nc = (int)min((long long)kW, v.n - c0);
+#pragma unroll
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = threadIdx.x + x * kThreads, i = e & (kW - 1), j = e / kW;
+        const long long o = c0 - up * kW + i + (c0 + j) * v.ld;
+        S.F[i][j] = (j < nc && CHK_TRI(v.sync, o, v.n, v.ld)) ? (double)__ldcg(v.L + o) : 0.0;
+    }
+}
+// Every store of the block's threads so far, then the flag.
+__device__ __forceinline__ void publish(int *flag, int epoch)
+{
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) st_release_gpu(flag, epoch);
+}
+
+// U_b and G1_b.  The inverse is built up from 8 x 8 diagonal blocks: with
+// D = [[D1, B], [0, D2]], U = [[U1, -U1 B U2], [0, U2]].  The four 8 x 8
+// inverses take one warp (a column per lane, 36 dependent FP64 instructions),
+// the products of the two levels above all four warps: 116 instructions in
+// a row instead of the 560 of a column-per-lane substitution (3.6 against
+// 17 us at one FP64 instruction per 64 cycles and warp).
+template <typename T>
+__device__ void prep_task(const Launch<T> &P, const View<T> &v, int b, PrepSmem &S)
+{
+
+    const SyncArgs &sy = v.sync;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const long long n = v.n, ld = v.ld;
+    const long long c0 = (long long)b * kW;
+    const int nc = (int)min((long long)kW, n - c0);
+    (void)wait_column(v, b);
+#pragma unroll
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = tid + x * kThreads, i = e & (kW - 1), j = e / kW;
+        double d = 0.0;
+        if (j < nc) {
+            if (i == j && v.pass > 0) d = __ldcg(v.dcar + c0 + j);
+            else if (i <= j && CHK_TRI(sy, c0 + i + (c0 + j) * ld, n, ld)) d = (double)__ldcg(v.L + c0 + i + (c0 + j) * ld);
+        } else if (i == j) {
+            d = 1.0;
+        }
+        S.D[i][j] = d;
+        S.U[i][j] = 0.0;
+    }
+    if (b >= 1) load_above(v, b, 1, S);
+    __syncthreads();
+    if (warp == 0) {
+        double d = S.D[lane][lane];
+        const bool bad = lane < nc && !(d > 0.0 && d <= DBL_MAX);
+        const unsigned badm = __ballot_sync(kFull, bad);
+        if (badm && lane == 0) record_error(sy, kStatusNotPD, c0 + (__ffs(badm) - 1));
+        if (bad) d = 1.0;
+        if (v.pass == 0 && lane < nc) __stcg(v.dcar + c0 + lane, d);
+        S.rd[lane] = rcp_refined(d);
+        __syncwarp();
+        const int h = lane & 24, col = lane & 7;
+        double u[8];
+#pragma unroll
+        for (int i = 7; i >= 0; --i) {
+            double s = (i == col) ? 1.0 : 0.0;
+#pragma unroll
+            for (int m = i + 1; m < 8; ++m) s = fma(-S.D[h + i][h + m], u[m], s);
+            u[i] = s * S.rd[h + i];
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) S.U[h + i][h + col] = u[i];
+    }
+    __syncthreads();
+    {
+        // 8 to 16: thread = (half, row, column)
+        const int h = (tid >> 6) * 16, i = (tid >> 3) & 7, j = tid & 7;
+        double s = 0.0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) s = fma(S.D[h + i][h + 8 + m], S.U[h + 8 + m][h + 8 + j], s);
+        S.M[(tid >> 6) * 8 + i][j] = s;
+        __syncthreads();
+        s = 0.0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) s = fma(S.U[h + i][h + m], S.M[(tid >> 6) * 8 + m][j], s);
+        S.U[h + i][h + 8 + j] = -s;
+        __syncthreads();
+    }
+    {
+        // 16 to 32: two rows a thread
+        constexpr int kH = kW / 2;
+        const int i = tid / kH, j = tid & (kH - 1);
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int m = 0; m < kH; ++m) {
+            const double u = S.U[kH + m][kH + j];
+            s0 = fma(S.D[i][kH + m], u, s0);
+            s1 = fma(S.D[i + 8][kH + m], u, s1);
+        }
+        S.M[i][j] = s0;
+        S.M[i + 8][j] = s1;
+        __syncthreads();
+        s0 = s1 = 0.0;
+#pragma unroll
+        for (int m = 0; m < kH; ++m) {
+            const double x = S.M[m][j];
+            s0 = fma(S.U[i][m], x, s0);
+            s1 = fma(S.U[i + 8][m], x, s1);
+        }
+        S.U[i][kH + j] = -s0;
+        S.U[i + 8][kH + j] = -s1;
+        __syncthreads();
+    }
+    double *ug = v.ug + (size_t)b * 3 * kW * kW;
+#pragma unroll
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = tid + x * kThreads;
+        __stcg(ug + e, S.U[e / kW][e & (kW - 1)]);
+    }
+    publish(v.uflag + b, sy.epoch);
+    if (b >= 1) {
+        form_g(S, ug + kW * kW);
+        publish(v.gflag + b, sy.epoch);
+    }
+}
+
+// G2_b, from PREP(b)'s U_b.
+template <typename T>
+__device__ void prep2_task(const View<T> &v, int b, PrepSmem &S)
+{
+    if (b < 2) return;
+    (void)wait_column(v, b);
+    load_above(v, b, 2, S);
+    (void)__all_sync(kFull, wait_eq(v.sync, v.uflag + b, v.sync.epoch, b));
+    __syncwarp();
+    double *ug = v.ug + (size_t)b * 3 * kW * kW;
+#pragma unroll
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = threadIdx.x + x * kThreads;
+        S.U[e / kW][e & (kW - 1)] = __ldcg(ug + e);
+    }
+    __syncthreads();
+    form_g(S, ug + 2 * kW * kW);
+    publish(v.g2flag + b, v.sync.epoch);
+}
+
+// ---------------------------------------------------------------- SUB
+
+// Sum over a staged tile's rows of F_{row, column} y_row, column = lane.
+// float: y comes as pairs (hi + lo = y to 48 bits) and the sum is kept as
+// s + c: products split exactly, the running sum compensated (two-sum), so
+// that the far sums lose about 2^-46 relative to their terms at FP32 speed
+// instead of a conversion and an FMA at the FP64 rate.
+__device__ __forceinline__ void tile_dot(const double *tl, const double *y, double &s, double &)
+{
+#pragma unroll
+    for (int j = 0; j < kW; j += 2) {
+        const double2 t = *reinterpret_cast<const double2 *>(tl + j);
+        const double2 u = *reinterpret_cast<const double2 *>(y + j);
+        s = fma(t.x, u.x, s);
+        s = fma(t.y, u.y, s);
+    }
+}
+__device__ __forceinline__ void pair_fma(float f, float2 u, float &s, float &c)
+{
+    const float p = __fmul_rn(f, u.x);
+    const float e = fmaf(f, u.x, -p);
+    const float t = __fadd_rn(s, p);
+    const float b = __fsub_rn(t, s);
+    const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b));
+    s = t;
+    c = __fadd_rn(c, __fadd_rn(fmaf(f, u.y, e), r));
+}
+__device__ __forceinline__ void tile_dot(const float *tl, const double *y, float &s, float &c)
+{
+    const float4 *yp = reinterpret_cast<const float4 *>(y);  // (hi, lo) of two rows
+#pragma unroll
+    for (int j = 0; j < kW; j += 4) {
+        const float4 t = *reinterpret_cast<const float4 *>(tl + j);
+        const float4 a = yp[j / 2], b = yp[j / 2 + 1];
+        pair_fma(t.x, make_float2(a.x, a.y), s, c);
+        pair_fma(t.y, make_float2(a.z, a.w), s, c);
+        pair_fma(t.z, make_float2(b.x, b.y), s, c);
+        pair_fma(t.w, make_float2(b.z, b.w), s, c);
+    }
+}
+__device__ __forceinline__ void put_y(double *y, int lane, double x, double) { y[lane] = x; }
+__device__ __forceinline__ void put_y(double *y, int lane, double x, float)
+{
+    const float hi = (float)x;
+    reinterpret_cast<float2 *>(y)[lane] = make_float2(hi, (float)(x - (double)hi));
+}
+
+// Warp-wide bounded wait for a tagged double per lane; zeros if it gave up,
+// so that the task reaches its barriers.  `far`: a step that is not the
+// chain's next.  Such a wait polls one word (the last one written) with
+// pauses of up to 128 ns and takes the values once it is there: dozens of
+// warps wait on the newest step, and a poll of all its words by each would
+// slow the L2 slices that the chain's own stores and loads go to.
+__device__ __forceinline__ double wait_p(const SyncArgs &sy, const long long *w2, const long long *probe,
+                                         long long ep64, long long who, bool far)
+{
+    double x = 0.0;
+    if (__all_sync(kFull, get_tagged(w2, ep64, &x))) return x;
+    const long long t0 = global_ns();
+    unsigned ns = 16;
+    for (unsigned it = 1;; ++it) {
+        bool look = true;
+        if (far) {
+            look = (ld_relaxed_gpu(probe) & ~0xffffffffll) == ep64;
+            look = __any_sync(kFull, look);
+            if (!look) {
+                __nanosleep(ns);
+                if (ns < 128) ns <<= 1;
+            }
+        }
+        if (look && __all_sync(kFull, get_tagged(w2, ep64, &x))) return x;
+        // (looked at by all lanes alike: a branch of lane 0 alone would leave
+        // the warp split, and every later shuffle would wait for the halves)
+        if ((it & 31u) == 0u) {
+            const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 28);
+            if (__any_sync(kFull, late || aborted(sy))) {
+                if ((threadIdx.x & 31) == 0 && late) record_error(sy, kStatusTimeout, who);
+                return 0.0;
+            }
+        }
+    }
+}
+// Warp-wide bounded wait for the flags f[first .. last] (last - first < 32 per
+// look, one a lane), the warp staying together.
+__device__ __forceinline__ void wait_flags(const SyncArgs &sy, const int *f, int first, int last, long long who)
+{
+    for (int r0 = first; r0 <= last; r0 += 32) {
+        const int r = min(r0 + ((int)threadIdx.x & 31), last);
+        const long long t0 = global_ns();
+        unsigned ns = 16;
+        for (unsigned it = 1; !__all_sync(kFull, ld_acquire_gpu(f + r) == sy.epoch); ++it) {
+            __nanosleep(ns);
+            if (ns < 256) ns <<= 1;
+            if ((it & 15u) == 0u) {
+                const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 26);
+                if (__any_sync(kFull, late || aborted(sy))) {
+                    if ((threadIdx.x & 31) == 0 && late) record_error(sy, kStatusTimeout, who);
+                    return;
+                }
+            }
+        }
+    }
+}
+
+template <typename T>
+__device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, SubSmem<T> &S)
+{
+    constexpr int SD = pass::Stride<T>::value;
+    const SyncArgs &sy = v.sync;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long n = v.n, ld = v.ld;
+    const long long c0 = (long long)b * kW;
+    const int nc = (int)min((long long)kW, n - c0);
+    const bool active = lane < nc;
+    const long long ep64 = (long long)sy.epoch << 32;
+    long long *ptag = v.ptag + (size_t)c * v.nb * kW * 2;
+    TEAM_TRACE(c, b, 0);
+    (void)wait_column(v, b);
+    if (warp == 0) {
+        const long long o = c0 + lane + c * v.ldv;
+        S.z[lane] = (active && CHK_RECT(sy, o, n, v.kb, v.ldv)) ? (double)v.V[o] : 0.0;
+    }
+    // tiles p <= b - 3 of column block b, dealt round-robin to the warps (the
+    // dealing and the order of the sums depend on the order of the factor
+    // alone), one staged ahead
+    const int far = b - 3;  // tiles 0 .. far - 1; tile b - 3 is split over the warps below
+    // this warp's rows of U_b, of tile b - 3 and columns of G1_b and G2_b, taken
+    // before the tiles so that nothing but the chain's own values is waited
+    // for behind p_{b-3}
+    const double *ug = v.ug + (size_t)b * 3 * kW * kW + warp * kPer * kW + lane;
+    const bool ok = __all_sync(kFull, wait_eq(sy, v.uflag + b, sy.epoch, b) &&
+                                          (b < 1 || wait_eq(sy, v.gflag + b, sy.epoch, b)) &&
+                                          (b < 2 || wait_eq(sy, v.g2flag + b, sy.epoch, b)));
+    const long long o3 = (long long)(b - 3) * kW + warp * kPer + (c0 + (active ? lane : 0)) * ld;
+    double u[kPer], g1[kPer], g2[kPer], t3[kPer];
+#pragma unroll
+    for (int jj = 0; jj < kPer; ++jj) {
+        u[jj] = ok ? __ldcg(ug + jj * kW) : 0.0;
+        g1[jj] = (ok && b >= 1) ? __ldcg(ug + kW * kW + jj * kW) : 0.0;
+        g2[jj] = (ok && b >= 2) ? __ldcg(ug + 2 * kW * kW + jj * kW) : 0.0;
+        t3[jj] = (b >= 3 && active && CHK_TRI(sy, o3 + jj, n, ld)) ? (double)__ldcg(v.L + o3 + jj) : 0.0;
+    }
+    auto stage = [&](int p, int slot) {
+        if (p < far) stage_tile(sy, S.tile[warp][slot], v.L, ld, (long long)p * kW, c0, n, v.vec, false, lane);
+        pass::cp_commit();
+    };
+    stage(warp, 0);
+    T s = T(0), e = T(0);
+    int slot = 0;
+    for (int q = 1, p = warp; seg_start(q - 1, v.seg) < far; ++q) {
+        const int start = seg_start(q, v.seg);
+        const int end = min(start, far);
+        for (; p < end; p += kWarps) {
+            stage(p + kWarps, slot ^ 1);
+            const long long *w = ptag + (size_t)p * kW * 2;
+            const double y = wait_p(sy, w + 2 * lane, w + 2 * kW - 1, ep64, b, true);
+            put_y(S.y[warp], lane, y, T(0));
+            pass::cp_wait<1>();
+            __syncwarp();
+            tile_dot(S.tile[warp][slot] + lane * SD, S.y[warp], s, e);
+            __syncwarp();
+            slot ^= 1;
+        }
+        if (start <= far) {
+            // what is left of v at the start of segment q, for the sweep
+            S.part[0][warp][lane] = (double)s + (double)e;
+            s = e = T(0);
+            __syncthreads();
+            if (warp == 0) {
+                const double z = S.z[lane] - ((S.part[0][0][lane] + S.part[0][1][lane]) + (S.part[0][2][lane] + S.part[0][3][lane]));
+                S.z[lane] = z;
+                __stcg(v.snap + ((size_t)(q - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)z);
+                __threadfence();  // before the step's result, which the sweep's inputs follow from
+            }
+            __syncthreads();
+        }
+    }
+    pass::cp_wait<0>();
+    TEAM_TRACE(c, b, 1);
+    // the steps before: a lane takes the tagged value of one of its warp's eight rows
+    auto tag_of = [&](int up) { return ptag + ((size_t)(b - up) * kW + warp * kPer + (lane & (kPer - 1))) * 2; };
+    double acc = (double)s + (double)e;
+    if (b >= 3) {
+        const double y = wait_p(sy, tag_of(3), nullptr, ep64, b, false);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj) acc = fma(t3[jj], __shfl_sync(kFull, y, jj), acc);
+    }
+    S.part[0][warp][lane] = acc;
+    // (a first look at p_{b-2}, before the barrier hides its latency)
+    double y2 = 0.0, y1 = 0.0;
+    const bool have2 = b >= 2 && get_tagged(tag_of(2), ep64, &y2);
+    __syncthreads();
+    const double rv = S.z[lane] - ((S.part[0][0][lane] + S.part[0][1][lane]) + (S.part[0][2][lane] + S.part[0][3][lane]));
+    double pz = 0.0;
+#pragma unroll
+    for (int jj = 0; jj < kPer; ++jj) pz = fma(u[jj], __shfl_sync(kFull, rv, warp * kPer + jj), pz);
+    TEAM_TRACE(c, b, 2);
+    // U^T (what is left) - G2 p_{b-2} - G1 p_{b-1}: this warp's share of each
+    const bool have1 = b >= 1 && get_tagged(tag_of(1), ep64, &y1);
+    if (b > 0 && b % v.seg == 0 && warp == kWarps - 1) {
+        // what is left at the start of the column's last segment, row block b - 2
+        // (the fence passes while the warp would wait for p_{b-1})
+        __stcg(v.snap + ((size_t)(b / v.seg - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)rv);
+        __threadfence();
+    }
+    if (b >= 2) {
+        if (!__all_sync(kFull, have2)) y2 = wait_p(sy, tag_of(2), nullptr, ep64, b, false);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj) pz = fma(-g2[jj], __shfl_sync(kFull, y2, jj), pz);
+    }
+    if (b >= 1) {
+        if (!__all_sync(kFull, have1)) y1 = wait_p(sy, tag_of(1), nullptr, ep64, b, false);
+        TEAM_TRACE(c, b, 3);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj) pz = fma(-g1[jj], __shfl_sync(kFull, y1, jj), pz);
+    }
+    S.part[1][warp][lane] = pz;
+    __syncthreads();
+    if (warp == 0 && !(c == 0 && b == P.skip_publish)) {
+        const double x = (S.part[1][0][lane] + S.part[1][1][lane]) + (S.part[1][2][lane] + S.part[1][3][lane]);
+        put_tagged(ptag + ((size_t)b * kW + lane) * 2, active ? x : 0.0, ep64);
+    }
+    TEAM_TRACE(c, b, 4);
+}
+
+// ---------------------------------------------------------------- COEF
+
+__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }  // j <= i
+
+// Bounded wait of one thread for a tagged double; 0 if it gave up.  `next`:
+// the Grams' chain, polled without a pause first.
+__device__ __forceinline__ double wait_one(const SyncArgs &sy, const long long *w2, long long ep64, long long who, bool next)
+{
+    double x = 0.0;
+    for (int it = 0; next && it < 32; ++it)
+        if (get_tagged(w2, ep64, &x)) return x;
+    if (!bounded_wait(sy, [&] { return get_tagged(w2, ep64, &x); }, [] {}, who, 128)) x = 0.0;
+    return x;
+}
+
+// Row r of the block: H_r = H_b + sum_{i<r} p_i p_i^T = L D L^T, z = L^{-1} p_r and,
+// with |D_q| = sigma_q D_q,
+//   Dc_q = 1 + sum_{q'<=q} sigma_q' z_q'^2 / |D_q'|,  a_q = sigma_q z_q,
+//   b_q = z_q / (|D_q| Dc_q),  e = Dc_kb^{-1/2},  the diagonal factor Dc_kb^{1/2}.
+// The Grams of the blocks form a chain (H_{b+1} = H_b + the block's Gram)
+// that is handed on before the factors are formed.  Four lanes share a row:
+// its factor's rows are dealt to them, so that a block of eight vectors
+// takes about 60 FP64 instructions a warp and step group instead of 250.
+template <typename T>
+__device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem &S)
+{
+    const SyncArgs &sy = v.sync;
+    const int lane = threadIdx.x & 31;
+    const long long ep64 = (long long)sy.epoch << 32;
+    const int kb = v.kb, KB = v.KB, ne = KB * (KB + 1) / 2;
+    const long long r0 = (long long)b * kW;
+    const int rows = (int)min((long long)kW, v.n - r0);
+    for (int x = threadIdx.x; x < kW * kb; x += kThreads) {
+        const int q = x / kW, i = x & (kW - 1);
+        S.p[i][q] = wait_one(sy, v.ptag + (((size_t)q * v.nb + b) * kW + i) * 2, ep64, b, false);
+    }
+    __syncthreads();
+    TEAM_TRACE(0, b, 5);
+    // the prefix Grams, entry x of the packed triangle: each of `ng` threads
+    // sums its share of the rows, then adds what comes before it
+    const int ng = KB <= 4 ? 8 : 2, nr = kW / ng;
+    const int x = threadIdx.x % ne, part = threadIdx.x / ne, i0 = part * nr;
+    const bool mine = part < ng;
+    int q = 0;
+    while ((q + 1) * (q + 2) / 2 <= x) ++q;
+    const int r = x - q * (q + 1) / 2;
+    const bool in = mine && q < kb;
+    double acc = 0.0;
+    if (mine) {
+#pragma unroll 4
+        for (int i = i0; i < i0 + nr; ++i) {
+            S.H[i][x] = acc;
+            if (in) acc = fma(S.p[i][q], S.p[i][r], acc);
+        }
+        S.g[part][x] = acc;
+    }
+    __syncthreads();
+    if (mine) {
+        double before = 0.0, all = 0.0;
+        for (int m = 0; m < ng; ++m) {
+            if (m == part) before = all;
+            all += S.g[m][x];
+        }
+        double h = (q == r) ? ((v.down_mask >> q) & 1u ? -1.0 : 1.0) : 0.0;
+        if (b > 0 && in) h = wait_one(sy, v.htag + ((size_t)(b - 1) * ne + x) * 2, ep64, b, true);
+        if (in && part == 0 && b + 1 < v.nb) put_tagged(v.htag + ((size_t)b * ne + x) * 2, h + all, ep64);
+        h += before;
+#pragma unroll 4
+        for (int i = i0; i < i0 + nr; ++i) S.H[i][x] += h;
+    }
+    __syncthreads();
+    // rows threadIdx.x / 4; the four lanes of a row take the factor's rows i = sub, sub + 4, ...;
+    // row kb of the elimination is p itself, which becomes z
+    const int row = threadIdx.x >> 2, sub = threadIdx.x & 3;
+    double *h = S.H[row], *t = S.p[row];
+    for (int j = 0; j < kb; ++j) {
+        const double id = rcp_refined(h[tri(j, j)]);
+        for (int i = sub; i <= kb; i += 4) {
+            if (i <= j) continue;
+            const double lij = (i == kb ? t[j] : h[tri(i, j)]) * id;
+            if (i == kb) {
+                for (int m = j + 1; m < kb; ++m) t[m] = fma(-lij, h[tri(m, j)], t[m]);
+            } else {
+                for (int m = j + 1; m <= i; ++m) h[tri(i, m)] = fma(-lij, h[tri(m, j)], h[tri(i, m)]);
+            }
+        }
+        __syncwarp();
+        for (int i = sub; i < kb; i += 4)
+            if (i > j) h[tri(i, j)] *= id;
+        __syncwarp();
+    }
+    // the terms of Dc and the inverses, then its prefix sums
+    bool bad = false;
+    for (int q = sub; q < kb; q += 4) {
+        const double sg = (v.down_mask >> q) & 1u ? -1.0 : 1.0;
+        const double ad = sg * h[tri(q, q)];
+        bad = bad || !(ad > 0.0 && ad <= DBL_MAX);
+        const double iad = rcp_refined(ad);
+        S.z[row][q] = sg * t[q] * t[q] * iad;
+        if (row == 0 && b > 0 && (b + 2) % v.seg == 0 && (b + 2) / v.seg <= v.nbound) {
+            // a segment starts at this block: the factor of H_b for its carries
+            double *dst = v.rst + (size_t)((b + 2) / v.seg - 1) * ne;
+            for (int m = 0; m < q; ++m) __stcg(dst + tri(q, m), h[tri(q, m)]);
+            __stcg(dst + tri(q, q), iad);
+        }
+    }
+    __syncwarp();
+    double Dc = 1.0;
+    T *cf = v.coef + (size_t)(r0 + row) * 2 * KB;
+    for (int q = 0; q < KB; ++q) {
+        if (q < kb) {
+            Dc += S.z[row][q];
+            bad = bad || !(Dc > 0.0 && Dc <= DBL_MAX);
+        }
+        if ((q & 3) == sub && row < rows) {
+            if (q < kb) {
+                const double sg = (v.down_mask >> q) & 1u ? -1.0 : 1.0;
+                const double ad = sg * h[tri(q, q)];
+                cf[2 * q] = (T)(sg * t[q]);
+                cf[2 * q + 1] = (T)(t[q] * rcp_refined(ad * Dc));
+            } else {
+                cf[2 * q] = T(0);
+                cf[2 * q + 1] = T(0);
+            }
+        }
+    }
+    if (sub == 0 && row < rows) {
+        const double rD = rsqrt_refined(Dc);
+        v.escale[r0 + row] = (T)rD;
+        v.dfac[r0 + row] = Dc * rD;
+    }
+    const unsigned badm = __ballot_sync(kFull, bad && row < rows);
+    if (badm && lane == 0) record_error(sy, kStatusNotPD, r0 + ((threadIdx.x + __ffs(badm) - 1) >> 2));
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) st_release_gpu(v.cflag + b, sy.epoch);
+    TEAM_TRACE(0, b, 6);
+}
+
+// ---------------------------------------------------------------- SWEEP
+
+// The warps that share a segment.
+template <int NV>
+__device__ __forceinline__ void unit_sync(int unit)
+{
+    static_assert(NV == 1 || NV == 2 || NV == kWarps, "warps of a segment");
+    if (NV == 1) __syncwarp();
+    else if (NV == kWarps) __syncthreads();
+    else if (unit == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+    else asm volatile("bar.sync 2, 64;" ::: "memory");
+}
+
+// Segments sg0 .. sg0 + UNITS - 1 of column block j.  NV warps share a
+// segment, VW of its KB = NV VW vectors each: a tile passes from warp to
+// warp in shared memory, each applying its vectors' rotations (lane =
+// column, the carries in registers), so that NV tiles are in work at once
+// and a tile's step takes the time of VW vectors, not of KB (in double 64
+// cycles per FMA and warp: 4 us instead of 16 with eight vectors).  The
+// order of the operations on an element is that of one warp doing all
+// vectors.  Tiles and coefficients are staged one step ahead.  The warps'
+// places are turned from task to task, so that the last place, which also
+// scales and stores the tile, falls on each of the SM's four FP64 pipes in
+// turn.  A wait that runs out leaves the task running on whatever it has
+// (the launch is being aborted), so that the warps' barriers stay matched.
+template <typename T, int VW, int NV>
+__device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task, SweepSmem<T, VW * NV, NV> &S)
+{
+    using SS = SweepSmem<T, VW * NV, NV>;
+    using V16 = typename pass::Vec16<T>::type;
+    constexpr int KB = VW * NV, NS = SS::NS;
+    constexpr int SD = pass::Stride<T>::value;
+    constexpr int E = 16 / (int)sizeof(T);
+    constexpr int CPC = kW / E;  // 16-byte chunks per column segment
+    const SyncArgs &sy = v.sync;
+    const int lane = threadIdx.x & 31;
+    const int place = ((threadIdx.x >> 5) + j + task) & (kWarps - 1);
+    const int unit = place / NV, part = place % NV;
+    const int sg = task * SS::UNITS + unit, nseg = segs_of(j, v.seg);
+    if (NV < kWarps && sg >= nseg) return;  // (whole segments' warps; they share no barrier with the others)
+    typename SS::Unit &U = S.unit[unit];
+    const long long n = v.n, ld = v.ld;
+    const bool last = sg == nseg - 1;
+    const int rb = seg_start(sg, v.seg);
+    const int re = last ? j : seg_start(sg + 1, v.seg) - 1;
+    const long long c0 = (long long)j * kW;
+    const bool active = c0 + lane < n;
+    // the coefficients of the segment's rows, and of row block j: column j's
+    // substitution steps were the last readers of its tiles as they entered
+    wait_flags(sy, v.cflag, rb, re, j);
+    if (!last) wait_flags(sy, v.cflag, j, j, j);
+    // the diagonal's row block: the diagonal as it enters the pass, its
+    // factors, and what the 16-byte chunk with the diagonal holds above it
+    double dc = 0.0, df = 0.0;
+    T dch[E];
+#pragma unroll
+    for (int w = 0; w < E; ++w) dch[w] = T(0);
+    if (last && active) {
+        if (part == NV - 1) {
+            dc = __ldcg(v.dcar + c0 + lane);
+            df = __ldcg(v.dfac + c0 + lane);
+        }
+        if (part == 0) {
+            const long long o = c0 + (lane & ~(E - 1)) + (c0 + lane) * ld;
+#pragma unroll
+            for (int w = 0; w < E; ++w)
+                if (w < (lane & (E - 1)) && CHK_TRI(sy, o + w, n, ld)) dch[w] = __ldcg(v.L + o + w);
+        }
+    }
+    auto stage = [&](int t) {  // tile and coefficients of row block rb + t
+        const int r = rb + t, slot = t % NS;
+        const long long r0 = (long long)r * kW;
+        T *tl = U.tile[slot];
+        if (v.vec) {
+            // (of the diagonal tile the chunks above the diagonal's)
+            const int below = r == j ? 0 : kW;
+#pragma unroll 4
+            for (int x = part * 32 + lane; x < kW * CPC; x += NV * 32) {
+                const int cc = x / CPC, ch = x % CPC;
+                const long long o = r0 + ch * E + (c0 + cc) * ld;
+                T *d = tl + cc * SD + ch * E;
+                if (ch * E + E > cc + below) continue;
+                if (c0 + cc < n && CHK_TRI(sy, o, n, ld) && CHK_TRI(sy, o + E - 1, n, ld)) {
+                    pass::cp16(d, v.L + o);
+                } else {
+#pragma unroll
+                    for (int w = 0; w < E; ++w) d[w] = T(0);
+                }
+            }
+        } else if (part == 0) {
+            stage_tile(sy, tl, v.L, ld, r0, c0, n, false, r == j, lane);
+        }
+        const T *cf = v.coef + (size_t)r0 * 2 * KB;
+        for (int x = part * 32 + lane; x < kW * 2 * KB / E; x += NV * 32) pass::cp16(U.cf[slot] + x * E, cf + x * E);
+        if (part == NV - 1 && lane < kW / E) pass::cp16(U.e[slot] + lane * E, v.escale + r0 + lane * E);
+    };
+    stage(0);
+    pass::cp_commit();
+    T uh[VW];
+    if (sg == 0) {
+#pragma unroll
+        for (int w = 0; w < VW; ++w) {
+            const int q = part * VW + w;
+            const long long o = c0 + lane + q * v.ldv;
+            uh[w] = (active && q < v.kb && CHK_RECT(sy, o, n, v.kb, v.ldv)) ? v.V[o] : T(0);
+        }
+    } else {
+        // the carry entering row block rb is |D|^{-1} L^{-1} w of the residual w kept there
+        const T *w = v.snap + ((size_t)(sg - 1) * v.nb * kW + c0 + lane) * KB;
+        const double *h = v.rst + (size_t)(sg - 1) * (KB * (KB + 1) / 2);
+        double z[KB];
+#pragma unroll
+        for (int q = 0; q < KB; ++q) z[q] = (active && q < v.kb && q < (part + 1) * VW) ? (double)__ldcg(w + q) : 0.0;
+#pragma unroll
+        for (int q = 1; q < KB; ++q) {
+            if (q < v.kb && q < (part + 1) * VW) {
+#pragma unroll
+                for (int m = 0; m < q; ++m) z[q] = fma(-__ldcg(h + tri(q, m)), z[m], z[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < KB; ++q)
+            if (q / VW == part) uh[q % VW] = q < v.kb ? (T)(z[q] * __ldcg(h + tri(q, q))) : T(0);
+    }
+    const int ntile = re - rb + 1;
+    for (int i = 0; i < ntile + NV - 1; ++i) {
+        if (i + 1 < ntile) stage(i + 1);
+        pass::cp_commit();
+        pass::cp_wait<1>();
+        unit_sync<NV>(unit);
+        const int t = i - part, r = rb + t;
+        if (t >= 0 && t < ntile) {
+            const bool diag = r == j;
+            const int slot = t % NS;
+            T *tl = U.tile[slot];
+            V16 *colv = reinterpret_cast<V16 *>(tl + lane * SD);
+            const T *cf = U.cf[slot] + 2 * VW * part;
+            T *mycol = tl + lane * SD;
+            if (diag && part == 0 && v.vec) {
+                const int i0 = lane & ~(E - 1);
+#pragma unroll
+                for (int w = 0; w < E; ++w) mycol[i0 + w] = dch[w];
+            }
+            T x[kW];
+#pragma unroll
+            for (int k = 0; k < CPC; ++k) {
+                const V16 y = colv[k];
+#pragma unroll
+                for (int w = 0; w < E; ++w) x[k * E + w] = pass::vget<T>(y, w);
+            }
+            // (a lane past the order, and a row at or below the diagonal, keeps what it has)
+            const int rows = !active ? 0 : diag ? lane : kW;
+#pragma unroll
+            for (int k = 0; k < kW; ++k) {
+                T a[VW], b[VW];
+#pragma unroll
+                for (int w = 0; w < VW; ++w) {
+                    a[w] = cf[k * 2 * KB + 2 * w];
+                    b[w] = cf[k * 2 * KB + 2 * w + 1];
+                }
+                if (k < rows) {
+#pragma unroll
+                    for (int w = 0; w < VW; ++w) {
+                        x[k] = fma(a[w], uh[w], x[k]);
+                        uh[w] = fma(-b[w], x[k], uh[w]);
+                    }
+                }
+            }
+            if (part == NV - 1) {
+#pragma unroll
+                for (int k = 0; k < kW; ++k)
+                    if (k < rows) x[k] *= U.e[slot][k];
+            }
+#pragma unroll
+            for (int k = 0; k < CPC; ++k) {
+                V16 y;
+                T *yp = reinterpret_cast<T *>(&y);
+#pragma unroll
+                for (int w = 0; w < E; ++w) yp[w] = x[k * E + w];
+                colv[k] = y;
+            }
+            if (diag && part == NV - 1) mycol[lane] = (T)(dc * df);
+            if (part == NV - 1) {
+                const long long r0 = (long long)r * kW;
+                if (diag && active) __stcg(v.dcar + c0 + lane, dc * df);
+                __syncwarp();
+                const int ch = lane % CPC, cc0 = lane / CPC, cstep = 32 / CPC;
+                if (v.vec) {
+                    const int below = diag ? 0 : kW;
+#pragma unroll
+                    for (int k = 0; k < CPC; ++k) {
+                        const int cc = cc0 + k * cstep;
+                        const long long o = r0 + ch * E + (c0 + cc) * ld;
+                        if (c0 + cc < n && ch * E + E - 1 <= cc + below && CHK_TRI(sy, o, n, ld) && CHK_TRI(sy, o + E - 1, n, ld))
+                            __stcg(reinterpret_cast<V16 *>(v.L + o), *reinterpret_cast<const V16 *>(tl + cc * SD + ch * E));
+                    }
+                    const int i0 = lane & ~(E - 1);
+                    if (diag && active && i0 + E - 1 > lane) {
+#pragma unroll
+                        for (int w = 0; w < E; ++w)
+                            if (i0 + w <= lane && CHK_TRI(sy, r0 + i0 + w + (c0 + lane) * ld, n, ld))
+                                __stcg(v.L + r0 + i0 + w + (c0 + lane) * ld, tl[lane * SD + i0 + w]);
+                    }
+                } else {
+#pragma unroll 8
+                    for (int cc = 0; cc < kW; ++cc)
+                        if (c0 + cc < n && (!diag || lane <= cc) && CHK_TRI(sy, (r0 + lane) + (c0 + cc) * ld, n, ld))
+                            __stcg(v.L + (r0 + lane) + (c0 + cc) * ld, tl[cc * SD + lane]);
+                }
+            }
+        }
+        unit_sync<NV>(unit);  // the next step's copies may take the slot of the tile that left
+    }
+    pass::cp_wait<0>();
+    if (P.trace && last && part == 0 && lane == 0)
+        P.trace[((size_t)v.pass * kTeamKb * v.nb + j) * kTracePoints + 7] = global_ns();
+    if (v.pass + 1 < v.npass) {
+        // count the segment done for the problem's next pass; a count left by
+        // an earlier launch is first lifted to (epoch << 32)
+        __threadfence();
+        unit_sync<NV>(unit);
+        if (part == 0 && lane == 0) {
+            unsigned long long *d = reinterpret_cast<unsigned long long *>(v.sdone + j);
+            atomicMax(d, (unsigned long long)sy.epoch << 32);
+            __threadfence();
+            atomicAdd(d, 1ull);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- entry
+
+template <typename T>
+__device__ __forceinline__ const Prob &prob_of(const Launch<T> &P, int i)
+{
+    return P.probs ? P.probs[i] : P.prob0;
+}
+template <typename T>
+__device__ __forceinline__ unsigned long long *ticket_of(const Launch<T> &P, int i)
+{
+    const Prob &pr = prob_of(P, i);
+    return reinterpret_cast<unsigned long long *>(pr.progress + prob_ticket(pr.nb, pr.k));
+}
+
+// Fill the view of pass s of problem i; false if a region fails its bounds check.
+template <typename T>
+__device__ bool set_view(const Launch<T> &P, int i, int s, int epoch, View<T> &v)
+{
+    const Prob &pr = prob_of(P, i);
+    const int nb = pr.nb, kb = min(kTeamKb, pr.k - s * kTeamKb), KB = kb_inst(kb);
+    const PassRec rc = pass_rec(nb, kb);
+    char *d = pr.data + pass_data_off(nb, s);
+    v.L = static_cast<T *>(pr.L);
+    v.ldv = pr.ldv;
+    v.V = static_cast<const T *>(pr.V) + (long long)s * kTeamKb * pr.ldv;
+    v.n = pr.n;
+    v.ld = pr.ld;
+    v.nb = nb;
+    v.pass = s;
+    v.npass = passes_of(pr.k);
+    v.units = units_of(KB);
+    v.kb = kb;
+    v.KB = KB;
+    v.seg = seg_of(nb, KB);
+    v.nbound = bounds_of(nb, KB);
+    v.look = look_of(kb);
+    v.down_mask = (unsigned)(pr.down_mask >> (s * kTeamKb)) & ((1u << kb) - 1u);
+    v.vec = ((pr.ld * (long long)sizeof(T)) & 15) == 0 && (reinterpret_cast<uintptr_t>(pr.L) & 15) == 0;
+    v.ug = reinterpret_cast<double *>(d + rc.ug);
+    v.coef = reinterpret_cast<T *>(d + rc.coef);
+    v.escale = reinterpret_cast<T *>(d + rc.escale);
+    v.dfac = reinterpret_cast<double *>(d + rc.dfac);
+    v.snap = reinterpret_cast<T *>(d + rc.snap);
+    v.rst = reinterpret_cast<double *>(d + rc.rst);
+    v.dcar = reinterpret_cast<double *>(pr.data + prob_dcar(nb, pr.k));
+    v.ptag = pr.progress + pass_tag_off(nb, s);
+    v.htag = v.ptag + (size_t)kb * nb * kW * 2;
+    v.uflag = pr.iflags + (size_t)s * 4 * nb;
+    v.gflag = v.uflag + nb;
+    v.g2flag = v.gflag + nb;
+    v.cflag = v.g2flag + nb;
+    v.sdone = pr.progress + prob_ticket(nb, pr.k) + 1;
+    v.sync.abort_flag = P.ctl + kCtlAbort;
+    v.sync.status = P.status;
+    v.sync.user_info = pr.info;
+    v.sync.epoch = epoch;
+    v.sync.timeout_ns = P.timeout_ns;
+    v.sync.chk_cut = P.chk_cut;
+#ifdef CHM_CHECK
+    return CHK_REGION(v.sync, pr.data, prob_data(nb, pr.k), P.ws_data, P.ws_data_bytes) &&
+           CHK_REGION(v.sync, pr.iflags, prob_flags(nb, pr.k) * sizeof(int), P.ws_iflags, P.ws_iflags_n * sizeof(int)) &&
+           CHK_REGION(v.sync, pr.progress, prob_tags(nb, pr.k) * sizeof(long long), P.ws_progress,
+                      P.ws_progress_n * sizeof(long long)) &&
+           CHK_REGION(v.sync, d, rc.bytes, pr.data, prob_data(nb, pr.k)) &&
+           CHK_REGION(v.sync, v.dcar, (size_t)nb * kW * sizeof(double), pr.data, prob_data(nb, pr.k)) &&
+           CHK_REGION(v.sync, v.ptag, ((size_t)kb * nb * kW * 2 + (size_t)nb * KB * (KB + 1)) * sizeof(long long),
+                      pr.progress, prob_tags(nb, pr.k) * sizeof(long long)) &&
+           CHK_RECT(v.sync, (long long)s, (long long)passes_of(pr.k), 1, 1 << 30);
+#else
+    return true;
+#endif
+}
+
+// What thread 0 hands the block: a task of the problem in the view.
+enum : int { kTaskNone = 0, kTaskPrep, kTaskPrep2, kTaskSub, kTaskCoef, kTaskSweep };
+struct Picked {
+    int kind, a, b;
+};
+
+// Task number x of the pass in `v` (x counts from the pass's first task),
+// walking the block's stage cursor forward; kTaskNone past the last stage
+// (the cursor then holds the pass's task count in `first`).
+template <typename T>
+__device__ Picked task_at(const View<T> &v, int x, Stage &st)
+{
+    Picked p{kTaskNone, 0, 0};
+    const int stages = stage_count(v.nb, v.look);
+    for (; st.t < stages; ++st.t) {
+        const int c = stage_tasks(st.t, v.nb, v.kb, v.seg, v.look, v.units);
+        if (x < st.first + c) break;
+        st.first += c;
+    }
+    if (st.t >= stages) return p;
+    int y = x - st.first;
+    const int t = st.t;
+    if (t == 0) {
+        const int c = 2 * min(v.nb, kPrepAhead);
+        if (y < c) return Picked{(y & 1) ? kTaskPrep2 : kTaskPrep, y >> 1, 0};
+        y -= c;
+    }
+    if (t + kPrepAhead < v.nb) {
+        if (y < 2) return Picked{y ? kTaskPrep2 : kTaskPrep, t + kPrepAhead, 0};
+        y -= 2;
+    }
+    if (t < v.nb) {
+        if (y < v.kb) return Picked{kTaskSub, y, t};
+        y -= v.kb;
+    }
+    const int u = t - v.look;
+    if (y == 0) return Picked{kTaskCoef, u, 0};
+    return Picked{kTaskSweep, u, y - 1};
+}
+
+// One ticket of problem i: the task number, or -1 if none is left.  The
+// ticket word is read first, so that an exhausted one is not counted up.
+template <typename T>
+__device__ __forceinline__ long long take_ticket(const Launch<T> &P, int i, long long ep64)
+{
+    const long long total = prob_of(P, i).ntasks;
+    unsigned long long *w = ticket_of(P, i);
+    const long long seen = ld_relaxed_gpu(reinterpret_cast<const long long *>(w));
+    if (seen >= ep64 + total) return -1;
+    if (seen < ep64) atomicMax(w, (unsigned long long)ep64);
+    const long long x = (long long)atomicAdd(w, 1ull) - ep64;
+    return x < total ? x : -1;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) team_kernel(Launch<T> P)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    TaskSmem<T> &S = *reinterpret_cast<TaskSmem<T> *>(raw);
+    __shared__ View<T> v;
+    __shared__ Picked s_task;
+    __shared__ int s_last, s_abort;
+    int *ctl = P.ctl;
+    const int epoch = ld_relaxed_gpu(ctl + kCtlEpoch);
+    const long long ep64 = (long long)epoch << 32;
+    // thread 0's scheduling state
+    const int team = blockIdx.x % P.nteams;
+    int prob = -1;      // the problem in the view
+    Stage st{0, 0, 0};  // cursor in its task list
+    if (threadIdx.x == 0) {
+        v.pass = -1;
+        s_task.kind = kTaskNone;
+    }
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_task.kind = kTaskNone;
+            int want = -1;
+            long long x = -1;
+            if (ld_relaxed_gpu(ctl + kCtlAbort) == 0 && P.nprobs == 1) {
+                want = 0;
+                x = take_ticket(P, 0, ep64);
+            } else if (ld_relaxed_gpu(ctl + kCtlAbort) == 0) {
+                // the problem at hand, then the team's (a new one once its
+                // own is handed out), then, when no problem is left, another team's
+                if (prob >= 0) {
+                    x = take_ticket(P, prob, ep64);
+                    want = prob;
+                }
+                int *word = ctl + kCtlTeam + team;
+                for (unsigned it = 0; x < 0 && it < (1u << 22); ++it) {
+                    const int cur = ld_relaxed_gpu(word);  // problem + 1; 0: none yet, -1: one is being named
+                    if (cur < 0) {
+                        __nanosleep(64);
+                        continue;
+                    }
+                    if (cur > 0 && cur - 1 != prob) {
+                        want = cur - 1;
+                        x = take_ticket(P, want, ep64);
+                        if (x >= 0) break;
+                    }
+                    if (ld_relaxed_gpu(ctl + kCtlPairNext) >= P.nprobs) break;
+                    if (atomicCAS(word, cur, -1) != cur) continue;
+                    const int next = atomicAdd(ctl + kCtlPairNext, 1);
+                    atomicExch(word, next < P.nprobs ? next + 1 : cur);
+                    prob = -1;  // (its tickets are all taken)
+                }
+                for (int d = 1; d < P.nteams && x < 0; ++d) {
+                    int h = team + d;
+                    if (h >= P.nteams) h -= P.nteams;
+                    const int cur = ld_relaxed_gpu(ctl + kCtlTeam + h);
+                    if (cur <= 0) continue;
+                    want = cur - 1;
+                    x = take_ticket(P, want, ep64);
+                }
+            }
+            if (x >= 0) {
+                if (want != prob) {
+                    prob = want;
+                    st = Stage{0, 0, 0};
+                    v.pass = -1;
+                }
+                bool ok = true;
+                const int np = passes_of(prob_of(P, prob).k);
+                if (v.pass < 0) ok = set_view(P, prob, 0, epoch, v);
+                Picked pk = ok ? task_at(v, (int)x - st.passes, st) : Picked{kTaskNone, 0, 0};
+                while (ok && pk.kind == kTaskNone && v.pass + 1 < np) {
+                    st = Stage{0, 0, st.passes + st.first};
+                    ok = set_view(P, prob, v.pass + 1, epoch, v);
+                    if (ok) pk = task_at(v, (int)x - st.passes, st);
+                }
+                s_task = pk;
+            }
+        }
+        __syncthreads();
+        const Picked pk = s_task;
+        if (pk.kind == kTaskNone) break;
+        if (pk.kind == kTaskPrep) {
+            prep_task<T>(P, v, pk.a, S.prep);
+        } else if (pk.kind == kTaskPrep2) {
+            prep2_task<T>(v, pk.a, S.prep);
+        } else if (pk.kind == kTaskSub) {
+            sub_task<T>(P, v, pk.a, pk.b, S.sub);
+        } else if (pk.kind == kTaskCoef) {
+            coef_task<T>(P, v, pk.a, S.coef);
+        } else {
+            switch (v.KB) {
+            case 1: sweep_task<T, 1, 1>(P, v, pk.a, pk.b, S.sweep1); break;
+            case 2: sweep_task<T, 1, 2>(P, v, pk.a, pk.b, S.sweep2); break;
+            case 4: sweep_task<T, 1, 4>(P, v, pk.a, pk.b, S.sweep4); break;
+            default: sweep_task<T, 2, 4>(P, v, pk.a, pk.b, S.sweep8); break;
+            }
+        }
+    }
+
+    // The last block to finish zeroes the control words for the next launch
+    // and advances the epoch.
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(ctl + kCtlExited, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        // A wait that ran out aborted the whole launch: every problem that
+        // recorded nothing stopped unfinished, so it is marked too (info -5:
+        // stopped by another problem's failure) and none reads as complete.
+        if (threadIdx.x == 0) s_abort = ld_relaxed_gpu(ctl + kCtlAbort);
+        __syncthreads();
+        if (s_abort) {
+            for (int i = threadIdx.x; i < P.nprobs; i += blockDim.x) {
+                long long *info = prob_of(P, i).info;
+                if (info) record_one(info, kStatusTimeout, -5);
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kCtlTeam + kMaxTeams; i += blockDim.x)
+            if (i != kCtlEpoch) ctl[i] = 0;  // (the words this kernel uses; the others stay zero)
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            ctl[kCtlEpoch] = epoch + 1;
+            __threadfence();
+        }
+    }
+}
+
+#undef TEAM_TRACE
+
+}  // namespace team
+}  // namespace chm
