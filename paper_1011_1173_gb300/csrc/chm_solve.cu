@@ -4,22 +4,28 @@
 // one persistent launch per group of right-hand sides.
 //
 // A launch runs C chains of R right-hand sides each.  Tasks are taken in
-// order from a launch-wide counter by blocks of four warps:
-//   t < nb: prepare block b = t: U_b = D_b^{-1}, G_b = U_b^T L_{b-1,b}^T and
-//     H_b = U_b L_{b,b+1} (D_b the diagonal block, L_{p,b} the 32 x 32 tile in
-//     row block p and column block b), shared by every chain;
-//   then, dealt round-robin to the chains, step s = 0 .. 2 nb - 1 of each:
-//     s <  nb: y_b = D_b^{-T} (b_b - sum_{p<b} L_{p,b}^T y_p), b = s
-//     s >= nb: x_b = D_b^{-1} (y_b - sum_{q>b} L_{b,q} x_q), b = 2 nb - 1 - s
+// order from a launch-wide counter by blocks of four warps: in stage t of the
+// forward half
+//   PREP(t + 4)  U_b = D_b^{-1} and G1_b = U_b^T L_{b-1,b}^T (D_b the diagonal
+//                block, L_{p,b} the 32 x 32 tile in row block p and column
+//                block b), shared by every chain;
+//   PREP2(t + 4) G2_b = U_b^T L_{b-2,b}^T;
+//   each chain's y_b = U_b^T (b_b - sum_{p<=b-3} L_{p,b}^T y_p) - G2_b y_{b-2} - G1_b y_{b-1}, b = t;
+//   PREPH(t)     H1_b = U_b L_{b,b+1} and H2_b = U_b L_{b,b+2};
+// and in the backward half, b = nb - 1 .. 0,
+//   each chain's x_b = U_b (y_b - sum_{q>=b+3} L_{b,q} x_q) - H2_b x_{b+2} - H1_b x_{b+1}.
 // A task waits only on tasks taken before it, so the launch cannot deadlock
 // whatever the number of resident blocks.
 //
-// A forward step sums the tiles whose y is already published, forms
-// z_b = U_b^T (b_b - sum over p <= b-2) once y_{b-2} is in, and then
-// y_b = z_b - G_b y_{b-1}; a backward step mirrors it with H_b.  Between one
-// block's result and the next block's there is one 32 x 32 product (eight
-// FMAs per warp and right-hand side), one barrier and a four-way sum.
-// Results pass between blocks as epoch-tagged doubles (no fence, no flag).
+// A step sums the tiles whose y is already published, staged through shared
+// memory (a lane reads down its column), the third and fourth tiles back
+// split over the four warps, and multiplies by U; between one block's result and the next
+// block's there is one 32 x 32 product (eight FMAs per warp and right-hand
+// side), one barrier and a four-way sum.  With the two nearest tiles
+// multiplied by U beforehand a step has three steps' time from y_{b-3} on
+// (with one, y_{b-2}'s way through the tile and U set the pace: 1.7 us a step
+// at n = 5000).  Results pass between blocks as epoch-tagged doubles (no
+// fence, no flag).
 //
 // Why chains: right-hand sides do not depend on each other, and a step is
 // bound by FP64 issue (one FP64 instruction per 64 cycles and warp), so a
@@ -34,20 +40,19 @@
 #include <algorithm>
 
 #include "chm.h"
-#include "chm_device.cuh"
 #include "chm_internal.h"
-#include "chm_layout.h"
+#include "chm_sub.cuh"
 
 namespace chm {
 namespace {
 
-constexpr int kSolveThreads = 128;
-constexpr int kSolveWarps = kSolveThreads / 32;
-constexpr int kSolveRhs = 4;                       // right-hand sides per chain (largest)
-constexpr int kSolveChains = 16;                   // chains per launch (largest)
-constexpr int kRowsPerWarp = kW / kSolveWarps;     // rows (or columns) of a split tile per warp
-constexpr int kPrepMats = 3;                       // U_b, G_b and H_b
-constexpr unsigned kFull = 0xffffffffu;
+using namespace chm::sub;
+
+constexpr int kSolveRhs = 4;      // right-hand sides per chain (largest)
+constexpr int kSolveChains = 16;  // chains per launch (largest)
+constexpr int kAhead = 4;         // stages by which PREP runs ahead of the chains
+constexpr int kPrepMats = 5;      // U_b, G1_b, G2_b, H1_b and H2_b
+constexpr size_t kMat = kW * kW;
 
 template <typename T>
 struct SolveArgs {
@@ -63,9 +68,9 @@ struct SolveArgs {
     const T *Y;
     long long ys, cs;
     int back_only;
-    double *inv;      // [nb][kPrepMats][kW][kW]: U_b = D_b^{-1} (row i at i * kW), G_b and H_b
-                      // (transposed: element (i, j) at j * kW + i)
-    int *uflag;       // [nb]: U_b, G_b and H_b published (== epoch)
+    double *inv;      // [nb][kPrepMats][kW][kW]: U_b = D_b^{-1} (row i at i * kW), G1_b, G2_b, H1_b and
+                      // H2_b (transposed: element (i, j) at j * kW + i)
+    int *uflag, *gflag, *g2flag, *hflag;  // [nb] each: U, G1, G2, both H published (== epoch)
     long long *ytag;  // [C][nb][kW][R][2]: y_b as tagged doubles
     long long *xtag;  // [C][nb][kW][R][2]: x_b as tagged doubles
     int *ctl;
@@ -81,21 +86,17 @@ struct SolveArgs {
     long long chk_cut;
 };
 
-// Shared memory of a block: a preparation task's matrices or a step's
-// partial sums.
-struct PrepSmem {
-    double D[kW][kW + 1];  // diagonal block (row, column); identity beyond the order
-    double U[kW][kW + 1];  // its inverse
-    double T[kW][kW + 1];  // the tile above it, then the tile to its right
-    double M[kW / 2][kW / 2 + 1];
-    double rd[kW];         // 1 / D_ii
-};
-template <int R>
-struct SolveSmem {
-    union {
-        PrepSmem prep;
-        double part[2][kSolveWarps][R][kW];
+// Shared memory of a block: a preparation task's matrices or a step's tiles
+// and partial sums.
+template <typename T, int R>
+union SolveSmem {
+    PrepSmem prep;
+    struct {
+        T tile[kWarps][2][kW * pass::Stride<T>::value];
+        double y[kWarps][R][kW];
+        double part[2][kWarps][R][kW];
     };
+    __device__ SolveSmem() {}
 };
 
 template <int R>
@@ -104,315 +105,298 @@ __device__ __forceinline__ size_t tag_at(int blk, int i, int r)
     return (((size_t)blk * kW + i) * R + r) * 2;
 }
 
-// The whole warp waits for the R tagged values of block `blk` (lane i gets
-// row i).  `next_step` marks the wait on the previous block's result, the
-// one step of the chain: it polls at short fixed intervals (only the next
-// block's four warps wait on a fresh result, and each step gains the time a
-// longer sleep would add); every other wait backs off up to 256 ns, since
-// hundreds of warps may be waiting on older results at once.  A wait that
-// gives up (recorded as a timeout, or the launch is aborted) yields zeros,
-// so that every warp still reaches the block's barriers; the result is then
-// unspecified and the status says so.
-template <int R>
-__device__ __forceinline__ void wait_block(const SyncArgs &sy, const long long *tags, long long ep64, int blk,
-                                           long long who, double *v, bool next_step = false)
-{
-    const int lane = threadIdx.x & 31;
-    const long long *w = tags + tag_at<R>(blk, lane, 0);
-    const long long t0 = global_ns();
-    unsigned ns = next_step ? 32 : 16;
-    for (unsigned it = 0;; ++it) {
-        bool ok = true;
-#pragma unroll
-        for (int r = 0; r < R; ++r) ok = get_tagged(w + 2 * r, ep64, &v[r]) && ok;
-        if (__all_sync(kFull, ok)) return;
-        // (looked at by all lanes alike: a branch of lane 0 alone would leave
-        // the warp split, and every later shuffle would wait for the halves)
-        if ((it & 15u) == 15u) {
-            const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 28);
-            if (__any_sync(kFull, late || aborted(sy))) {
-                if (lane == 0 && late) record_error(sy, kStatusTimeout, who);
-#pragma unroll
-                for (int r = 0; r < R; ++r) v[r] = 0.0;
-                return;
-            }
-        }
-        __nanosleep(ns);
-        if (!next_step && ns < 256) ns <<= 1;
-    }
-}
-
 // Sum of the four warps' partial products of row `lane`, for each r.
-template <int R>
-__device__ __forceinline__ double part_sum(const SolveSmem<R> &S, int buf, int r, int lane)
+template <typename T, int R>
+__device__ __forceinline__ double part_sum(const SolveSmem<T, R> &S, int buf, int r, int lane)
 {
     return (S.part[buf][0][r][lane] + S.part[buf][1][r][lane]) + (S.part[buf][2][r][lane] + S.part[buf][3][r][lane]);
 }
 
-// U_b, G_b and H_b of block b.  The inverse goes by halves: with
-// D = [[D1, B], [0, D2]], U = [[U1, -U1 B U2], [0, U2]]; the two 16 x 16
-// inverses take one warp (a column per lane, 136 dependent FMAs instead of
-// the 528 of a whole column each) and the products all four.
+// The tile at row block p, column block q: F[j][m] = L[p kW + j, q kW + m] (`rows`), or
+// F[j][m] = L[p kW + m, q kW + j]; zero past the order.
+template <typename T>
+__device__ __forceinline__ void load_tile(const SolveArgs<T> &a, const SyncArgs &sy, int p, int q, bool rows, PrepSmem &S)
+{
+    (void)sy;
+#pragma unroll
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = threadIdx.x + x * kThreads, i = e & (kW - 1), j = e / kW;
+        const long long r = (long long)p * kW + i, c = (long long)q * kW + j, o = r + c * a.ld;
+        const double v = (r < a.n && c < a.n && CHK_TRI(sy, o, a.n, a.ld)) ? (double)__ldg(a.L + o) : 0.0;
+        if (rows) S.F[i][j] = v;
+        else S.F[j][i] = v;
+    }
+}
+
+// U_b, and for the forward half G1_b.
 template <typename T>
 __device__ void prep_task(const SolveArgs<T> &a, const SyncArgs &sy, int b, PrepSmem &S)
 {
-    constexpr int kH = kW / 2;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31;
     const long long n = a.n, ld = a.ld;
     const long long c0 = (long long)b * kW;
     const int nc = (int)min((long long)kW, n - c0);
-    const bool above = b >= 1 && !a.back_only;  // G_b serves the forward steps only
-
-    // the diagonal block (identity beyond the order) and the tile above it,
-    // S.T[j][m] = L[(b-1) kW + j, c0 + m]
-    for (int e = threadIdx.x; e < kW * kW; e += kSolveThreads) {
-        const int i = e & (kW - 1), j = e / kW;
-        double v = 0.0;
-        if (j < nc) {
-            if (i <= j && CHK_TRI(sy, c0 + i + (c0 + j) * ld, n, ld)) v = (double)__ldg(a.L + c0 + i + (c0 + j) * ld);
-        } else if (i == j) {
-            v = 1.0;
-        }
-        S.D[i][j] = v;
-        if (above)
-            S.T[i][j] = (j < nc && CHK_TRI(sy, c0 - kW + i + (c0 + j) * ld, n, ld))
-                            ? (double)__ldg(a.L + c0 - kW + i + (c0 + j) * ld) : 0.0;
+    const bool above = b >= 1 && !a.back_only;
+#pragma unroll
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = threadIdx.x + x * kThreads, i = e & (kW - 1), j = e / kW;
+        double d = i == j ? 1.0 : 0.0;  // identity beyond the order
+        if (j < nc && i <= j) d = CHK_TRI(sy, c0 + i + (c0 + j) * ld, n, ld) ? (double)__ldg(a.L + c0 + i + (c0 + j) * ld) : 0.0;
+        S.D[i][j] = d;
+        S.U[i][j] = 0.0;
     }
+    if (above) load_tile(a, sy, b - 1, b, true, S);
     __syncthreads();
-    if (warp == 0) {
-        double d = S.D[lane][lane];
-        if (!(d > 0.0 && d <= DBL_MAX)) {  // not a Cholesky factor
-            record_error(sy, kStatusNotPD, c0 + lane);
-            d = 1.0;
-        }
-        S.rd[lane] = 1.0 / d;
-        __syncwarp();
-        // column `col` of the inverse of diagonal half h: back substitution on D_h u = e_col
-        const int h = lane & kH, col = lane & (kH - 1);
-        double u[kH];
-#pragma unroll
-        for (int i = kH - 1; i >= 0; --i) {
-            double s = (i == col) ? 1.0 : 0.0;
-#pragma unroll
-            for (int m = i + 1; m < kH; ++m) s = fma(-S.D[h + i][h + m], u[m], s);
-            u[i] = s * S.rd[h + i];
-        }
-#pragma unroll
-        for (int i = 0; i < kH; ++i) {
-            S.U[h + i][h + col] = u[i];
-            if (h) S.U[h + i][col] = 0.0;
-        }
+    double d = S.D[lane][lane];
+    if (threadIdx.x < 32 && !(d > 0.0 && d <= DBL_MAX)) {  // not a Cholesky factor
+        record_error(sy, kStatusNotPD, c0 + lane);
+        d = 1.0;
     }
-    __syncthreads();
-    // M = B U2, then U12 = -U1 M: two outputs a thread, a row pair per half warp
-    const int mi = threadIdx.x / kH, mj = threadIdx.x & (kH - 1);
+    __syncwarp();
+    invert_block(S, d);
+    double *inv = a.inv + (size_t)b * kPrepMats * kMat;
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        const int i = mi + 8 * v;
-        double s = 0.0;
-#pragma unroll
-        for (int m = 0; m < kH; ++m) s = fma(S.D[i][kH + m], S.U[kH + m][kH + mj], s);
-        S.M[i][mj] = s;
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = threadIdx.x + x * kThreads;
+        __stcg(inv + e, S.U[e / kW][e & (kW - 1)]);
     }
-    __syncthreads();
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        const int i = mi + 8 * v;
-        double s = 0.0;
-#pragma unroll
-        for (int m = 0; m < kH; ++m) s = fma(S.U[i][m], S.M[m][mj], s);
-        S.U[i][kH + mj] = -s;
-    }
-    __syncthreads();
-    double *inv = a.inv + (size_t)b * kPrepMats * kW * kW;
-    for (int e = threadIdx.x; e < kW * kW; e += kSolveThreads) __stcg(inv + e, S.U[e / kW][e & (kW - 1)]);
-    // G: G[i][j] = sum_{m<=i} U[m][i] T[j][m]; rows i = warp, warp + 4, ... (so
-    // that the four warps' triangles weigh the same), lane = j
+    publish(a.uflag + b, sy.epoch);
     if (above) {
-        for (int ii = 0; ii < kRowsPerWarp; ++ii) {
-            const int i = ii * kSolveWarps + warp;
-            double s0 = 0.0, s1 = 0.0;
-            for (int m = 0; m <= i; m += 2) {
-                s0 = fma(S.U[m][i], S.T[lane][m], s0);
-                if (m < i) s1 = fma(S.U[m + 1][i], S.T[lane][m + 1], s1);
-            }
-            __stcg(inv + kW * kW + (size_t)lane * kW + i, s0 + s1);
-        }
+        form_g(S, inv + kMat);
+        publish(a.gflag + b, sy.epoch);
     }
-    // H: H[i][j] = sum_{m>=i} U[i][m] T[m][j], T the tile to the right of the diagonal block
-    if (b + 1 < a.nb) {
-        __syncthreads();
-        const long long q1 = c0 + kW;
-        const int nc1 = (int)min((long long)kW, n - q1);
-        for (int e = threadIdx.x; e < kW * kW; e += kSolveThreads) {
-            const int i = e & (kW - 1), j = e / kW;
-            S.T[i][j] = (j < nc1 && CHK_TRI(sy, c0 + i + (q1 + j) * ld, n, ld)) ? (double)__ldg(a.L + c0 + i + (q1 + j) * ld)
-                                                                                : 0.0;
-        }
-        __syncthreads();
-        for (int ii = 0; ii < kRowsPerWarp; ++ii) {
-            const int i = ii * kSolveWarps + warp;
-            double s0 = 0.0, s1 = 0.0;
-            for (int m = kW - 1; m >= i; m -= 2) {
-                s0 = fma(S.U[i][m], S.T[m][lane], s0);
-                if (m > i) s1 = fma(S.U[i][m - 1], S.T[m - 1][lane], s1);
-            }
-            __stcg(inv + 2 * kW * kW + (size_t)lane * kW + i, s0 + s1);
-        }
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) st_release_gpu(a.uflag + b, sy.epoch);
 }
 
-// The block's four warps wait for U_b, G_b and H_b; false if the wait gave up.
+// U_b from PREP(b).
 template <typename T>
-__device__ __forceinline__ bool wait_prep(const SolveArgs<T> &a, const SyncArgs &sy, int b)
+__device__ __forceinline__ const double *take_u(const SolveArgs<T> &a, const SyncArgs &sy, int b, PrepSmem &S)
 {
-    const bool ok = __all_sync(kFull, wait_eq(sy, a.uflag + b, sy.epoch, b));
-    __syncwarp();
-    return ok;
+    wait_flags(sy, a.uflag, b, b, b);
+    const double *inv = a.inv + (size_t)b * kPrepMats * kMat;
+#pragma unroll
+    for (int x = 0; x < kW * kW / kThreads; ++x) {
+        const int e = threadIdx.x + x * kThreads;
+        S.U[e / kW][e & (kW - 1)] = __ldcg(inv + e);
+    }
+    return inv;
+}
+
+// G2_b.
+template <typename T>
+__device__ void prep2_task(const SolveArgs<T> &a, const SyncArgs &sy, int b, PrepSmem &S)
+{
+    if (b < 2) return;
+    load_tile(a, sy, b - 2, b, true, S);
+    take_u(a, sy, b, S);
+    __syncthreads();
+    form_g(S, a.inv + ((size_t)b * kPrepMats + 2) * kMat);
+    publish(a.g2flag + b, sy.epoch);
+}
+
+// H1_b and H2_b: out[j kW + i] = H[i][j] = sum_{m>=i} U[i][m] L[m, j]; rows
+// i = warp, warp + 4, ..., lane = j (see form_g).
+template <typename T>
+__device__ void preph_task(const SolveArgs<T> &a, const SyncArgs &sy, int b, PrepSmem &S)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    take_u(a, sy, b, S);
+    for (int h = 1; h <= 2 && b + h < a.nb; ++h) {
+        load_tile(a, sy, b, b + h, false, S);
+        __syncthreads();
+        double acc[kPer];
+#pragma unroll
+        for (int ii = 0; ii < kPer; ++ii) acc[ii] = 0.0;
+#pragma unroll
+        for (int m = 0; m < kW; ++m) {
+            const double f = S.F[lane][m];
+#pragma unroll
+            for (int ii = 0; ii <= m / kWarps; ++ii) acc[ii] = fma(S.U[ii * kWarps + warp][m], f, acc[ii]);
+        }
+        double *out = a.inv + ((size_t)b * kPrepMats + 2 + h) * kMat;
+#pragma unroll
+        for (int ii = 0; ii < kPer; ++ii) __stcg(out + (size_t)lane * kW + ii * kWarps + warp, acc[ii]);
+        __syncthreads();
+    }
+    publish(a.hflag + b, sy.epoch);
+}
+
+// t[j] = L[row j, column lane] of a staged tile, in double.
+template <typename T>
+__device__ __forceinline__ void tile_column(const T *tl, double (&t)[kW])
+{
+    constexpr int E = 16 / (int)sizeof(T);
+    using V16 = typename pass::Vec16<T>::type;
+#pragma unroll
+    for (int j = 0; j < kW; j += E) {
+        const V16 x = *reinterpret_cast<const V16 *>(tl + j);
+#pragma unroll
+        for (int e = 0; e < E; ++e) t[j + e] = (double)pass::vget<T>(x, e);
+    }
+}
+// acc[r] += sum over the tile's 32 entries of t[j] y[r][j].
+template <int R>
+__device__ __forceinline__ void tile_sum(const double (&t)[kW], const double (*y)[kW], double (&acc)[R])
+{
+#pragma unroll
+    for (int j = 0; j < kW; j += 2)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const double2 u = *reinterpret_cast<const double2 *>(&y[r][j]);
+            acc[r] = fma(t[j], u.x, acc[r]);
+            acc[r] = fma(t[j + 1], u.y, acc[r]);
+        }
 }
 
 // Chain c's step at block b, forward.
 template <typename T, int R>
-__device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int c, int b, SolveSmem<R> &S)
+__device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int c, int b, SolveSmem<T, R> &S)
 {
+    constexpr int SD = pass::Stride<T>::value;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long ld = a.ld;
+    const long long n = a.n, ld = a.ld;
     const long long c0 = (long long)b * kW;
-    const int nc = (int)min((long long)kW, a.n - c0);
+    const int nc = (int)min((long long)kW, n - c0);
     const bool active = lane < nc;
-    const long long who = b;
     const int r0 = c * R;  // this chain's first right-hand side
     long long *ytag = a.ytag + (size_t)c * a.nb * kW * R * 2;
+    const bool vec = ((ld * (long long)sizeof(T)) & 15) == 0 && (reinterpret_cast<uintptr_t>(a.L) & 15) == 0;
 
     double rhs[R];
 #pragma unroll
     for (int r = 0; r < R; ++r)
-        rhs[r] = (active && r0 + r < a.nr && CHK_RECT(sy, c0 + lane + (r0 + r) * a.ldb, a.n, a.nr, a.ldb))
+        rhs[r] = (active && r0 + r < a.nr && CHK_RECT(sy, c0 + lane + (r0 + r) * a.ldb, n, a.nr, a.ldb))
                      ? (double)a.B[c0 + lane + (r0 + r) * a.ldb] : 0.0;
-    // tiles p <= b - 3 of column block b, dealt round-robin to the warps (a
-    // fixed order of the sums: results do not depend on timing); lane =
-    // column of the block, the tile's 32 rows read down the column
+    const int far = b - 4;  // tiles 0 .. far - 1; tiles b - 4 and b - 3 are split over the warps below
+    auto stage = [&](int p, int slot) {
+        if (p < far) stage_tile(sy, S.tile[warp][slot], a.L, ld, (long long)p * kW, c0, n, vec, false, lane);
+        pass::cp_commit();
+    };
+    stage(warp, 0);
+    // this warp's columns of G1_b and G2_b, taken before the tiles so that
+    // behind y_{b-4} nothing but the chain's own values is waited for
+    wait_flags(sy, a.uflag, b, b, b);
+    if (b >= 1) wait_flags(sy, a.gflag, b, b, b);
+    if (b >= 2) wait_flags(sy, a.g2flag, b, b, b);
+    const double *inv = a.inv + (size_t)b * kPrepMats * kMat + warp * kPer * kW + lane;
+    double g1[kPer], g2[kPer];
+#pragma unroll
+    for (int jj = 0; jj < kPer; ++jj) {
+        g1[jj] = b >= 1 ? __ldcg(inv + kMat + jj * kW) : 0.0;
+        g2[jj] = b >= 2 ? __ldcg(inv + 2 * kMat + jj * kW) : 0.0;
+    }
+    // tiles p <= b - 5 of column block b, dealt round-robin to the warps (a
+    // fixed order of the sums: results do not depend on timing)
     double acc[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = 0.0;
-    const long long colo = (c0 + (active ? lane : 0)) * ld;
-    const T *col = a.L + colo;
-    for (int p = warp; p <= b - 3; p += kSolveWarps) {
-        const T *src = col + (long long)p * kW;
+    int slot = 0;
+    for (int p = warp; p < far; p += kWarps) {
+        stage(p + kWarps, slot ^ 1);
+        // (the tile's column in registers, and in double, before y is waited for)
+        pass::cp_wait<1>();
+        __syncwarp();
         double t[kW];
+        tile_column<T>(S.tile[warp][slot] + lane * SD, t);
+        const long long *w = ytag + tag_at<R>(p, 0, 0);
+        double y[R];
+        // (a warp's last tile is waited for as closely as the chain's next steps)
+        wait_vals<R>(sy, w + tag_at<R>(0, lane, 0), p + kWarps < far ? w + tag_at<R>(1, 0, 0) - 1 : nullptr, ep64, b, y);
 #pragma unroll
-        for (int j = 0; j < kW; ++j)
-            t[j] = (active && CHK_TRI(sy, colo + (long long)p * kW + j, a.n, ld)) ? (double)__ldg(src + j) : 0.0;
-        double yv[R];
-        wait_block<R>(sy, ytag, ep64, p, who, yv);
-#pragma unroll
-        for (int j = 0; j < kW; ++j)
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] = fma(t[j], __shfl_sync(kFull, yv[r], j), acc[r]);
+        for (int r = 0; r < R; ++r) S.y[warp][r][lane] = y[r];
+        __syncwarp();
+        tile_sum<R>(t, S.y[warp], acc);
+        __syncwarp();
+        slot ^= 1;
     }
-    // this warp's rows of U_b and columns of G_b (see the products below)
-    const bool ok = wait_prep(a, sy, b);
-    const double *inv = a.inv + (size_t)b * kPrepMats * kW * kW;
-    double u[kRowsPerWarp], g[kRowsPerWarp];
+    pass::cp_wait<0>();
+    // the steps before: a lane takes the values of one of its warp's eight rows
+    auto tag_of = [&](int up) { return ytag + tag_at<R>(b - up, warp * kPer + (lane & (kPer - 1)), 0); };
+    // this warp's rows of tiles b - 4 and b - 3, and of U_b
+    const long long o4 = (long long)(b - 4) * kW + warp * kPer + (c0 + (active ? lane : 0)) * ld;
+    double t4[kPer], t3[kPer], u[kPer];
 #pragma unroll
-    for (int jj = 0; jj < kRowsPerWarp; ++jj) {
-        const int j = warp * kRowsPerWarp + jj;
-        u[jj] = ok ? __ldcg(inv + j * kW + lane) : 0.0;
-        g[jj] = (ok && b >= 1) ? __ldcg(inv + kW * kW + j * kW + lane) : 0.0;
+    for (int jj = 0; jj < kPer; ++jj) {
+        t4[jj] = (b >= 4 && active && CHK_TRI(sy, o4 + jj, n, ld)) ? (double)__ldg(a.L + o4 + jj) : 0.0;
+        t3[jj] = (b >= 3 && active && CHK_TRI(sy, o4 + kW + jj, n, ld)) ? (double)__ldg(a.L + o4 + kW + jj) : 0.0;
     }
-    // tile b - 2: its rows split over the warps
-    if (b >= 2) {
-        const T *src = col + (long long)(b - 2) * kW + warp * kRowsPerWarp;
-        double t[kRowsPerWarp];
+    if (b >= 4) {
+        double y[R];
+        wait_vals<R>(sy, tag_of(4), nullptr, ep64, b, y);
 #pragma unroll
-        for (int jj = 0; jj < kRowsPerWarp; ++jj) t[jj] = active ? (double)__ldg(src + jj) : 0.0;
-        double yv[R];
-        wait_block<R>(sy, ytag, ep64, b - 2, who, yv);
+        for (int jj = 0; jj < kPer; ++jj)
 #pragma unroll
-        for (int jj = 0; jj < kRowsPerWarp; ++jj)
+            for (int r = 0; r < R; ++r) acc[r] = fma(t4[jj], __shfl_sync(kFull, y[r], jj), acc[r]);
+    }
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-                acc[r] = fma(t[jj], __shfl_sync(kFull, yv[r], warp * kRowsPerWarp + jj), acc[r]);
+    for (int jj = 0; jj < kPer; ++jj) u[jj] = __ldcg(inv + jj * kW);
+    if (b >= 3) {
+        double y[R];
+        wait_vals<R>(sy, tag_of(3), nullptr, ep64, b, y);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj)
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = fma(t3[jj], __shfl_sync(kFull, y[r], jj), acc[r]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) S.part[0][warp][r][lane] = acc[r];
     __syncthreads();
-    double rv[R];  // b_b - sum_{p <= b-2} L_{p,b}^T y_p, row `lane`
-#pragma unroll
-    for (int r = 0; r < R; ++r) rv[r] = rhs[r] - part_sum(S, 0, r, lane);
-    // z_b = U^T r: z_i = sum_{j <= i} U_ji r_j, the j split over the warps
     double pz[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) pz[r] = 0.0;
+    for (int r = 0; r < R; ++r) {
+        const double rv = rhs[r] - part_sum(S, 0, r, lane);
+        pz[r] = 0.0;
 #pragma unroll
-    for (int jj = 0; jj < kRowsPerWarp; ++jj) {
-        const int j = warp * kRowsPerWarp + jj;
+        for (int jj = 0; jj < kPer; ++jj) pz[r] = fma(u[jj], __shfl_sync(kFull, rv, warp * kPer + jj), pz[r]);
+    }
+    if (b >= 2) {
+        double y[R];
+        wait_vals<R>(sy, tag_of(2), nullptr, ep64, b, y);
 #pragma unroll
-        for (int r = 0; r < R; ++r) pz[r] = fma(u[jj], __shfl_sync(kFull, rv[r], j), pz[r]);
+        for (int jj = 0; jj < kPer; ++jj)
+#pragma unroll
+            for (int r = 0; r < R; ++r) pz[r] = fma(-g2[jj], __shfl_sync(kFull, y[r], jj), pz[r]);
+    }
+    if (b >= 1) {
+        double y[R];
+        wait_vals<R>(sy, tag_of(1), nullptr, ep64, b, y);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj)
+#pragma unroll
+            for (int r = 0; r < R; ++r) pz[r] = fma(-g1[jj], __shfl_sync(kFull, y[r], jj), pz[r]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) S.part[1][warp][r][lane] = pz[r];
     __syncthreads();
-    double z[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) z[r] = part_sum(S, 1, r, lane);
-    // (part[0] is free again: every warp read it before the barrier above)
-    // y_b = z_b - G_b y_{b-1}: the step that waits on the previous block
-    double py[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) py[r] = 0.0;
-    if (b >= 1) {
-        double yv[R];
-        wait_block<R>(sy, ytag, ep64, b - 1, who, yv, true);
-#pragma unroll
-        for (int jj = 0; jj < kRowsPerWarp; ++jj)
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                py[r] = fma(g[jj], __shfl_sync(kFull, yv[r], warp * kRowsPerWarp + jj), py[r]);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) S.part[0][warp][r][lane] = py[r];
-    __syncthreads();
     if (warp == 0) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) put_tagged(ytag + tag_at<R>(b, lane, r), z[r] - part_sum(S, 0, r, lane), ep64);
+        for (int r = 0; r < R; ++r) put_tagged(ytag + tag_at<R>(b, lane, r), part_sum(S, 1, r, lane), ep64);
     }
 }
 
 // Chain c's step at block b, backward.
 template <typename T, int R>
-__device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int c, int b,
-                              SolveSmem<R> &S)
+__device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long long ep64, int c, int b, SolveSmem<T, R> &S)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long n = a.n, ld = a.ld;
     const long long c0 = (long long)b * kW;
     const int nc = (int)min((long long)kW, n - c0);
     const bool active = lane < nc;
-    const long long who = b;
-    const bool has_next = b + 1 < a.nb;
-    const int r0 = c * R;
-    long long *xtag = a.xtag + (size_t)c * a.nb * kW * R * 2;
+    const int r0 = c * R, nb = a.nb;
+    long long *xtag = a.xtag + (size_t)c * nb * kW * R * 2;
 
-    // this warp's columns of U_b and H_b (see the products below)
-    const bool ok = wait_prep(a, sy, b);
-    const double *inv = a.inv + (size_t)b * kPrepMats * kW * kW;
-    double u[kRowsPerWarp], h[kRowsPerWarp];
+    // this warp's columns of H1_b and H2_b
+    wait_flags(sy, a.uflag, b, b, b);
+    wait_flags(sy, a.hflag, b, b, b);
+    const double *inv = a.inv + (size_t)b * kPrepMats * kMat;
+    double h1[kPer], h2[kPer];
 #pragma unroll
-    for (int jj = 0; jj < kRowsPerWarp; jj += 2) {
-        const int j = warp * kRowsPerWarp + jj;
-        const double2 v = ok ? __ldcg(reinterpret_cast<const double2 *>(inv + lane * kW + j)) : make_double2(0.0, 0.0);
-        u[jj] = v.x;
-        u[jj + 1] = v.y;
+    for (int jj = 0; jj < kPer; ++jj) {
+        const int j = warp * kPer + jj;
+        h1[jj] = b + 1 < nb ? __ldcg(inv + 3 * kMat + j * kW + lane) : 0.0;
+        h2[jj] = b + 2 < nb ? __ldcg(inv + 4 * kMat + j * kW + lane) : 0.0;
     }
-#pragma unroll
-    for (int jj = 0; jj < kRowsPerWarp; ++jj)
-        h[jj] = (ok && has_next) ? __ldcg(inv + 2 * kW * kW + (warp * kRowsPerWarp + jj) * kW + lane) : 0.0;
-
-    // tiles q >= b + 3 of row block b, from the last one up, dealt
+    // tiles q >= b + 5 of row block b, from the last one up, dealt
     // round-robin to the warps; lane = row of the block, so each column of a
     // tile is one coalesced read
     double acc[R];
@@ -420,37 +404,21 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
     for (int r = 0; r < R; ++r) acc[r] = 0.0;
     const long long rowo = c0 + (active ? lane : 0);
     const T *row = a.L + rowo;
-    for (int q = a.nb - 1 - warp; q >= b + 3; q -= kSolveWarps) {
+    for (int q = nb - 1 - warp; q >= b + 5; q -= kWarps) {
         const long long q0 = (long long)q * kW;
         const int ncq = (int)min((long long)kW, n - q0);
         double t[kW];
 #pragma unroll
         for (int i = 0; i < kW; ++i)
             t[i] = (active && i < ncq && CHK_TRI(sy, rowo + (q0 + i) * ld, n, ld)) ? (double)__ldg(row + (q0 + i) * ld) : 0.0;
-        double xv[R];
-        wait_block<R>(sy, xtag, ep64, q, who, xv);
+        const long long *w = xtag + tag_at<R>(q, 0, 0);
+        double x[R];
+        wait_vals<R>(sy, w + tag_at<R>(0, lane, 0), q - kWarps >= b + 5 ? w + tag_at<R>(1, 0, 0) - 1 : nullptr, ep64, b, x);
 #pragma unroll
-        for (int i = 0; i < kW; ++i)
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] = fma(t[i], __shfl_sync(kFull, xv[r], i), acc[r]);
-    }
-    // tile b + 2: its columns split over the warps
-    if (b + 2 < a.nb) {
-        const long long q0 = (long long)(b + 2) * kW;
-        const int ncq = (int)min((long long)kW, n - q0);
-        double t[kRowsPerWarp];
-#pragma unroll
-        for (int cc = 0; cc < kRowsPerWarp; ++cc) {
-            const int i = warp * kRowsPerWarp + cc;
-            t[cc] = (active && i < ncq && CHK_TRI(sy, rowo + (q0 + i) * ld, n, ld)) ? (double)__ldg(row + (q0 + i) * ld) : 0.0;
-        }
-        double xv[R];
-        wait_block<R>(sy, xtag, ep64, b + 2, who, xv);
-#pragma unroll
-        for (int cc = 0; cc < kRowsPerWarp; ++cc)
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                acc[r] = fma(t[cc], __shfl_sync(kFull, xv[r], warp * kRowsPerWarp + cc), acc[r]);
+        for (int r = 0; r < R; ++r) S.y[warp][r][lane] = x[r];
+        __syncwarp();
+        tile_sum<R>(t, S.y[warp], acc);
+        __syncwarp();
     }
     // y_b: this chain's forward result, or the caller's
     double yv[R];
@@ -459,61 +427,93 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
         for (int r = 0; r < R; ++r)
             yv[r] = (active && r0 + r < a.nr) ? (double)__ldcg(a.Y + (c0 + lane) * a.ys + (r0 + r) * a.cs) : 0.0;
     } else {
-        wait_block<R>(sy, a.ytag + (size_t)c * a.nb * kW * R * 2, ep64, b, who, yv);
+        wait_vals<R>(sy, a.ytag + (size_t)c * nb * kW * R * 2 + tag_at<R>(b, lane, 0), nullptr, ep64, b, yv);
+    }
+    auto tag_of = [&](int dn) { return xtag + tag_at<R>(b + dn, warp * kPer + (lane & (kPer - 1)), 0); };
+    // this warp's columns of tiles b + 4 and b + 3, and of U_b
+    double t4[kPer], t3[kPer], u[kPer];
+#pragma unroll
+    for (int jj = 0; jj < kPer; ++jj) {
+        const long long q3 = (long long)(b + 3) * kW + warp * kPer + jj, q4 = q3 + kW;
+        t4[jj] = (active && q4 < n && CHK_TRI(sy, rowo + q4 * ld, n, ld)) ? (double)__ldg(row + q4 * ld) : 0.0;
+        t3[jj] = (active && q3 < n && CHK_TRI(sy, rowo + q3 * ld, n, ld)) ? (double)__ldg(row + q3 * ld) : 0.0;
+    }
+    if (b + 4 < nb) {
+        double x[R];
+        wait_vals<R>(sy, tag_of(4), nullptr, ep64, b, x);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj)
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = fma(t4[jj], __shfl_sync(kFull, x[r], jj), acc[r]);
+    }
+#pragma unroll
+    for (int jj = 0; jj < kPer; jj += 2) {
+        const double2 x = __ldcg(reinterpret_cast<const double2 *>(inv + lane * kW + warp * kPer + jj));
+        u[jj] = x.x;
+        u[jj + 1] = x.y;
+    }
+    if (b + 3 < nb) {
+        double x[R];
+        wait_vals<R>(sy, tag_of(3), nullptr, ep64, b, x);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj)
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = fma(t3[jj], __shfl_sync(kFull, x[r], jj), acc[r]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) S.part[0][warp][r][lane] = acc[r];
     __syncthreads();
-    double rv[R];  // y_b - sum_{q >= b+2} L_{b,q} x_q, row `lane`
-#pragma unroll
-    for (int r = 0; r < R; ++r) rv[r] = yv[r] - part_sum(S, 0, r, lane);
-    // z'_b = U r: z_i = sum_{j >= i} U_ij r_j, the j split over the warps
     double pz[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) pz[r] = 0.0;
+    for (int r = 0; r < R; ++r) {
+        const double rv = yv[r] - part_sum(S, 0, r, lane);
+        pz[r] = 0.0;
 #pragma unroll
-    for (int jj = 0; jj < kRowsPerWarp; ++jj) {
-        const int j = warp * kRowsPerWarp + jj;
+        for (int jj = 0; jj < kPer; ++jj) pz[r] = fma(u[jj], __shfl_sync(kFull, rv, warp * kPer + jj), pz[r]);
+    }
+    if (b + 2 < nb) {
+        double x[R];
+        wait_vals<R>(sy, tag_of(2), nullptr, ep64, b, x);
 #pragma unroll
-        for (int r = 0; r < R; ++r) pz[r] = fma(u[jj], __shfl_sync(kFull, rv[r], j), pz[r]);
+        for (int jj = 0; jj < kPer; ++jj)
+#pragma unroll
+            for (int r = 0; r < R; ++r) pz[r] = fma(-h2[jj], __shfl_sync(kFull, x[r], jj), pz[r]);
+    }
+    if (b + 1 < nb) {
+        double x[R];
+        wait_vals<R>(sy, tag_of(1), nullptr, ep64, b, x);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj)
+#pragma unroll
+            for (int r = 0; r < R; ++r) pz[r] = fma(-h1[jj], __shfl_sync(kFull, x[r], jj), pz[r]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) S.part[1][warp][r][lane] = pz[r];
     __syncthreads();
-    double z[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) z[r] = part_sum(S, 1, r, lane);
-    // x_b = z'_b - H_b x_{b+1}: the step that waits on the previous block
-    double px[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) px[r] = 0.0;
-    if (has_next) {
-        double xv[R];
-        wait_block<R>(sy, xtag, ep64, b + 1, who, xv, true);
-#pragma unroll
-        for (int jj = 0; jj < kRowsPerWarp; ++jj)
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                px[r] = fma(h[jj], __shfl_sync(kFull, xv[r], warp * kRowsPerWarp + jj), px[r]);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) S.part[0][warp][r][lane] = px[r];
-    __syncthreads();
     if (warp == 0) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const double x = z[r] - part_sum(S, 0, r, lane);
+            const double x = part_sum(S, 1, r, lane);
             put_tagged(xtag + tag_at<R>(b, lane, r), x, ep64);
-            if (active && r0 + r < a.nr && CHK_RECT(sy, c0 + lane + (r0 + r) * a.ldb, a.n, a.nr, a.ldb))
+            if (active && r0 + r < a.nr && CHK_RECT(sy, c0 + lane + (r0 + r) * a.ldb, n, a.nr, a.ldb))
                 a.B[c0 + lane + (r0 + r) * a.ldb] = (T)x;
         }
     }
 }
 
-template <typename T, int R>
-__global__ void __launch_bounds__(kSolveThreads) solve_kernel(SolveArgs<T> a)
+// Tasks of a launch: 2 kAhead to start with, then per stage kStageExtra and
+// one per chain (in the backward half of both: the chains' alone).
+constexpr int kStageExtra = 3;
+__host__ __device__ inline int solve_tasks(int nb, int chains, bool back_only)
 {
-    __shared__ SolveSmem<R> S;
+    return 2 * kAhead + nb * (kStageExtra + chains) + (back_only ? 0 : nb * chains);
+}
+
+template <typename T, int R>
+__global__ void __launch_bounds__(kThreads, R == 1 ? 3 : 2) solve_kernel(SolveArgs<T> a)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    SolveSmem<T, R> &S = *reinterpret_cast<SolveSmem<T, R> *>(raw);
     __shared__ int s_task, s_last;
     SyncArgs sy;
     sy.abort_flag = a.ctl + kCtlAbort;
@@ -526,24 +526,57 @@ __global__ void __launch_bounds__(kSolveThreads) solve_kernel(SolveArgs<T> a)
     const size_t tags = (size_t)a.chains * a.nb * kW * R * 2;
     // bounds-checked builds: the workspace regions inside their allocations
     const bool ws_in = CHK_REGION(sy, a.inv, (size_t)a.nb * kPrepMats * kW * kW * sizeof(double), a.ws_data, a.ws_data_bytes) &&
-                       CHK_REGION(sy, a.uflag, (size_t)a.nb * sizeof(int), a.ws_iflags, a.ws_iflags_n * sizeof(int)) &&
+                       CHK_REGION(sy, a.uflag, 4 * (size_t)a.nb * sizeof(int), a.ws_iflags, a.ws_iflags_n * sizeof(int)) &&
                        CHK_REGION(sy, a.ytag, tags * sizeof(long long), a.ws_progress, a.ws_progress_n * sizeof(long long)) &&
                        CHK_REGION(sy, a.xtag, tags * sizeof(long long), a.ws_progress, a.ws_progress_n * sizeof(long long));
     (void)tags;
 
-    const int nb = a.nb, steps = a.back_only ? nb : 2 * nb;
+    const int nb = a.nb, total = solve_tasks(nb, a.chains, a.back_only);
+    const int per = kStageExtra + a.chains;
     for (;;) {
         if (threadIdx.x == 0) s_task = (!ws_in || aborted(sy)) ? -1 : atomicAdd(a.ctl + kCtlPairNext, 1);
         __syncthreads();
         const int t = s_task;
-        if (t < 0 || t >= nb + a.chains * steps) break;
-        if (t < nb) {
-            // a back substitution starts at the last block
-            prep_task<T>(a, sy, a.back_only ? nb - 1 - t : t, S.prep);
+        if (t < 0 || t >= total) break;
+        // the task: a preparation (0 PREP, 1 PREP2, 2 PREPH) of the i-th block the
+        // launch comes to, or chain c's step
+        int prep = -1, i = 0, c = 0, s = 0;
+        if (t < 2 * kAhead) {
+            prep = t & 1;
+            i = t >> 1;
+        } else if (t < 2 * kAhead + nb * per) {
+            const int x = t - 2 * kAhead, r = x % per;
+            s = x / per;
+            if (r < 2) {
+                prep = r;
+                i = s + kAhead;
+            } else if (r < 2 + a.chains) {
+                c = r - 2;
+            } else {
+                prep = 2;
+                i = s;
+            }
         } else {
-            const int c = (t - nb) % a.chains, s = (t - nb) / a.chains + (a.back_only ? nb : 0);
-            if (s < nb) forward_task<T, R>(a, sy, ep64, c, s, S);
-            else backward_task<T, R>(a, sy, ep64, c, 2 * nb - 1 - s, S);
+            const int x = t - 2 * kAhead - nb * per;
+            c = x % a.chains;
+            s = nb + x / a.chains;
+        }
+        if (a.back_only) {
+            // a back substitution comes to the last block first and needs no G
+            const int b = nb - 1 - i;
+            if (prep == 0 && b >= 0) prep_task<T>(a, sy, b, S.prep);
+            else if (prep == 1 && b >= 0) preph_task<T>(a, sy, b, S.prep);
+            else if (prep < 0) backward_task<T, R>(a, sy, ep64, c, nb - 1 - s, S);
+        } else if (prep >= 0) {
+            if (i < nb) {
+                if (prep == 0) prep_task<T>(a, sy, i, S.prep);
+                else if (prep == 1) prep2_task<T>(a, sy, i, S.prep);
+                else preph_task<T>(a, sy, i, S.prep);
+            }
+        } else if (s < nb) {
+            forward_task<T, R>(a, sy, ep64, c, s, S);
+        } else {
+            backward_task<T, R>(a, sy, ep64, c, 2 * nb - 1 - s, S);
         }
         __syncthreads();
     }
@@ -583,10 +616,11 @@ int launch_solve(const void *L, long long n, long long ld, void *B, long long ld
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return CHM_ERR_CUDA;
     static int occ[64] = {0};
+    const int smem = (int)sizeof(SolveSmem<T, R>);
     if (!occ[dev]) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, solve_kernel<T, R>, kSolveThreads, 0) !=
-                cudaSuccess ||
+        if (cudaFuncSetAttribute(solve_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, solve_kernel<T, R>, kThreads, smem) != cudaSuccess ||
             b < 1)
             return CHM_ERR_CUDA;
         occ[dev] = b;
@@ -607,6 +641,9 @@ int launch_solve(const void *L, long long n, long long ld, void *B, long long ld
     a.back_only = Y != nullptr;
     a.inv = reinterpret_cast<double *>(sc.data);
     a.uflag = sc.iflags;
+    a.gflag = a.uflag + nb;
+    a.g2flag = a.gflag + nb;
+    a.hflag = a.g2flag + nb;
     a.ytag = sc.progress;
     a.xtag = sc.progress + (size_t)a.chains * nb * kW * R * 2;
     a.ctl = sc.ctl;
@@ -619,9 +656,8 @@ int launch_solve(const void *L, long long n, long long ld, void *B, long long ld
     a.ws_progress = sc.progress;
     a.ws_progress_n = sc.progress_cap;
     a.chk_cut = check_cut();
-    const long long tasks = nb + (long long)a.chains * (a.back_only ? nb : 2 * nb);
-    const int grid = (int)std::min<long long>(tasks, (long long)sm_count(dev) * occ[dev]);
-    solve_kernel<T, R><<<grid, kSolveThreads, 0, stream>>>(a);
+    const int grid = (int)std::min<long long>(solve_tasks(nb, a.chains, a.back_only), (long long)sm_count(dev) * occ[dev]);
+    solve_kernel<T, R><<<grid, kThreads, smem, stream>>>(a);
     return cudaGetLastError() == cudaSuccess ? CHM_OK : CHM_ERR_CUDA;
 }
 
@@ -652,7 +688,7 @@ ScratchNeed solve_need(long long n, long long nrhs)
     const size_t nr = (size_t)std::min<long long>(std::max(1ll, nrhs), solve_group(n));
     const size_t R = (size_t)solve_rhs((int)nr), cols = (nr + R - 1) / R * R;
     ScratchNeed need;
-    need.iflags = (nb + 63) & ~(size_t)63;
+    need.iflags = (4 * nb + 63) & ~(size_t)63;
     need.progress = 2 * nb * kW * cols * 2;
     need.data = nb * kPrepMats * kW * kW * sizeof(double);
     return need;

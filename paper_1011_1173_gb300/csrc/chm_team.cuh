@@ -42,16 +42,13 @@
 // each.
 #pragma once
 
-#include "chm_device.cuh"
-#include "chm_pass.cuh"
+#include "chm_sub.cuh"
 #include "chm_team_layout.h"
 
 namespace chm {
 namespace team {
 
-constexpr int kThreads = 128;
-constexpr int kWarps = 4;
-constexpr int kPer = kW / kWarps;  // rows of a split 32 x 32 product per warp
+using namespace chm::sub;
 
 template <typename T>
 struct Launch {
@@ -104,13 +101,6 @@ struct Stage {
     int passes;   // tasks of the passes before
 };
 
-struct PrepSmem {
-    double D[kW][kW + 1];
-    double U[kW][kW + 1];
-    double F[kW][kW + 1];
-    double M[kW / 2][kW / 2 + 1];
-    double rd[kW];
-};
 template <typename T>
 struct SubSmem {
     T tile[kWarps][2][kW * pass::Stride<T>::value];
@@ -149,7 +139,6 @@ union TaskSmem {
     __device__ TaskSmem() {}
 };
 
-constexpr unsigned kFull = 0xffffffffu;
 
 // Stamp `pt` of column block b of vector c (diagnostics): 0 SUB taken, 1 its
 // tiles summed, 2 what is left multiplied by U, 3 the previous step seen, 4
@@ -160,33 +149,6 @@ constexpr unsigned kFull = 0xffffffffu;
         if (P.trace && threadIdx.x == 0)                                                                         \
             P.trace[((size_t)(v.pass * kTeamKb + (c)) * v.nb + (b)) * kTracePoints + (pt)] = global_ns();        \
     } while (0)
-
-// Stage the 32 x 32 tile at row r0, column c0 into dst[column][Stride], read
-// through L2 (an earlier pass of the launch may have written it on another
-// SM): 16-byte asynchronous copies if `vec`, else loads of one element,
-// eight in flight per lane (a 4-byte cp.async would go through L1).  `diag`:
-// the diagonal tile, rows <= column only; the rest is zero.
-template <typename T>
-__device__ __forceinline__ void stage_tile(const SyncArgs &sy, T *dst, const T *L, long long ld, long long r0,
-                                           long long c0, long long n, bool vec, bool diag, int lane)
-{
-    constexpr int SD = pass::Stride<T>::value;
-    if (vec) {
-        pass::stage_tile(sy, dst, L, ld, r0, c0, n, kW, true, lane);
-        return;
-    }
-#pragma unroll 1
-    for (int c = 0; c < kW; c += 8) {
-        T x[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const long long o = (r0 + lane) + (c0 + c + i) * ld;
-            x[i] = (c0 + c + i < n && (!diag || lane <= c + i) && CHK_TRI(sy, o, n, ld)) ? __ldcg(L + o) : T(0);
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) dst[(c + i) * SD + lane] = x[i];
-    }
-}
 
 // ---------------------------------------------------------------- PREP
 
@@ -202,24 +164,6 @@ __device__ __forceinline__ bool wait_column(const View<T> &v, int b)
     return ok;
 }
 
-// out[j kW + i] = G[i][j] = sum_{m<=i} U[m][i] F[j][m]; rows i = warp,
-// warp + 4, ... (so that the four warps' triangles weigh the same: 144
-// FMAs each, with U's zeros in the rows' last groups of four), lane = j.
-__device__ __forceinline__ void form_g(const PrepSmem &S, double *out)
-{
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double acc[kPer];
-#pragma unroll
-    for (int ii = 0; ii < kPer; ++ii) acc[ii] = 0.0;
-#pragma unroll
-    for (int m = 0; m < kW; ++m) {
-        const double f = S.F[lane][m];
-#pragma unroll
-        for (int ii = m / kWarps; ii < kPer; ++ii) acc[ii] = fma(S.U[m][ii * kWarps + warp], f, acc[ii]);
-    }
-#pragma unroll
-    for (int ii = 0; ii < kPer; ++ii) __stcg(out + (size_t)lane * kW + ii * kWarps + warp, acc[ii]);
-}
 // The tile `up` blocks above diagonal block b: F[j][m] = L[(b - up) kW + j, b kW + m].
 template <typename T>
 __device__ __forceinline__ void load_above(const View<T> &v, int b, int up, PrepSmem &S)
@@ -233,20 +177,7 @@ __device__ __forceinline__ void load_above(const View<T> &v, int b, int up, Prep
         S.F[i][j] = (j < nc && CHK_TRI(v.sync, o, v.n, v.ld)) ? (double)__ldcg(v.L + o) : 0.0;
     }
 }
-// Every store of the block's threads so far, then the flag.
-__device__ __forceinline__ void publish(int *flag, int epoch)
-{
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) st_release_gpu(flag, epoch);
-}
-
-// U_b and G1_b.  The inverse is built up from 8 x 8 diagonal blocks: with
-// D = [[D1, B], [0, D2]], U = [[U1, -U1 B U2], [0, U2]].  The four 8 x 8
-// inverses take one warp (a column per lane, 36 dependent FP64 instructions),
-// the products of the two levels above all four warps: 116 instructions in
-// a row instead of the 560 of a column-per-lane substitution (3.6 against
-// 17 us at one FP64 instruction per 64 cycles and warp).
+// U_b and G1_b.
 template <typename T>
 __device__ void prep_task(const Launch<T> &P, const View<T> &v, int b, PrepSmem &S)
 {
@@ -272,67 +203,15 @@ __device__ void prep_task(const Launch<T> &P, const View<T> &v, int b, PrepSmem 
     }
     if (b >= 1) load_above(v, b, 1, S);
     __syncthreads();
+    double d = S.D[lane][lane];
     if (warp == 0) {
-        double d = S.D[lane][lane];
         const bool bad = lane < nc && !(d > 0.0 && d <= DBL_MAX);
         const unsigned badm = __ballot_sync(kFull, bad);
         if (badm && lane == 0) record_error(sy, kStatusNotPD, c0 + (__ffs(badm) - 1));
         if (bad) d = 1.0;
         if (v.pass == 0 && lane < nc) __stcg(v.dcar + c0 + lane, d);
-        S.rd[lane] = rcp_refined(d);
-        __syncwarp();
-        const int h = lane & 24, col = lane & 7;
-        double u[8];
-#pragma unroll
-        for (int i = 7; i >= 0; --i) {
-            double s = (i == col) ? 1.0 : 0.0;
-#pragma unroll
-            for (int m = i + 1; m < 8; ++m) s = fma(-S.D[h + i][h + m], u[m], s);
-            u[i] = s * S.rd[h + i];
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) S.U[h + i][h + col] = u[i];
     }
-    __syncthreads();
-    {
-        // 8 to 16: thread = (half, row, column)
-        const int h = (tid >> 6) * 16, i = (tid >> 3) & 7, j = tid & 7;
-        double s = 0.0;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) s = fma(S.D[h + i][h + 8 + m], S.U[h + 8 + m][h + 8 + j], s);
-        S.M[(tid >> 6) * 8 + i][j] = s;
-        __syncthreads();
-        s = 0.0;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) s = fma(S.U[h + i][h + m], S.M[(tid >> 6) * 8 + m][j], s);
-        S.U[h + i][h + 8 + j] = -s;
-        __syncthreads();
-    }
-    {
-        // 16 to 32: two rows a thread
-        constexpr int kH = kW / 2;
-        const int i = tid / kH, j = tid & (kH - 1);
-        double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-        for (int m = 0; m < kH; ++m) {
-            const double u = S.U[kH + m][kH + j];
-            s0 = fma(S.D[i][kH + m], u, s0);
-            s1 = fma(S.D[i + 8][kH + m], u, s1);
-        }
-        S.M[i][j] = s0;
-        S.M[i + 8][j] = s1;
-        __syncthreads();
-        s0 = s1 = 0.0;
-#pragma unroll
-        for (int m = 0; m < kH; ++m) {
-            const double x = S.M[m][j];
-            s0 = fma(S.U[i][m], x, s0);
-            s1 = fma(S.U[i + 8][m], x, s1);
-        }
-        S.U[i][kH + j] = -s0;
-        S.U[i + 8][kH + j] = -s1;
-        __syncthreads();
-    }
+    invert_block(S, d);
     double *ug = v.ug + (size_t)b * 3 * kW * kW;
 #pragma unroll
     for (int x = 0; x < kW * kW / kThreads; ++x) {
@@ -413,63 +292,6 @@ __device__ __forceinline__ void put_y(double *y, int lane, double x, float)
     reinterpret_cast<float2 *>(y)[lane] = make_float2(hi, (float)(x - (double)hi));
 }
 
-// Warp-wide bounded wait for a tagged double per lane; zeros if it gave up,
-// so that the task reaches its barriers.  `far`: a step that is not the
-// chain's next.  Such a wait polls one word (the last one written) with
-// pauses of up to 128 ns and takes the values once it is there: dozens of
-// warps wait on the newest step, and a poll of all its words by each would
-// slow the L2 slices that the chain's own stores and loads go to.
-__device__ __forceinline__ double wait_p(const SyncArgs &sy, const long long *w2, const long long *probe,
-                                         long long ep64, long long who, bool far)
-{
-    double x = 0.0;
-    if (__all_sync(kFull, get_tagged(w2, ep64, &x))) return x;
-    const long long t0 = global_ns();
-    unsigned ns = 16;
-    for (unsigned it = 1;; ++it) {
-        bool look = true;
-        if (far) {
-            look = (ld_relaxed_gpu(probe) & ~0xffffffffll) == ep64;
-            look = __any_sync(kFull, look);
-            if (!look) {
-                __nanosleep(ns);
-                if (ns < 128) ns <<= 1;
-            }
-        }
-        if (look && __all_sync(kFull, get_tagged(w2, ep64, &x))) return x;
-        // (looked at by all lanes alike: a branch of lane 0 alone would leave
-        // the warp split, and every later shuffle would wait for the halves)
-        if ((it & 31u) == 0u) {
-            const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 28);
-            if (__any_sync(kFull, late || aborted(sy))) {
-                if ((threadIdx.x & 31) == 0 && late) record_error(sy, kStatusTimeout, who);
-                return 0.0;
-            }
-        }
-    }
-}
-// Warp-wide bounded wait for the flags f[first .. last] (last - first < 32 per
-// look, one a lane), the warp staying together.
-__device__ __forceinline__ void wait_flags(const SyncArgs &sy, const int *f, int first, int last, long long who)
-{
-    for (int r0 = first; r0 <= last; r0 += 32) {
-        const int r = min(r0 + ((int)threadIdx.x & 31), last);
-        const long long t0 = global_ns();
-        unsigned ns = 16;
-        for (unsigned it = 1; !__all_sync(kFull, ld_acquire_gpu(f + r) == sy.epoch); ++it) {
-            __nanosleep(ns);
-            if (ns < 256) ns <<= 1;
-            if ((it & 15u) == 0u) {
-                const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 26);
-                if (__any_sync(kFull, late || aborted(sy))) {
-                    if ((threadIdx.x & 31) == 0 && late) record_error(sy, kStatusTimeout, who);
-                    return;
-                }
-            }
-        }
-    }
-}
-
 template <typename T>
 __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, SubSmem<T> &S)
 {
@@ -491,27 +313,36 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
     // tiles p <= b - 3 of column block b, dealt round-robin to the warps (the
     // dealing and the order of the sums depend on the order of the factor
     // alone), one staged ahead
-    const int far = b - 3;  // tiles 0 .. far - 1; tile b - 3 is split over the warps below
-    // this warp's rows of U_b, of tile b - 3 and columns of G1_b and G2_b, taken
-    // before the tiles so that nothing but the chain's own values is waited
-    // for behind p_{b-3}
+    const int far = b - 4;  // tiles 0 .. far - 1; tiles b - 4 and b - 3 are split over the warps below
+    // this warp's columns of G1_b and G2_b, taken before the tiles so that
+    // nothing but the chain's own values is waited for behind p_{b-4}
     const double *ug = v.ug + (size_t)b * 3 * kW * kW + warp * kPer * kW + lane;
-    const bool ok = __all_sync(kFull, wait_eq(sy, v.uflag + b, sy.epoch, b) &&
-                                          (b < 1 || wait_eq(sy, v.gflag + b, sy.epoch, b)) &&
-                                          (b < 2 || wait_eq(sy, v.g2flag + b, sy.epoch, b)));
-    const long long o3 = (long long)(b - 3) * kW + warp * kPer + (c0 + (active ? lane : 0)) * ld;
-    double u[kPer], g1[kPer], g2[kPer], t3[kPer];
+    wait_flags(sy, v.uflag, b, b, b);
+    if (b >= 1) wait_flags(sy, v.gflag, b, b, b);
+    if (b >= 2) wait_flags(sy, v.g2flag, b, b, b);
+    double g1[kPer], g2[kPer];
 #pragma unroll
     for (int jj = 0; jj < kPer; ++jj) {
-        u[jj] = ok ? __ldcg(ug + jj * kW) : 0.0;
-        g1[jj] = (ok && b >= 1) ? __ldcg(ug + kW * kW + jj * kW) : 0.0;
-        g2[jj] = (ok && b >= 2) ? __ldcg(ug + 2 * kW * kW + jj * kW) : 0.0;
-        t3[jj] = (b >= 3 && active && CHK_TRI(sy, o3 + jj, n, ld)) ? (double)__ldcg(v.L + o3 + jj) : 0.0;
+        g1[jj] = b >= 1 ? __ldcg(ug + kW * kW + jj * kW) : 0.0;
+        g2[jj] = b >= 2 ? __ldcg(ug + 2 * kW * kW + jj * kW) : 0.0;
     }
+    // (lane = column) a tile's column segment to L2: the tiles three steps on,
+    // and the two read element by element behind the loop
+    auto prefetch = [&](int p) {
+        const long long o = (long long)p * kW + (c0 + lane) * ld;
+        if (p >= 0 && p < b && active && CHK_TRI(sy, o, n, ld) && CHK_TRI(sy, o + kW - 1, n, ld)) {
+            pass::prefetch_l2n(v.L + o);
+            if (sizeof(T) * kW > 128) pass::prefetch_l2n(v.L + o + kW / 2);
+        }
+    };
     auto stage = [&](int p, int slot) {
-        if (p < far) stage_tile(sy, S.tile[warp][slot], v.L, ld, (long long)p * kW, c0, n, v.vec, false, lane);
+        if (p < far) {
+            stage_tile(sy, S.tile[warp][slot], v.L, ld, (long long)p * kW, c0, n, v.vec, false, lane);
+            prefetch(p + 2 * kWarps);
+        }
         pass::cp_commit();
     };
+    if (warp < 2) prefetch(b - 3 - warp);
     stage(warp, 0);
     T s = T(0), e = T(0);
     int slot = 0;
@@ -521,7 +352,8 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
         for (; p < end; p += kWarps) {
             stage(p + kWarps, slot ^ 1);
             const long long *w = ptag + (size_t)p * kW * 2;
-            const double y = wait_p(sy, w + 2 * lane, w + 2 * kW - 1, ep64, b, true);
+            // (a warp's last tile is waited for as closely as the chain's next steps)
+            const double y = wait_p(sy, w + 2 * lane, p + kWarps < far ? w + 2 * kW - 1 : nullptr, ep64, b);
             put_y(S.y[warp], lane, y, T(0));
             pass::cp_wait<1>();
             __syncwarp();
@@ -547,12 +379,38 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
     TEAM_TRACE(c, b, 1);
     // the steps before: a lane takes the tagged value of one of its warp's eight rows
     auto tag_of = [&](int up) { return ptag + ((size_t)(b - up) * kW + warp * kPer + (lane & (kPer - 1))) * 2; };
-    double acc = (double)s + (double)e;
-    if (b >= 3) {
-        const double y = wait_p(sy, tag_of(3), nullptr, ep64, b, false);
+    // this warp's rows of tiles b - 4 and b - 3, and of U_b
+    const long long o4 = (long long)(b - 4) * kW + warp * kPer + (c0 + (active ? lane : 0)) * ld;
+    double t4[kPer], t3[kPer], u[kPer];
 #pragma unroll
-        for (int jj = 0; jj < kPer; ++jj) acc = fma(t3[jj], __shfl_sync(kFull, y, jj), acc);
+    for (int jj = 0; jj < kPer; ++jj) {
+        t4[jj] = (b >= 4 && active && CHK_TRI(sy, o4 + jj, n, ld)) ? (double)__ldcg(v.L + o4 + jj) : 0.0;
+        t3[jj] = (b >= 3 && active && CHK_TRI(sy, o4 + kW + jj, n, ld)) ? (double)__ldcg(v.L + o4 + kW + jj) : 0.0;
     }
+    double acc = (double)s + (double)e, acc3 = 0.0;
+    if (b >= 4) {
+        const double y = wait_p(sy, tag_of(4), nullptr, ep64, b);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj) acc = fma(t4[jj], __shfl_sync(kFull, y, jj), acc);
+    }
+#pragma unroll
+    for (int jj = 0; jj < kPer; ++jj) u[jj] = __ldcg(ug + jj * kW);
+    if (b > 1 && (b - 1) % v.seg == 0) {
+        // a segment starts at row block b - 3: what is left there
+        S.part[1][warp][lane] = acc;
+        __syncthreads();
+        if (warp == kWarps - 1) {
+            const double z = S.z[lane] - ((S.part[1][0][lane] + S.part[1][1][lane]) + (S.part[1][2][lane] + S.part[1][3][lane]));
+            __stcg(v.snap + ((size_t)((b - 1) / v.seg - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)z);
+            __threadfence();
+        }
+    }
+    if (b >= 3) {
+        const double y = wait_p(sy, tag_of(3), nullptr, ep64, b);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj) acc3 = fma(t3[jj], __shfl_sync(kFull, y, jj), acc3);
+    }
+    acc += acc3;
     S.part[0][warp][lane] = acc;
     // (a first look at p_{b-2}, before the barrier hides its latency)
     double y2 = 0.0, y1 = 0.0;
@@ -572,12 +430,12 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
         __threadfence();
     }
     if (b >= 2) {
-        if (!__all_sync(kFull, have2)) y2 = wait_p(sy, tag_of(2), nullptr, ep64, b, false);
+        if (!__all_sync(kFull, have2)) y2 = wait_p(sy, tag_of(2), nullptr, ep64, b);
 #pragma unroll
         for (int jj = 0; jj < kPer; ++jj) pz = fma(-g2[jj], __shfl_sync(kFull, y2, jj), pz);
     }
     if (b >= 1) {
-        if (!__all_sync(kFull, have1)) y1 = wait_p(sy, tag_of(1), nullptr, ep64, b, false);
+        if (!__all_sync(kFull, have1)) y1 = wait_p(sy, tag_of(1), nullptr, ep64, b);
         TEAM_TRACE(c, b, 3);
 #pragma unroll
         for (int jj = 0; jj < kPer; ++jj) pz = fma(-g1[jj], __shfl_sync(kFull, y1, jj), pz);
@@ -799,21 +657,26 @@ __device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task
                 if (w < (lane & (E - 1)) && CHK_TRI(sy, o + w, n, ld)) dch[w] = __ldcg(v.L + o + w);
         }
     }
+    // 16-byte chunk `ch` of the columns cc0, cc0 + cstep, ... is this lane's to copy
+    constexpr int cstep = NV * 32 / CPC;
+    const int ch = lane % CPC, cc0 = part * (32 / CPC) + lane / CPC;
+    const int ncol = (int)min((long long)kW, n - c0);
+    const T *const lcol = v.L + ch * E + (c0 + cc0) * ld;
     auto stage = [&](int t) {  // tile and coefficients of row block rb + t
         const int r = rb + t, slot = t % NS;
         const long long r0 = (long long)r * kW;
         T *tl = U.tile[slot];
         if (v.vec) {
-            // (of the diagonal tile the chunks above the diagonal's)
-            const int below = r == j ? 0 : kW;
-#pragma unroll 4
-            for (int x = part * 32 + lane; x < kW * CPC; x += NV * 32) {
-                const int cc = x / CPC, ch = x % CPC;
-                const long long o = r0 + ch * E + (c0 + cc) * ld;
-                T *d = tl + cc * SD + ch * E;
-                if (ch * E + E > cc + below) continue;
-                if (c0 + cc < n && CHK_TRI(sy, o, n, ld) && CHK_TRI(sy, o + E - 1, n, ld)) {
-                    pass::cp16(d, v.L + o);
+            // this lane's chunk of every cstep-th column (of the diagonal tile
+            // the chunks above the diagonal's)
+            const int first = r == j ? (ch + 1) * E : 0;
+            const T *src = lcol + r0;
+            T *d = tl + cc0 * SD + ch * E;
+#pragma unroll
+            for (int cc = cc0; cc < kW; cc += cstep, src += cstep * ld, d += cstep * SD) {
+                if (cc < first) continue;
+                if (cc < ncol && CHK_TRI(sy, src - v.L, n, ld) && CHK_TRI(sy, src - v.L + E - 1, n, ld)) {
+                    pass::cp16(d, src);
                 } else {
 #pragma unroll
                     for (int w = 0; w < E; ++w) d[w] = T(0);
@@ -916,16 +779,16 @@ __device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task
                 const long long r0 = (long long)r * kW;
                 if (diag && active) __stcg(v.dcar + c0 + lane, dc * df);
                 __syncwarp();
-                const int ch = lane % CPC, cc0 = lane / CPC, cstep = 32 / CPC;
                 if (v.vec) {
-                    const int below = diag ? 0 : kW;
+                    const int first = diag ? ch * E + E - 1 : 0;
+                    constexpr int step = 32 / CPC;
+                    const int k0 = lane / CPC;
+                    T *g = v.L + r0 + ch * E + (c0 + k0) * ld;
+                    const T *d = tl + k0 * SD + ch * E;
 #pragma unroll
-                    for (int k = 0; k < CPC; ++k) {
-                        const int cc = cc0 + k * cstep;
-                        const long long o = r0 + ch * E + (c0 + cc) * ld;
-                        if (c0 + cc < n && ch * E + E - 1 <= cc + below && CHK_TRI(sy, o, n, ld) && CHK_TRI(sy, o + E - 1, n, ld))
-                            __stcg(reinterpret_cast<V16 *>(v.L + o), *reinterpret_cast<const V16 *>(tl + cc * SD + ch * E));
-                    }
+                    for (int cc = k0; cc < kW; cc += step, g += step * ld, d += step * SD)
+                        if (cc >= first && cc < ncol && CHK_TRI(sy, g - v.L, n, ld) && CHK_TRI(sy, g - v.L + E - 1, n, ld))
+                            __stcg(reinterpret_cast<V16 *>(g), *reinterpret_cast<const V16 *>(d));
                     const int i0 = lane & ~(E - 1);
                     if (diag && active && i0 + E - 1 > lane) {
 #pragma unroll
