@@ -32,9 +32,10 @@
 // step of four right-hand sides takes three times a step of one.  C chains
 // side by side fill the SMs that one chain leaves idle; the tiles they share
 // meet in L2, and U, G and H are formed once instead of once per four
-// right-hand sides.  n = 5000, float64, 16 right-hand sides: 1.13 ms in 16
-// chains against 6.96 ms as four launches of four right-hand sides each; the
-// FP64 rate allows 0.76 ms (400 M FMAs).
+// right-hand sides.  n = 5000, float64: 16 right-hand sides 0.91 ms in 16
+// chains against 6.96 ms as four launches of four right-hand sides each (the
+// FP64 rate allows 0.76 ms: 400 M FMAs), one right-hand side 0.41 against
+// 0.53 ms, bound by the chain: 314 steps of 1.3 us.
 #include <float.h>
 
 #include <algorithm>

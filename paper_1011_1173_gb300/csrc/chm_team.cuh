@@ -28,12 +28,14 @@
 // its own; the next pass of a factor enters column b once b's sweep is done.
 //
 // What bounds it.  A vector's substitution is the serial chain: nb steps of
-// about 1.7 us (a flag through L2, 8 FMAs at one FP64 instruction per 64
-// cycles and warp, a barrier, a four-way sum).  Vectors do not wait for each
-// other, and nothing else is on the chain: the sweep trails it by one
-// segment, whatever the number of vectors.  With many vectors or factors the
-// FP64 rate binds (three FMAs per element and vector: one in the
-// substitution, two in the sweep).
+// 1.3 us (a value through L2, 8 FMAs at one FP64 instruction per 64 cycles
+// and warp, a barrier, a four-way sum; up to 2 us where sweeps share the FP64
+// pipes).  Vectors do not wait for each other, and nothing else is on the
+// chain: the sweep trails it by one segment, whatever the number of vectors.
+// With many vectors or factors the FP64 rate binds (three FMAs per element
+// and vector: one in the substitution, two in the sweep).  n = 5000 in double,
+// one call: k = 1 0.37 ms (the wave kernel 1.08), k = 16 1.68 ms (1.97), of
+// which the FMAs are 0.05 and 1.1 ms.
 //
 // Precision: CHM_F64 is double throughout.  CHM_F32_MIXED substitutes in
 // double (P, U, G) with the far sums in pairs of floats (48 bits), forms the
@@ -103,10 +105,11 @@ struct Stage {
 
 template <typename T>
 struct SubSmem {
-    T tile[kWarps][2][kW * pass::Stride<T>::value];
-    double y[kWarps][kW];   // the p a warp works with (double), or its float pairs
-    double part[2][kWarps][kW];
-    double z[kW];           // what is left of v
+    T tile[2][kWarps][kW * pass::Stride<T>::value];  // two groups of four tiles, [column][row]
+    double part[2][kWarps][kW];        // the warps' sums at segment starts, in turn
+    double fin[2][kWarps][kW];         // and behind the tiles, and of the step's products
+    double y[kWarps][kW];              // a group's values of p, or their float pairs
+    double z[kW];                      // the entries of v
 };
 struct CoefSmem {
     static constexpr int ne = kTeamKb * (kTeamKb + 1) / 2;
@@ -247,55 +250,52 @@ __device__ void prep2_task(const View<T> &v, int b, PrepSmem &S)
 
 // ---------------------------------------------------------------- SUB
 
-// Sum over a staged tile's rows of F_{row, column} y_row, column = lane.
-// float: y comes as pairs (hi + lo = y to 48 bits) and the sum is kept as
-// s + c: products split exactly, the running sum compensated (two-sum), so
-// that the far sums lose about 2^-46 relative to their terms at FP32 speed
-// instead of a conversion and an FMA at the FP64 rate.
-__device__ __forceinline__ void tile_dot(const double *tl, const double *y, double &s, double &)
+// s + e += F_{row, column} y over the eight rows of a tile a warp holds,
+// column = lane.  float: y comes as pairs (hi + lo = y to 48 bits) and the
+// sum is kept as s + e: products split exactly, the running sum compensated
+// (two-sum), so that the far sums lose about 2^-46 relative to their terms at
+// FP32 speed instead of a conversion and an FMA at the FP64 rate.
+__device__ __forceinline__ void rows_dot(const double (&f)[kPer], const double *y, double &s, double &)
 {
 #pragma unroll
-    for (int j = 0; j < kW; j += 2) {
-        const double2 t = *reinterpret_cast<const double2 *>(tl + j);
+    for (int j = 0; j < kPer; j += 2) {
         const double2 u = *reinterpret_cast<const double2 *>(y + j);
-        s = fma(t.x, u.x, s);
-        s = fma(t.y, u.y, s);
+        s = fma(f[j], u.x, s);
+        s = fma(f[j + 1], u.y, s);
     }
 }
-__device__ __forceinline__ void pair_fma(float f, float2 u, float &s, float &c)
+__device__ __forceinline__ void pair_fma(float f, float hi, float lo, float &s, float &e)
 {
-    const float p = __fmul_rn(f, u.x);
-    const float e = fmaf(f, u.x, -p);
-    const float t = __fadd_rn(s, p);
-    const float b = __fsub_rn(t, s);
-    const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b));
-    s = t;
-    c = __fadd_rn(c, __fadd_rn(fmaf(f, u.y, e), r));
+    const float p = __fmul_rn(f, hi);
+    const float d = fmaf(f, hi, -p);
+    const float u = __fadd_rn(s, p);
+    const float b = __fsub_rn(u, s);
+    const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(u, b)), __fsub_rn(p, b));
+    s = u;
+    e = __fadd_rn(e, __fadd_rn(fmaf(f, lo, d), r));
 }
-__device__ __forceinline__ void tile_dot(const float *tl, const double *y, float &s, float &c)
+__device__ __forceinline__ void rows_dot(const float (&f)[kPer], const double *y, float &s, float &e)
 {
-    const float4 *yp = reinterpret_cast<const float4 *>(y);  // (hi, lo) of two rows
 #pragma unroll
-    for (int j = 0; j < kW; j += 4) {
-        const float4 t = *reinterpret_cast<const float4 *>(tl + j);
-        const float4 a = yp[j / 2], b = yp[j / 2 + 1];
-        pair_fma(t.x, make_float2(a.x, a.y), s, c);
-        pair_fma(t.y, make_float2(a.z, a.w), s, c);
-        pair_fma(t.z, make_float2(b.x, b.y), s, c);
-        pair_fma(t.w, make_float2(b.z, b.w), s, c);
+    for (int j = 0; j < kPer; j += 2) {
+        const float4 u = *reinterpret_cast<const float4 *>(y + j);  // (hi, lo) of two rows
+        pair_fma(f[j], u.x, u.y, s, e);
+        pair_fma(f[j + 1], u.z, u.w, s, e);
     }
 }
-__device__ __forceinline__ void put_y(double *y, int lane, double x, double) { y[lane] = x; }
-__device__ __forceinline__ void put_y(double *y, int lane, double x, float)
+__device__ __forceinline__ void put_y(double *y, double x, double) { *y = x; }
+__device__ __forceinline__ void put_y(double *y, double x, float)
 {
     const float hi = (float)x;
-    reinterpret_cast<float2 *>(y)[lane] = make_float2(hi, (float)(x - (double)hi));
+    *reinterpret_cast<float2 *>(y) = make_float2(hi, (float)(x - (double)hi));
 }
 
 template <typename T>
 __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, SubSmem<T> &S)
 {
     constexpr int SD = pass::Stride<T>::value;
+    constexpr int E = 16 / (int)sizeof(T);  // elements of a 16-byte chunk
+    using V16 = typename pass::Vec16<T>::type;
     const SyncArgs &sy = v.sync;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long n = v.n, ld = v.ld;
@@ -307,13 +307,18 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
     TEAM_TRACE(c, b, 0);
     (void)wait_column(v, b);
     if (warp == 0) {
+        // (read by other warps behind the first barrier)
         const long long o = c0 + lane + c * v.ldv;
         S.z[lane] = (active && CHK_RECT(sy, o, n, v.kb, v.ldv)) ? (double)v.V[o] : 0.0;
     }
-    // tiles p <= b - 3 of column block b, dealt round-robin to the warps (the
-    // dealing and the order of the sums depend on the order of the factor
-    // alone), one staged ahead
-    const int far = b - 4;  // tiles 0 .. far - 1; tiles b - 4 and b - 3 are split over the warps below
+    // The tiles p <= b - 3 of column block b, in groups of four (the first of
+    // two, so that segments start between groups).  A warp takes eight rows
+    // of every tile, so that the newest step costs it eight FMAs; the order
+    // of its sums depends on nothing but the order of the factor.  A group is
+    // staged one group ahead, a tile by each warp (whole columns: a warp that
+    // fetched its own rows of each would touch four times the lines), and
+    // its 32 values of p come in one look, a lane each.
+    const int far = b - 2;  // tiles 0 .. far - 1
     // this warp's columns of G1_b and G2_b, taken before the tiles so that
     // nothing but the chain's own values is waited for behind p_{b-4}
     const double *ug = v.ug + (size_t)b * 3 * kW * kW + warp * kPer * kW + lane;
@@ -326,97 +331,85 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
         g1[jj] = b >= 1 ? __ldcg(ug + kW * kW + jj * kW) : 0.0;
         g2[jj] = b >= 2 ? __ldcg(ug + 2 * kW * kW + jj * kW) : 0.0;
     }
-    // (lane = column) a tile's column segment to L2: the tiles three steps on,
-    // and the two read element by element behind the loop
-    auto prefetch = [&](int p) {
-        const long long o = (long long)p * kW + (c0 + lane) * ld;
-        if (p >= 0 && p < b && active && CHK_TRI(sy, o, n, ld) && CHK_TRI(sy, o + kW - 1, n, ld)) {
-            pass::prefetch_l2n(v.L + o);
-            if (sizeof(T) * kW > 128) pass::prefetch_l2n(v.L + o + kW / 2);
-        }
-    };
-    auto stage = [&](int p, int slot) {
-        if (p < far) {
-            stage_tile(sy, S.tile[warp][slot], v.L, ld, (long long)p * kW, c0, n, v.vec, false, lane);
-            prefetch(p + 2 * kWarps);
-        }
+    auto stage = [&](int i) {
+        const int p = 4 * i - 2 + warp;
+        if (p >= 0 && p < far) stage_tile(sy, S.tile[i & 1][warp], v.L, ld, (long long)p * kW, c0, n, v.vec, false, lane);
         pass::cp_commit();
     };
-    if (warp < 2) prefetch(b - 3 - warp);
-    stage(warp, 0);
+    // this lane's row of the four tiles' p it looks for
+    const long long *const mytag = ptag + ((size_t)(lane / kPer) * kW + warp * kPer + lane % kPer) * 2;
+    // What is left of v at a segment's start, for the sweep: one warp (another
+    // each time) adds the warps' sums behind the next group's barrier, while
+    // the others go on; two buffers in turn keep them from overwriting what
+    // it reads.
+    int start = 0;  // the segment whose start's sums are in S.part
+    stage(0);
     T s = T(0), e = T(0);
-    int slot = 0;
-    for (int q = 1, p = warp; seg_start(q - 1, v.seg) < far; ++q) {
-        const int start = seg_start(q, v.seg);
-        const int end = min(start, far);
-        for (; p < end; p += kWarps) {
-            stage(p + kWarps, slot ^ 1);
-            const long long *w = ptag + (size_t)p * kW * 2;
-            // (a warp's last tile is waited for as closely as the chain's next steps)
-            const double y = wait_p(sy, w + 2 * lane, p + kWarps < far ? w + 2 * kW - 1 : nullptr, ep64, b);
-            put_y(S.y[warp], lane, y, T(0));
-            pass::cp_wait<1>();
-            __syncwarp();
-            tile_dot(S.tile[warp][slot] + lane * SD, S.y[warp], s, e);
-            __syncwarp();
-            slot ^= 1;
+    for (int i = 0; 4 * i - 2 < far; ++i) {
+        pass::cp_wait<0>();
+        __syncthreads();  // group i is staged, group i - 1 is done with
+        stage(i + 1);
+        if (start > 0 && warp == (i & (kWarps - 1))) {
+            double(*part)[kW] = S.part[start & 1];
+            const double z = S.z[lane] - ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]));
+            __stcg(v.snap + ((size_t)(start - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)z);
+            __threadfence();  // before the step's result, which the sweep's inputs follow from
         }
-        if (start <= far) {
-            // what is left of v at the start of segment q, for the sweep
-            S.part[0][warp][lane] = (double)s + (double)e;
-            s = e = T(0);
-            __syncthreads();
-            if (warp == 0) {
-                const double z = S.z[lane] - ((S.part[0][0][lane] + S.part[0][1][lane]) + (S.part[0][2][lane] + S.part[0][3][lane]));
-                S.z[lane] = z;
-                __stcg(v.snap + ((size_t)(q - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)z);
-                __threadfence();  // before the step's result, which the sweep's inputs follow from
+        start = 0;
+        const int p0 = 4 * i - 2, t1 = min(4, far - p0);
+        const bool nearby = p0 + 8 >= far;  // the last tiles are waited for without a pause
+        int t = i == 0 ? 2 : 0;
+        double y = 0.0;
+        bool have = p0 + lane / kPer < 0 || lane / kPer >= t1;
+        long long t0 = 0;
+        for (unsigned it = 0;; ++it) {
+            if (!have) {
+                have = get_tagged(mytag + (long long)p0 * kW * 2, ep64, &y);
+                if (have) put_y(&S.y[warp][lane], y, T(0));
             }
-            __syncthreads();
+            const unsigned m = __ballot_sync(kFull, have);
+            __syncwarp();
+            for (; t < t1 && ((m >> (8 * t)) & 0xffu) == 0xffu; ++t) {
+                T f[kPer];
+                const V16 *rows = reinterpret_cast<const V16 *>(S.tile[i & 1][t] + lane * SD + warp * kPer);
+#pragma unroll
+                for (int ch = 0; ch < kPer / E; ++ch) {
+                    const V16 x = rows[ch];
+#pragma unroll
+                    for (int w = 0; w < E; ++w) f[ch * E + w] = pass::vget<T>(x, w);
+                }
+                rows_dot(f, S.y[warp] + t * kPer, s, e);
+            }
+            if (t >= t1) break;
+            if (!nearby) __nanosleep(100);
+            if (it == 0) t0 = global_ns();
+            if ((it & 31u) == 31u) {
+                const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 28);
+                if (__any_sync(kFull, late || aborted(sy))) {
+                    if (lane == 0 && late) record_error(sy, kStatusTimeout, b);
+                    break;  // (the launch is being aborted)
+                }
+            }
+        }
+        __syncwarp();
+        if (4 * (i + 1) % v.seg == 0 && 4 * i + 2 < far) {
+            start = 4 * (i + 1) / v.seg;
+            S.part[start & 1][warp][lane] = (double)s + (double)e;
         }
     }
     pass::cp_wait<0>();
     TEAM_TRACE(c, b, 1);
     // the steps before: a lane takes the tagged value of one of its warp's eight rows
     auto tag_of = [&](int up) { return ptag + ((size_t)(b - up) * kW + warp * kPer + (lane & (kPer - 1))) * 2; };
-    // this warp's rows of tiles b - 4 and b - 3, and of U_b
-    const long long o4 = (long long)(b - 4) * kW + warp * kPer + (c0 + (active ? lane : 0)) * ld;
-    double t4[kPer], t3[kPer], u[kPer];
-#pragma unroll
-    for (int jj = 0; jj < kPer; ++jj) {
-        t4[jj] = (b >= 4 && active && CHK_TRI(sy, o4 + jj, n, ld)) ? (double)__ldcg(v.L + o4 + jj) : 0.0;
-        t3[jj] = (b >= 3 && active && CHK_TRI(sy, o4 + kW + jj, n, ld)) ? (double)__ldcg(v.L + o4 + kW + jj) : 0.0;
-    }
-    double acc = (double)s + (double)e, acc3 = 0.0;
-    if (b >= 4) {
-        const double y = wait_p(sy, tag_of(4), nullptr, ep64, b);
-#pragma unroll
-        for (int jj = 0; jj < kPer; ++jj) acc = fma(t4[jj], __shfl_sync(kFull, y, jj), acc);
-    }
+    double u[kPer];
 #pragma unroll
     for (int jj = 0; jj < kPer; ++jj) u[jj] = __ldcg(ug + jj * kW);
-    if (b > 1 && (b - 1) % v.seg == 0) {
-        // a segment starts at row block b - 3: what is left there
-        S.part[1][warp][lane] = acc;
-        __syncthreads();
-        if (warp == kWarps - 1) {
-            const double z = S.z[lane] - ((S.part[1][0][lane] + S.part[1][1][lane]) + (S.part[1][2][lane] + S.part[1][3][lane]));
-            __stcg(v.snap + ((size_t)((b - 1) / v.seg - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)z);
-            __threadfence();
-        }
-    }
-    if (b >= 3) {
-        const double y = wait_p(sy, tag_of(3), nullptr, ep64, b);
-#pragma unroll
-        for (int jj = 0; jj < kPer; ++jj) acc3 = fma(t3[jj], __shfl_sync(kFull, y, jj), acc3);
-    }
-    acc += acc3;
-    S.part[0][warp][lane] = acc;
+    S.fin[0][warp][lane] = (double)s + (double)e;
     // (a first look at p_{b-2}, before the barrier hides its latency)
     double y2 = 0.0, y1 = 0.0;
     const bool have2 = b >= 2 && get_tagged(tag_of(2), ep64, &y2);
     __syncthreads();
-    const double rv = S.z[lane] - ((S.part[0][0][lane] + S.part[0][1][lane]) + (S.part[0][2][lane] + S.part[0][3][lane]));
+    const double rv = S.z[lane] - ((S.fin[0][0][lane] + S.fin[0][1][lane]) + (S.fin[0][2][lane] + S.fin[0][3][lane]));
     double pz = 0.0;
 #pragma unroll
     for (int jj = 0; jj < kPer; ++jj) pz = fma(u[jj], __shfl_sync(kFull, rv, warp * kPer + jj), pz);
@@ -440,10 +433,10 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
 #pragma unroll
         for (int jj = 0; jj < kPer; ++jj) pz = fma(-g1[jj], __shfl_sync(kFull, y1, jj), pz);
     }
-    S.part[1][warp][lane] = pz;
+    S.fin[1][warp][lane] = pz;
     __syncthreads();
     if (warp == 0 && !(c == 0 && b == P.skip_publish)) {
-        const double x = (S.part[1][0][lane] + S.part[1][1][lane]) + (S.part[1][2][lane] + S.part[1][3][lane]);
+        const double x = (S.fin[1][0][lane] + S.fin[1][1][lane]) + (S.fin[1][2][lane] + S.fin[1][3][lane]);
         put_tagged(ptag + ((size_t)b * kW + lane) * 2, active ? x : 0.0, ep64);
     }
     TEAM_TRACE(c, b, 4);
