@@ -75,7 +75,9 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 NCU_TRAFFIC = {("wave_kernel<double>", "4ab9131a4a9fb172", 5000, 16): 210.58e6,
                ("wave_kernel<float>", "4ab9131a4a9fb172", 8192, 16): 307.99e6,
                ("wave_kernel<double>", "1732a41a06476ee3", 5000, 16): 209.77e6}
-KERNEL_SOURCES = ("paper_1011_1173_gb300/csrc/chm_wave.cuh", "paper_1011_1173_gb300/csrc/chm_device.cuh",
+KERNEL_SOURCES = ("paper_1011_1173_gb300/csrc/chm_team.cuh", "paper_1011_1173_gb300/csrc/chm_team_layout.h",
+                  "paper_1011_1173_gb300/csrc/chm_sub.cuh",
+                  "paper_1011_1173_gb300/csrc/chm_wave.cuh", "paper_1011_1173_gb300/csrc/chm_device.cuh",
                   "paper_1011_1173_gb300/csrc/chm_layout.h", "paper_1011_1173_gb300/csrc/chm_modify.cu")
 
 
@@ -118,9 +120,18 @@ def measured_fp32_tflops():
     return _ALU["f32"]
 
 
+def team_kernel_takes(n, k, mixed):
+    """Whether path 1 runs the team kernel or the wave kernel (the rule of
+    use_team in csrc/chm_modify.cu); names the kernel in the output only."""
+    k = min(k, 64)
+    if mixed:
+        return n <= 8192
+    return n <= 6144 or (n <= 8192 and k <= 16) or (n <= 12288 and k <= 8) or (n <= 16384 and k <= 4)
+
+
 def launches_per_modification(path, k, dtype="f64"):
-    """Kernels of this library one modification launches: the wave kernel once
-    per 64 vectors; the pass kernels per pass of up to 16 vectors either two
+    """Kernels of this library one modification launches: the team or the wave
+    kernel once per 64 vectors; the pass kernels per pass of up to 16 vectors either two
     (a fused pass of up to 8: the inverse diagonal blocks, then the forward
     substitution whose workers also form the coefficients and sweep) or six
     (the inverse diagonal blocks, the forward substitution, the block Grams,
@@ -935,7 +946,7 @@ def main():
     if path == chm.PATH_PASS:
         kernel = "pass kernels<%s>" % ("float" if mixed else "double")
     else:
-        kernel = "wave_kernel<float>" if mixed else "wave_kernel<double>"
+        kernel = "%s_kernel<%s>" % ("team" if team_kernel_takes(n, k, mixed) else "wave", "float" if mixed else "double")
     hbm_gbs = alg_bytes(n, k, elt) / (launch_ms / 1e3) / 1e9
     peak_hbm, hbm_src = measured_hbm_gbs()
     if mixed:

@@ -344,7 +344,7 @@ int chm_solve(const void *L, int64_t n, int64_t ld, void *B, int64_t ldb, int64_
  * take chm_solve's two substitutions.  Otherwise the two calls follow each
  * other on the stream.  Precision: CHM_F64 in double; CHM_F32_MIXED as each part of
  * the pair: a carried right-hand side's forward half in float like the
- * pass's Apply, the back substitution with double arithmetic on float data.
+ * pass's Apply, the back substitution as chm_solve's.
  * d_info receives the modification's status; a failure of the solve part
  * (a diagonal entry not positive) goes to the stream's status word
  * (chm_status_sync).  k == 0 is chm_solve alone, nrhs == 0 chm_modify_ex
@@ -436,9 +436,10 @@ int chm_microbench(int which, double *out, int nout);
  * rotations, restated exactly) with different work splits:
  *   wave  one persistent launch per 64 vectors, on one of two kernels.  The
  *         team kernel (orders up to 8192; in double above 6144 only up to 16
- *         vectors) substitutes every vector through the factor as it enters
- *         a pass of up to 8 vectors, each vector a chain of its own, and
- *         sweeps each tile once per pass.  The wave kernel (the rest): each
+ *         vectors, but 8 of them up to order 12288 and 4 up to 16384)
+ *         substitutes every vector through the factor as it enters a pass of
+ *         up to 8 vectors, each vector a chain of its own, and sweeps each
+ *         tile once per pass.  The wave kernel (the rest): each
  *         vector is a wave that sweeps the factor, its forward-substitution
  *         chain driven by the sweep's carries.
  *   pass  per block of up to 16 vectors (Sec. 4.1's blocking): a forward
@@ -447,10 +448,12 @@ int chm_microbench(int which, double *out, int nout);
  *         in double), and one sweep that reads and writes each tile of the
  *         factor once for the whole block of vectors.
  * The automatic rule takes the pass kernels when the factor's upper
- * triangle is at least 32 MB (float) or 256 MB with k <= 8 (double), and
- * for a factor of order >= 64 in page-locked host memory modified by two or
- * more vectors (it then crosses the CPU-GPU link three times per pass of up
- * to 16 vectors; the wave kernel twice per vector).
+ * triangle is at least 32 MB in float (with 8 or more vectors above order
+ * 6500 only) or 256 MB in double (with one vector; two above order 12000, up
+ * to 8 above 16384), and for a factor of order >= 64 in page-locked host
+ * memory modified by two or more vectors (it then crosses the CPU-GPU link
+ * three times per pass of up to 16 vectors; the wave kernel twice per
+ * vector).
  * chm_config_get also answers "pass_d_f32", "pass_d_f64", "pass_kb_f32"
  * and "pass_kb_f64" (the values in effect, tuning cache aside) and
  * "checked" (1 in the bounds-checked build).  The bounds-checked

@@ -64,7 +64,7 @@ int relayout(Plan *p)
     p->tmpl.assign(act.size(), Prob());
     for (Prob &pr : p->tmpl) memset(&pr, 0, sizeof(pr));
     if (act.empty()) return CHM_OK;
-    team_carve(shapes.data(), (int)shapes.size(), p->sc, p->tmpl.data());
+    team_carve(shapes.data(), (int)shapes.size(), p->dtype, p->sc, p->tmpl.data());
     for (size_t q = 0; q < act.size(); ++q) {
         const int i = act[q];
         Prob &pr = p->tmpl[q];

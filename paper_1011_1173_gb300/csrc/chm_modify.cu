@@ -243,17 +243,19 @@ int check_reachable(const void *p)
 }
 
 // Path 1's two kernels.  The team kernel spends three FMAs per element and
-// vector where the wave kernel spends two, but does not sweep the factor
-// vector after vector: it is ahead until a large factor and many vectors in
-// double keep the wave kernel at the FP64 rate.  Measured, ms per modification
-// (team / wave), double: n = 512 k = 1 0.10 / 0.15, k = 16 0.27 / 0.38; n = 5000
-// k = 1 0.42 / 1.10, k = 16 1.70 / 1.98, k = 64 6.18 / 6.61; n = 8192 k = 16
-// 3.82 / 3.97, k = 64 14.5 / 13.8; float: n = 2000 k = 1 0.14 / 0.41, k = 16
-// 0.28 / 0.65; n = 8192 k = 64 5.5 / 8.6.
+// vector where the wave kernel spends two, and reads each tile once per
+// vector, but does not sweep the factor vector after vector: it is ahead
+// until the factor leaves L2, or many vectors in double keep the wave kernel
+// at the FP64 rate.  Measured, ms per modification (team / wave), double:
+// n = 512 k = 1 0.07 / 0.15, k = 16 0.29 / 0.38; n = 5000 k = 1 0.37 / 1.10,
+// k = 16 1.69 / 1.98, k = 64 6.2 / 6.6; n = 8192 k = 8 2.1 / 2.9, k = 16 3.9 /
+// 4.0, k = 64 14.5 / 13.8; n = 12000 k = 8 4.35 / 4.48; n = 16384 k = 4 4.3
+// (the pass kernels 4.8), k = 6 6.6 / 6.2, k = 8 7.7 / 7.4; float: n = 2000
+// k = 1 0.13 / 0.41, k = 16 0.27 / 0.65; n = 8192 k = 64 5.5 / 8.6.
 bool use_team(long long n, long long k, int dtype)
 {
-    if (n > 8192) return false;
-    return dtype != CHM_F64 || n <= 6144 || k <= 16;
+    if (dtype != CHM_F64) return n <= 8192;
+    return n <= 6144 || (n <= 8192 && k <= 16) || (n <= 12288 && k <= 8) || (n <= 16384 && k <= 4);
 }
 
 // The scratch of path 1 for one launch.
@@ -424,7 +426,7 @@ static int enqueue_single(void *L, long long n, long long ld, const void *V, lon
         Prob pr;
         memset(&pr, 0, sizeof(pr));
         const ProbShape sh{n, kw};
-        if (team) team_carve(&sh, 1, sc, &pr);
+        if (team) team_carve(&sh, 1, dtype, sc, &pr);
         else carve(&sh, 1, sc, &pr);
         pr.L = L;
         pr.V = static_cast<const char *>(V) + (size_t)q0 * ldv * elt;

@@ -178,7 +178,7 @@ int launch_slot(Server *s, Slot &sl)
     const int np = (int)sl.reqs.size();
     std::vector<Prob> probs(np);
     for (Prob &p : probs) memset(&p, 0, sizeof(p));
-    team_carve(shapes.data(), np, sl.sc, probs.data());
+    team_carve(shapes.data(), np, s->dtype, sl.sc, probs.data());
     long long ntasks = 0;
     for (int i = 0; i < np; ++i) {
         Request *r = sl.reqs[i];

@@ -24,7 +24,7 @@ ScratchNeed team_need(const ProbShape *shapes, int count)
     return r;
 }
 
-void team_carve(const ProbShape *shapes, int count, const Scratch &sc, Prob *problems)
+void team_carve(const ProbShape *shapes, int count, int dtype, const Scratch &sc, Prob *problems)
 {
     size_t fi = 0, fp = 0, fd = 0;
     for (int i = 0; i < count; ++i) {
@@ -32,7 +32,7 @@ void team_carve(const ProbShape *shapes, int count, const Scratch &sc, Prob *pro
         Prob &p = problems[i];
         p.nb = nb;
         p.k = k;
-        p.ntasks = team::prob_tasks(nb, k);
+        p.ntasks = team::prob_tasks(nb, k, dtype == CHM_F64);
         p.iflags = sc.iflags + fi;
         p.progress = sc.progress + fp;
         p.data = sc.data + fd;

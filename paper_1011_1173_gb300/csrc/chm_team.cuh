@@ -101,13 +101,15 @@ struct Stage {
     int t;        // stage
     int first;    // its first task
     int passes;   // tasks of the passes before
+    int segs;     // segments of column t - look (once that is a column)
+    int left;     // columns until there is one more
 };
 
 template <typename T>
 struct SubSmem {
     T tile[2][kWarps][kW * pass::Stride<T>::value];  // two groups of four tiles, [column][row]
-    double part[2][kWarps][kW];        // the warps' sums at segment starts, in turn
-    double fin[2][kWarps][kW];         // and behind the tiles, and of the step's products
+    double part[4][kWarps][kW];        // the warps' sums at segment starts, in turn
+    double fin[kWarps][kW];            // and behind the tiles
     double y[kWarps][kW];              // a group's values of p, or their float pairs
     double z[kW];                      // the entries of v
 };
@@ -136,6 +138,7 @@ union TaskSmem {
     SubSmem<T> sub;
     CoefSmem coef;
     SweepSmem<T, 1, 1> sweep1;
+    SweepSmem<T, 1, 2> sweep12;
     SweepSmem<T, 2, 2> sweep2;
     SweepSmem<T, 4, 4> sweep4;
     SweepSmem<T, 8, 4> sweep8;
@@ -161,7 +164,7 @@ template <typename T>
 __device__ __forceinline__ bool wait_column(const View<T> &v, int b)
 {
     if (v.pass == 0) return true;
-    const long long want = ((long long)v.sync.epoch << 32) + (long long)v.pass * segs_of(b, seg_of(v.nb, kTeamKb));
+    const long long want = ((long long)v.sync.epoch << 32) + (long long)v.pass * segs_of(b, seg_of(v.nb, kTeamKb, sizeof(T) == 8));
     const bool ok = __all_sync(kFull, wait_ge(v.sync, v.sdone + b, want, b));
     __syncwarp();
     return ok;
@@ -339,24 +342,30 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
     // this lane's row of the four tiles' p it looks for
     const long long *const mytag = ptag + ((size_t)(lane / kPer) * kW + warp * kPer + lane % kPer) * 2;
     // What is left of v at a segment's start, for the sweep: one warp (another
-    // each time) adds the warps' sums behind the next group's barrier, while
-    // the others go on; two buffers in turn keep them from overwriting what
-    // it reads.
-    int start = 0;  // the segment whose start's sums are in S.part
+    // each time) adds the warps' sums behind the next barrier, while the
+    // others go on; four buffers in turn (a group holds at most two starts)
+    // keep them from overwriting what it reads.
+    int mid = 0, end = 0;  // the segments whose starts' sums are in S.part: within and behind the last group
+    int next = 1, at = seg_start(1, v.seg);  // the next segment and where it starts
+    auto keep = [&](int sg) {
+        double(*part)[kW] = S.part[sg & 3];
+        const double z = S.z[lane] - ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]));
+        __stcg(v.snap + ((size_t)(sg - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)z);
+        __threadfence();  // before the step's result, which the sweep's inputs follow from
+    };
     stage(0);
-    T s = T(0), e = T(0);
+    T s = T(0), e = T(0), sm = T(0), em = T(0);  // the sums, and as they stood behind a group's second tile
     for (int i = 0; 4 * i - 2 < far; ++i) {
         pass::cp_wait<0>();
         __syncthreads();  // group i is staged, group i - 1 is done with
         stage(i + 1);
-        if (start > 0 && warp == (i & (kWarps - 1))) {
-            double(*part)[kW] = S.part[start & 1];
-            const double z = S.z[lane] - ((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]));
-            __stcg(v.snap + ((size_t)(start - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)z);
-            __threadfence();  // before the step's result, which the sweep's inputs follow from
-        }
-        start = 0;
+        if (mid > 0 && warp == (i & (kWarps - 1))) keep(mid);
+        if (end > 0 && warp == ((i + 2) & (kWarps - 1))) keep(end);
         const int p0 = 4 * i - 2, t1 = min(4, far - p0);
+        // segments that start at the group's third tile and behind it
+        mid = end = 0;
+        if (at == 4 * i && at < far) mid = next++, at += v.seg;
+        if (at == 4 * i + 2 && at < far) end = next++, at += v.seg;
         const bool nearby = p0 + 8 >= far;  // the last tiles are waited for without a pause
         int t = i == 0 ? 2 : 0;
         double y = 0.0;
@@ -379,6 +388,10 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
                     for (int w = 0; w < E; ++w) f[ch * E + w] = pass::vget<T>(x, w);
                 }
                 rows_dot(f, S.y[warp] + t * kPer, s, e);
+                if (t == 1) {
+                    sm = s;
+                    em = e;
+                }
             }
             if (t >= t1) break;
             if (!nearby) __nanosleep(100);
@@ -392,10 +405,8 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
             }
         }
         __syncwarp();
-        if (4 * (i + 1) % v.seg == 0 && 4 * i + 2 < far) {
-            start = 4 * (i + 1) / v.seg;
-            S.part[start & 1][warp][lane] = (double)s + (double)e;
-        }
+        if (mid > 0) S.part[mid & 3][warp][lane] = (double)sm + (double)em;
+        if (end > 0) S.part[end & 3][warp][lane] = (double)s + (double)e;
     }
     pass::cp_wait<0>();
     TEAM_TRACE(c, b, 1);
@@ -404,22 +415,24 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
     double u[kPer];
 #pragma unroll
     for (int jj = 0; jj < kPer; ++jj) u[jj] = __ldcg(ug + jj * kW);
-    S.fin[0][warp][lane] = (double)s + (double)e;
+    S.fin[warp][lane] = (double)s + (double)e;
     // (a first look at p_{b-2}, before the barrier hides its latency)
     double y2 = 0.0, y1 = 0.0;
     const bool have2 = b >= 2 && get_tagged(tag_of(2), ep64, &y2);
     __syncthreads();
-    const double rv = S.z[lane] - ((S.fin[0][0][lane] + S.fin[0][1][lane]) + (S.fin[0][2][lane] + S.fin[0][3][lane]));
+    const double rv = S.z[lane] - ((S.fin[0][lane] + S.fin[1][lane]) + (S.fin[2][lane] + S.fin[3][lane]));
     double pz = 0.0;
 #pragma unroll
     for (int jj = 0; jj < kPer; ++jj) pz = fma(u[jj], __shfl_sync(kFull, rv, warp * kPer + jj), pz);
     TEAM_TRACE(c, b, 2);
     // U^T (what is left) - G2 p_{b-2} - G1 p_{b-1}: this warp's share of each
     const bool have1 = b >= 1 && get_tagged(tag_of(1), ep64, &y1);
-    if (b > 0 && b % v.seg == 0 && warp == kWarps - 1) {
+    // (the fences pass while the warps would wait for p_{b-1})
+    if (mid > 0 && warp == 1) keep(mid);
+    if (end > 0 && warp == 2) keep(end);
+    if (at == b - 2 && warp == kWarps - 1) {
         // what is left at the start of the column's last segment, row block b - 2
-        // (the fence passes while the warp would wait for p_{b-1})
-        __stcg(v.snap + ((size_t)(b / v.seg - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)rv);
+        __stcg(v.snap + ((size_t)(next - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)rv);
         __threadfence();
     }
     if (b >= 2) {
@@ -433,10 +446,11 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
 #pragma unroll
         for (int jj = 0; jj < kPer; ++jj) pz = fma(-g1[jj], __shfl_sync(kFull, y1, jj), pz);
     }
-    S.fin[1][warp][lane] = pz;
+    double(*sum)[kW] = reinterpret_cast<double(*)[kW]>(&S.tile[0][0][0]);  // (the tiles are done with)
+    sum[warp][lane] = pz;
     __syncthreads();
     if (warp == 0 && !(c == 0 && b == P.skip_publish)) {
-        const double x = (S.fin[1][0][lane] + S.fin[1][1][lane]) + (S.fin[1][2][lane] + S.fin[1][3][lane]);
+        const double x = (sum[0][lane] + sum[1][lane]) + (sum[2][lane] + sum[3][lane]);
         put_tagged(ptag + ((size_t)b * kW + lane) * 2, active ? x : 0.0, ep64);
     }
     TEAM_TRACE(c, b, 4);
@@ -541,9 +555,10 @@ __device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem 
         bad = bad || !(ad > 0.0 && ad <= DBL_MAX);
         const double iad = rcp_refined(ad);
         S.z[row][q] = sg * t[q] * t[q] * iad;
-        if (row == 0 && b > 0 && (b + 2) % v.seg == 0 && (b + 2) / v.seg <= v.nbound) {
+        const int start = seg_at(b, v.seg);
+        if (row == 0 && start > 0 && start <= v.nbound) {
             // a segment starts at this block: the factor of H_b for its carries
-            double *dst = v.rst + (size_t)((b + 2) / v.seg - 1) * ne;
+            double *dst = v.rst + (size_t)(start - 1) * ne;
             for (int m = 0; m < q; ++m) __stcg(dst + tri(q, m), h[tri(q, m)]);
             __stcg(dst + tri(q, q), iad);
         }
@@ -595,23 +610,26 @@ __device__ __forceinline__ void unit_sync(int unit)
 }
 
 // Segments sg0 .. sg0 + UNITS - 1 of column block j.  NV warps share a
-// segment, VW of its KB = NV VW vectors each: a tile passes from warp to
-// warp in shared memory, each applying its vectors' rotations (lane =
-// column, the carries in registers), so that NV tiles are in work at once
-// and a tile's step takes the time of VW vectors, not of KB (in double 64
-// cycles per FMA and warp: 4 us instead of 16 with eight vectors).  The
-// order of the operations on an element is that of one warp doing all
-// vectors.  Tiles and coefficients are staged one step ahead.  The warps'
+// segment, VW of its KB vectors each: a tile passes from warp to warp in
+// shared memory, each applying its vectors' rotations (lane = column, the
+// carries in registers), so that NV tiles are in work at once and a tile's
+// step takes the time of VW vectors, not of KB (in double 64 cycles per FMA
+// and warp: 4 us instead of 16 with eight vectors).  The order of the
+// operations on an element is that of one warp doing all vectors.  For one
+// vector in double and a short column a second warp scales and stores what
+// the first has rotated (a tile 4.0 instead of 6.3 us).  Tiles and coefficients are staged one step ahead.  The warps'
 // places are turned from task to task, so that the last place, which also
 // scales and stores the tile, falls on each of the SM's four FP64 pipes in
 // turn.  A wait that runs out leaves the task running on whatever it has
 // (the launch is being aborted), so that the warps' barriers stay matched.
-template <typename T, int VW, int NV>
-__device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task, SweepSmem<T, VW * NV, NV> &S)
+template <typename T, int VW, int NV, int KB>
+__device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task, SweepSmem<T, KB, NV> &S)
 {
-    using SS = SweepSmem<T, VW * NV, NV>;
+    using SS = SweepSmem<T, KB, NV>;
+    constexpr int NR = KB / VW;  // places that rotate; with NR < NV the last one only scales and stores
+    static_assert(KB % VW == 0 && (NR == NV || NR == NV - 1), "places of a segment");
     using V16 = typename pass::Vec16<T>::type;
-    constexpr int KB = VW * NV, NS = SS::NS;
+    constexpr int NS = SS::NS;
     constexpr int SD = pass::Stride<T>::value;
     constexpr int E = 16 / (int)sizeof(T);
     constexpr int CPC = kW / E;  // 16-byte chunks per column segment
@@ -685,7 +703,11 @@ __device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task
     stage(0);
     pass::cp_commit();
     T uh[VW];
-    if (sg == 0) {
+#pragma unroll
+    for (int w = 0; w < VW; ++w) uh[w] = T(0);
+    if (NR < NV && part >= NR) {
+        // (this place rotates nothing)
+    } else if (sg == 0) {
 #pragma unroll
         for (int w = 0; w < VW; ++w) {
             const int q = part * VW + w;
@@ -729,71 +751,86 @@ __device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task
 #pragma unroll
                 for (int w = 0; w < E; ++w) mycol[i0 + w] = dch[w];
             }
-            T x[kW];
+            if (NR == NV || part < NR) {
+                T x[kW];
 #pragma unroll
-            for (int k = 0; k < CPC; ++k) {
-                const V16 y = colv[k];
+                for (int k = 0; k < CPC; ++k) {
+                    const V16 y = colv[k];
 #pragma unroll
-                for (int w = 0; w < E; ++w) x[k * E + w] = pass::vget<T>(y, w);
-            }
-            // (a lane past the order, and a row at or below the diagonal, keeps what it has)
-            const int rows = !active ? 0 : diag ? lane : kW;
-#pragma unroll
-            for (int k = 0; k < kW; ++k) {
-                T a[VW], b[VW];
-#pragma unroll
-                for (int w = 0; w < VW; ++w) {
-                    a[w] = cf[k * 2 * KB + 2 * w];
-                    b[w] = cf[k * 2 * KB + 2 * w + 1];
+                    for (int w = 0; w < E; ++w) x[k * E + w] = pass::vget<T>(y, w);
                 }
-                if (k < rows) {
+                // (a lane past the order, and a row at or below the diagonal, keeps what it has)
+                const int rows = !active ? 0 : diag ? lane : kW;
+#pragma unroll
+                for (int k = 0; k < kW; ++k) {
+                    T a[VW], b[VW];
 #pragma unroll
                     for (int w = 0; w < VW; ++w) {
-                        x[k] = fma(a[w], uh[w], x[k]);
-                        uh[w] = fma(-b[w], x[k], uh[w]);
+                        a[w] = cf[k * 2 * KB + 2 * w];
+                        b[w] = cf[k * 2 * KB + 2 * w + 1];
+                    }
+                    if (k < rows) {
+#pragma unroll
+                        for (int w = 0; w < VW; ++w) {
+                            x[k] = fma(a[w], uh[w], x[k]);
+                            uh[w] = fma(-b[w], x[k], uh[w]);
+                        }
                     }
                 }
-            }
-            if (part == NV - 1) {
+                if (NR == NV && part == NV - 1) {
 #pragma unroll
-                for (int k = 0; k < kW; ++k)
-                    if (k < rows) x[k] *= U.e[slot][k];
-            }
+                    for (int k = 0; k < kW; ++k)
+                        if (k < rows) x[k] *= U.e[slot][k];
+                }
 #pragma unroll
-            for (int k = 0; k < CPC; ++k) {
-                V16 y;
-                T *yp = reinterpret_cast<T *>(&y);
+                for (int k = 0; k < CPC; ++k) {
+                    V16 y;
+                    T *yp = reinterpret_cast<T *>(&y);
 #pragma unroll
-                for (int w = 0; w < E; ++w) yp[w] = x[k * E + w];
-                colv[k] = y;
+                    for (int w = 0; w < E; ++w) yp[w] = x[k * E + w];
+                    colv[k] = y;
+                }
             }
             if (diag && part == NV - 1) mycol[lane] = (T)(dc * df);
             if (part == NV - 1) {
                 const long long r0 = (long long)r * kW;
                 if (diag && active) __stcg(v.dcar + c0 + lane, dc * df);
                 __syncwarp();
+                constexpr bool scale = NR < NV;  // the rows' scales are still to be applied
+                const T *er = U.e[slot];
                 if (v.vec) {
-                    const int first = diag ? ch * E + E - 1 : 0;
+                    // whole chunks above the diagonal, then, one column a lane, the
+                    // diagonal's chunk
+                    const int first = diag ? (ch + 1) * E : 0;
                     constexpr int step = 32 / CPC;
                     const int k0 = lane / CPC;
                     T *g = v.L + r0 + ch * E + (c0 + k0) * ld;
                     const T *d = tl + k0 * SD + ch * E;
 #pragma unroll
                     for (int cc = k0; cc < kW; cc += step, g += step * ld, d += step * SD)
-                        if (cc >= first && cc < ncol && CHK_TRI(sy, g - v.L, n, ld) && CHK_TRI(sy, g - v.L + E - 1, n, ld))
-                            __stcg(reinterpret_cast<V16 *>(g), *reinterpret_cast<const V16 *>(d));
+                        if (cc >= first && cc < ncol && CHK_TRI(sy, g - v.L, n, ld) && CHK_TRI(sy, g - v.L + E - 1, n, ld)) {
+                            V16 y = *reinterpret_cast<const V16 *>(d);
+                            if (scale) {
+                                T *yp = reinterpret_cast<T *>(&y);
+#pragma unroll
+                                for (int w = 0; w < E; ++w) yp[w] *= er[ch * E + w];
+                            }
+                            __stcg(reinterpret_cast<V16 *>(g), y);
+                        }
                     const int i0 = lane & ~(E - 1);
-                    if (diag && active && i0 + E - 1 > lane) {
+                    if (diag && active) {
 #pragma unroll
                         for (int w = 0; w < E; ++w)
                             if (i0 + w <= lane && CHK_TRI(sy, r0 + i0 + w + (c0 + lane) * ld, n, ld))
-                                __stcg(v.L + r0 + i0 + w + (c0 + lane) * ld, tl[lane * SD + i0 + w]);
+                                __stcg(v.L + r0 + i0 + w + (c0 + lane) * ld,
+                                       tl[lane * SD + i0 + w] * (scale && i0 + w < lane ? er[i0 + w] : T(1)));
                     }
                 } else {
 #pragma unroll 8
                     for (int cc = 0; cc < kW; ++cc)
                         if (c0 + cc < n && (!diag || lane <= cc) && CHK_TRI(sy, (r0 + lane) + (c0 + cc) * ld, n, ld))
-                            __stcg(v.L + (r0 + lane) + (c0 + cc) * ld, tl[cc * SD + lane]);
+                            __stcg(v.L + (r0 + lane) + (c0 + cc) * ld,
+                                   tl[cc * SD + lane] * (scale && (!diag || lane < cc) ? er[lane] : T(1)));
                 }
             }
         }
@@ -846,11 +883,11 @@ __device__ bool set_view(const Launch<T> &P, int i, int s, int epoch, View<T> &v
     v.nb = nb;
     v.pass = s;
     v.npass = passes_of(pr.k);
-    v.units = units_of(KB);
+    v.units = units_of(nb, KB, sizeof(T) == 8);
     v.kb = kb;
     v.KB = KB;
-    v.seg = seg_of(nb, KB);
-    v.nbound = bounds_of(nb, KB);
+    v.seg = seg_of(nb, KB, sizeof(T) == 8);
+    v.nbound = bounds_of(nb, KB, sizeof(T) == 8);
     v.look = look_of(kb);
     v.down_mask = (unsigned)(pr.down_mask >> (s * kTeamKb)) & ((1u << kb) - 1u);
     v.vec = ((pr.ld * (long long)sizeof(T)) & 15) == 0 && (reinterpret_cast<uintptr_t>(pr.L) & 15) == 0;
@@ -903,10 +940,25 @@ __device__ Picked task_at(const View<T> &v, int x, Stage &st)
 {
     Picked p{kTaskNone, 0, 0};
     const int stages = stage_count(v.nb, v.look);
+    // (the column's segments are counted along: a division per stage and block
+    // would cost microseconds)
+    if (st.t == 0) {
+        st.segs = 1;
+        st.left = v.seg + 2 - seg_off(v.seg);  // segs_of grows where b - 2 + off is a multiple of seg
+    }
+    const int ush = v.units >> 1;  // units 1, 2, 4: a shift by 0, 1, 2
     for (; st.t < stages; ++st.t) {
-        const int c = stage_tasks(st.t, v.nb, v.kb, v.seg, v.look, v.units);
+        int c = 0;
+        if (st.t == 0) c += 2 * min(v.nb, kPrepAhead);
+        if (st.t + kPrepAhead < v.nb) c += 2;
+        if (st.t < v.nb) c += v.kb;
+        if (st.t >= v.look) c += 1 + ((st.segs + v.units - 1) >> ush);
         if (x < st.first + c) break;
         st.first += c;
+        if (st.t >= v.look && --st.left == 0) {
+            ++st.segs;
+            st.left = v.seg;
+        }
     }
     if (st.t >= stages) return p;
     int y = x - st.first;
@@ -957,7 +1009,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) team_kernel(
     // thread 0's scheduling state
     const int team = blockIdx.x % P.nteams;
     int prob = -1;      // the problem in the view
-    Stage st{0, 0, 0};  // cursor in its task list
+    Stage st{0, 0, 0, 0, 0};  // cursor in its task list
     if (threadIdx.x == 0) {
         v.pass = -1;
         s_task.kind = kTaskNone;
@@ -1008,7 +1060,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) team_kernel(
             if (x >= 0) {
                 if (want != prob) {
                     prob = want;
-                    st = Stage{0, 0, 0};
+                    st = Stage{0, 0, 0, 0, 0};
                     v.pass = -1;
                 }
                 bool ok = true;
@@ -1016,7 +1068,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) team_kernel(
                 if (v.pass < 0) ok = set_view(P, prob, 0, epoch, v);
                 Picked pk = ok ? task_at(v, (int)x - st.passes, st) : Picked{kTaskNone, 0, 0};
                 while (ok && pk.kind == kTaskNone && v.pass + 1 < np) {
-                    st = Stage{0, 0, st.passes + st.first};
+                    st = Stage{0, 0, st.passes + st.first, 0, 0};
                     ok = set_view(P, prob, v.pass + 1, epoch, v);
                     if (ok) pk = task_at(v, (int)x - st.passes, st);
                 }
@@ -1036,10 +1088,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) team_kernel(
             coef_task<T>(P, v, pk.a, S.coef);
         } else {
             switch (v.KB) {
-            case 1: sweep_task<T, 1, 1>(P, v, pk.a, pk.b, S.sweep1); break;
-            case 2: sweep_task<T, 1, 2>(P, v, pk.a, pk.b, S.sweep2); break;
-            case 4: sweep_task<T, 1, 4>(P, v, pk.a, pk.b, S.sweep4); break;
-            default: sweep_task<T, 2, 4>(P, v, pk.a, pk.b, S.sweep8); break;
+            case 1:
+                if (sizeof(T) == 8 && v.units == 2) sweep_task<T, 1, 2, 1>(P, v, pk.a, pk.b, S.sweep12);
+                else sweep_task<T, 1, 1, 1>(P, v, pk.a, pk.b, S.sweep1);
+                break;
+            case 2: sweep_task<T, 1, 2, 2>(P, v, pk.a, pk.b, S.sweep2); break;
+            case 4: sweep_task<T, 1, 4, 4>(P, v, pk.a, pk.b, S.sweep4); break;
+            default: sweep_task<T, 2, 4, 8>(P, v, pk.a, pk.b, S.sweep8); break;
             }
         }
     }

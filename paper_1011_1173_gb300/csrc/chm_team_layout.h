@@ -17,30 +17,43 @@ constexpr int kTeamKb = 8;
 CHM_HD inline int kb_inst(int kb) { return kb <= 1 ? 1 : kb <= 2 ? 2 : kb <= 4 ? 4 : 8; }
 CHM_HD inline int passes_of(int k) { return (k + kTeamKb - 1) / kTeamKb; }
 
-// Segments of a column swept by one task: its four warps take four segments
-// of one vector, two of two, or one of four or eight (one or two vectors a
-// warp, see sweep_task).
-CHM_HD inline int units_of(int KB) { return KB == 1 ? 4 : KB == 2 ? 2 : 1; }
+// Segments of a column swept by one task of four warps: one of four or eight
+// vectors, two of two, four of one; in double up to 64 row blocks two of one,
+// with a second warp each that scales and stores (see sweep_task).
+CHM_HD inline bool store_warp(int nb, int KB, bool f64) { return f64 && KB == 1 && nb <= 64; }
+CHM_HD inline int units_of(int nb, int KB, bool f64) { return KB >= 4 ? 1 : KB == 2 || store_warp(nb, KB, f64) ? 2 : 4; }
 
-// Row blocks per sweep segment, a multiple of four.  One or two vectors:
-// four, while that takes at most 64 segments of a column (whose starts'
+// Row blocks per sweep segment.  One or two vectors: two up to 64 row blocks
+// in double (n = 512 0.094 to 0.070 ms; in float, whose tiles take a third of
+// the time, no gain), else four, while that takes at most 64 segments of a column (whose starts'
 // residuals are kept, n values per vector each): the last segment is what
 // is left to do when the substitution ends.  More vectors: a twelfth of the
-// column, since a task of `seg` tiles fills and drains its four warps'
-// pipeline in seg + 3 steps (n = 5000, 16 vectors, double: 2.06 ms with
-// segments of four, 1.69 with sixteen).
-CHM_HD inline int seg_of(int nb, int KB)
+// column, at least four, since a task of `seg` tiles fills and drains its
+// four warps' pipeline in seg + 3 steps (n = 5000, 16 vectors, double: 2.06 ms
+// with segments of four, 1.69 with sixteen).  A multiple of four from four on.
+CHM_HD inline int seg_of(int nb, int KB, bool f64)
 {
+    if (f64 && KB <= 2 && nb <= 64) return 2;
     const int s = (KB <= 2 ? (nb + 63) / 64 : (nb + 11) / 12) + 3;
     return s < 7 ? 4 : s & ~3;
 }
-// Segment s >= 1 starts at row block s seg - 2.  A start needs the residual a
-// SUB step keeps, which covers row blocks up to b - 2 of column block b, so
-// b's last segment is the one that starts at or before row block b - 2.
-CHM_HD inline int segs_of(int b, int seg) { return 1 + b / seg; }
-CHM_HD inline int seg_start(int s, int seg) { return s > 0 ? s * seg - 2 : 0; }
-// Segment starts of the last column (the most any has).
-CHM_HD inline int bounds_of(int nb, int KB) { return (nb - 1) / seg_of(nb, KB); }
+// Segment s >= 1 starts at row block s seg - off: where a group of four tiles
+// of the substitution (4 i - 2 .. 4 i + 1) begins, and for segments of two
+// also in its middle.  A start needs the residual a SUB step keeps, which
+// covers row blocks up to b - 2 of column block b, so b's last segment is the
+// one that starts at or before row block b - 2.
+CHM_HD inline int seg_off(int seg) { return seg == 2 ? 0 : 2; }
+CHM_HD inline int seg_start(int s, int seg) { return s > 0 ? s * seg - seg_off(seg) : 0; }
+CHM_HD inline int segs_of(int b, int seg)
+{
+    const int x = b - 2 + seg_off(seg);
+    return 1 + (x > 0 ? x / seg : 0);
+}
+// Segment s if one starts at row block r (> 0), else 0.
+CHM_HD inline int seg_at(int r, int seg) { return r > 0 && (r + seg_off(seg)) % seg == 0 ? (r + seg_off(seg)) / seg : 0; }
+// Segment starts of the last column (the most any has); in double there are at
+// least as many as in float.
+CHM_HD inline int bounds_of(int nb, int KB, bool f64) { return segs_of(nb - 1, seg_of(nb, KB, f64)) - 1; }
 
 // Byte offsets inside the data record of one pass of kb vectors (element
 // sizes are the double's, so that one size serves both types).
@@ -55,7 +68,7 @@ struct PassRec {
 };
 CHM_HD inline PassRec pass_rec(int nb, int kb)
 {
-    const size_t rows = (size_t)nb * kW, KB = (size_t)kb_inst(kb), nd = (size_t)bounds_of(nb, kb_inst(kb));
+    const size_t rows = (size_t)nb * kW, KB = (size_t)kb_inst(kb), nd = (size_t)bounds_of(nb, kb_inst(kb), true);
     PassRec r;
     size_t x = 0;
     r.ug = x;     x += rows * 3 * kW * 8;
@@ -118,12 +131,12 @@ CHM_HD inline int stage_tasks(int t, int nb, int kb, int seg, int look, int unit
     return c;
 }
 // All tasks of a problem.
-inline int prob_tasks(int nb, int k)
+inline int prob_tasks(int nb, int k, bool f64)
 {
     int total = 0;
     for (int s = 0; s < passes_of(k); ++s) {
         const int kb = k - s * kTeamKb < kTeamKb ? k - s * kTeamKb : kTeamKb;
-        const int KB = kb_inst(kb), look = look_of(kb), units = units_of(KB), seg = seg_of(nb, KB);
+        const int KB = kb_inst(kb), look = look_of(kb), units = units_of(nb, KB, f64), seg = seg_of(nb, KB, f64);
         for (int t = 0; t < stage_count(nb, look); ++t) total += stage_tasks(t, nb, kb, seg, look, units);
     }
     return total;
