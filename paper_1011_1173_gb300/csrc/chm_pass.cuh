@@ -528,6 +528,114 @@ __device__ __forceinline__ void lane_mv_reg(const T (&mrow)[kB], const T *x, T (
     for (int q = 0; q < KB; ++q) out[q] = a0[q] + a1[q];
 }
 
+// A warp's 32 x 32 matrix times 32 x KB product, every lane with KB of the
+// results: element e of lane's share is entry (row(lane, e), col(lane, e)).
+//
+// What bounds such a product is shared memory: with a row of the result per
+// lane (lane_mv) every lane takes all of x, 32 KB values, and the eight
+// products of a chain step with eight vectors in float keep the chain
+// block's shared memory busy for 1.1 us of a 2.0 us step.  With eight vectors
+// in float a lane therefore sums half of the 32 terms of four rows and half
+// of the vectors and swaps two rows' sums with the lane that has the other
+// half: 32 16-byte loads and 8 shuffles instead of 72 loads (n = 32768: 2.52 to
+// 2.42 ms, the median step 2.05 to 1.8 us; n = 16384: 1.26 to 1.22).  Not with four, whose chain
+// waits for the workers' sums rather than for its products (1.59 to 1.78 ms),
+// and not in double, where the FP64 rate binds.
+template <typename T, int KB>
+struct MvShare {
+    static constexpr bool split = sizeof(T) == 4 && KB == 8;
+    static constexpr int Q = split ? KB / 2 : KB;  // consecutive vectors of one row
+    static __device__ __forceinline__ int row(int lane, int e)
+    {
+        return split ? (lane & 7) + (lane >> 4) * 16 + (e / Q) * 8 : lane;
+    }
+    static __device__ __forceinline__ int col(int lane, int e) { return split ? ((lane >> 3) & 1) * Q + e % Q : e; }
+};
+// The lane's share of a Rows array.
+template <typename T, int KB>
+__device__ __forceinline__ void share_store(T *base, int lane, const T (&v)[KB])
+{
+    using M = MvShare<T, KB>;
+    if constexpr (M::split) {
+        constexpr int E = 4;
+#pragma unroll
+        for (int e = 0; e < KB; e += E) {
+            float4 x;
+#pragma unroll
+            for (int u = 0; u < E; ++u) reinterpret_cast<T *>(&x)[u] = v[e + u];
+            *reinterpret_cast<float4 *>(base + M::row(lane, e) * Rows<T, KB>::KS + M::col(lane, e)) = x;
+        }
+    } else {
+        row_store<T, KB>(base, lane, v);
+    }
+}
+template <typename T, int KB>
+__device__ __forceinline__ void share_load(const T *base, int lane, T (&v)[KB])
+{
+    using M = MvShare<T, KB>;
+    if constexpr (M::split) {
+        constexpr int E = 4;
+#pragma unroll
+        for (int e = 0; e < KB; e += E) {
+            const float4 x = *reinterpret_cast<const float4 *>(base + M::row(lane, e) * Rows<T, KB>::KS + M::col(lane, e));
+#pragma unroll
+            for (int u = 0; u < E; ++u) v[e + u] = reinterpret_cast<const T *>(&x)[u];
+        }
+    } else {
+        row_load<T, KB>(base, lane, v);
+    }
+}
+// out (+)= M x, the lane's share (M staged with Stride, x a Rows array).
+template <typename T, int KB>
+__device__ __forceinline__ void share_mv(const T *M, const T *x, T (&out)[KB], int lane, bool acc = false)
+{
+    using Sh = MvShare<T, KB>;
+    if constexpr (Sh::split) {
+        constexpr int Q = Sh::Q, E = 4, S = Stride<T>::value, XS = Rows<T, KB>::KS;
+        const int g = lane & 7, h = lane >> 4;
+        // (rows g, g + 8, g + 16, g + 24: eight lanes' 16-byte loads meet distinct banks)
+        const T *mr = M + g * S + h * (kB / 2);
+        const T *xr = x + h * (kB / 2) * XS + ((lane >> 3) & 1) * Q;
+        T a[4][Q];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) a[i][q] = T(0);
+#pragma unroll
+        for (int c = 0; c < kB / 2; c += 4) {
+            float4 m[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) m[i] = *reinterpret_cast<const float4 *>(mr + i * 8 * S + c);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                T xv[Q];
+#pragma unroll
+                for (int q = 0; q < Q; q += E) {
+                    const float4 w = *reinterpret_cast<const float4 *>(xr + (c + u) * XS + q);
+#pragma unroll
+                    for (int z = 0; z < E; ++z) xv[q + z] = reinterpret_cast<const T *>(&w)[z];
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const T mv = u == 0 ? m[i].x : u == 1 ? m[i].y : u == 2 ? m[i].z : m[i].w;
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) a[i][q] = fma(mv, xv[q], a[i][q]);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const T other = __shfl_xor_sync(0xffffffffu, h ? a[i][q] : a[i + 2][q], 16);
+                const T sum = (h ? a[i + 2][q] : a[i][q]) + other;
+                out[i * Q + q] = acc ? out[i * Q + q] + sum : sum;
+            }
+    } else {
+        lane_mv<T, KB>(M, x, out, lane, acc);
+    }
+}
+
 // A value published as epoch-tagged 64-bit words (one per 32 bits of T):
 // each 8-byte store is single-copy atomic, so a reader that sees every word
 // tagged with the current epoch has the value, and no fence or flag is needed.
@@ -971,11 +1079,11 @@ __device__ void trsm_chain(const Args<T> &A, unsigned char *smem)
 #pragma unroll
             for (int q = 0; q < KB; ++q) acc[q] = T(0);
             for (int j = 1; j <= cc && j <= m; ++j)
-                lane_mv<T, KB>(S.G[m % C::RS][j - 1], S.P[(m - j) % C::RP], acc, lane, true);
-            row_load<T, KB>(S.Z[m % C::RZ], lane, out);
+                share_mv<T, KB>(S.G[m % C::RS][j - 1], S.P[(m - j) % C::RP], acc, lane, true);
+            share_load<T, KB>(S.Z[m % C::RZ], lane, out);
 #pragma unroll
             for (int q = 0; q < KB; ++q) out[q] -= acc[q];
-            row_store<T, KB>(S.P[m % C::RP], lane, out);
+            share_store<T, KB>(S.P[m % C::RP], lane, out);
             __syncwarp();
             mb_arrive(&S.p_full[m % C::RP]);
             mb_arrive(&S.w_empty[m % C::RZ]);
@@ -1024,17 +1132,17 @@ __device__ void trsm_chain(const Args<T> &A, unsigned char *smem)
                 const int b = m + j;
                 if (b >= nb) break;
                 T out[KB];
-                lane_mv<T, KB>(S.near[j - cc - 1][m % C::RS], pm, out, lane);
+                share_mv<T, KB>(S.near[j - cc - 1][m % C::RS], pm, out, lane);
                 // the running sum of block b's near terms, offsets d, d - 1, ..., j:
                 // offset j + 1's warp left the terms above in its slot at step m - 1
                 if (j < d && j + 1 <= b) {
                     MW(S.t_full[(j - cc) % kNearWarps], m - 1, C::RT, b);
                     T up[KB];
-                    row_load<T, KB>(S.Tn[j - cc][b % C::RT], lane, up);
+                    share_load<T, KB>(S.Tn[j - cc][b % C::RT], lane, up);
 #pragma unroll
                     for (int q = 0; q < KB; ++q) out[q] += up[q];
                 }
-                row_store<T, KB>(S.Tn[j - cc - 1][b % C::RT], lane, out);
+                share_store<T, KB>(S.Tn[j - cc - 1][b % C::RT], lane, out);
             }
             __syncwarp();
             mb_arrive(&S.p_empty[m % C::RP]);
@@ -1168,6 +1276,7 @@ __device__ bool trsm_workers(const Args<T> &A, unsigned char *smem)
     using W = WorkerCfg<T, KB>;
     constexpr int SD = Stride<T>::value;
     constexpr int TW = Tag<T>::words;
+    using Sh = MvShare<T, KB>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp >= W::warps) return false;
     T *base = reinterpret_cast<T *>(smem + (size_t)warp * W::warp_bytes);
@@ -1188,8 +1297,7 @@ __device__ bool trsm_workers(const Args<T> &A, unsigned char *smem)
         const bool col_ok = c0 + lane < n;
         T z[KB];
 #pragma unroll
-        for (int q = 0; q < KB; ++q)
-            z[q] = col_ok ? vin(A, sy, c0 + lane, q) : T(0);
+        for (int e = 0; e < KB; ++e) z[e] = vin(A, sy, c0 + Sh::row(lane, e), Sh::col(lane, e));
         const int nfar = b - d;
         for (int r = 0; r < W::NS - 1 && r < nfar; ++r) {
             stage_tile(sy, base + (size_t)(r % W::NS) * kB * SD, A.L, ld, (long long)r * kB, c0, n, kB, vec, lane);
@@ -1198,9 +1306,9 @@ __device__ bool trsm_workers(const Args<T> &A, unsigned char *smem)
         for (int r = 0; r < nfar; ++r) {
             if (r > 0 && r % A.seg == 0) {
                 // a sweep segment boundary: the residual before row block r
-                T *sn = A.snap + (((size_t)(r / A.seg - 1) * nb + b) * kB + lane) * KB;
+                T *sn = A.snap + ((size_t)(r / A.seg - 1) * nb + b) * kB * KB;
 #pragma unroll
-                for (int q = 0; q < KB; ++q) sn[q] = z[q];
+                for (int e = 0; e < KB; ++e) sn[Sh::row(lane, e) * KB + Sh::col(lane, e)] = z[e];
                 if (A.fused) {
                     // tiles 0 .. r - 1 are read and the residual is out: the
                     // sweep may now rewrite the tiles of the segment that ends here
@@ -1240,7 +1348,7 @@ __device__ bool trsm_workers(const Args<T> &A, unsigned char *smem)
             cp_wait<W::NS - 1>();
             __syncwarp();
             T t[KB];
-            lane_mv<T, KB>(base + (size_t)(r % W::NS) * kB * SD, Pr, t, lane);
+            share_mv<T, KB>(base + (size_t)(r % W::NS) * kB * SD, Pr, t, lane);
 #pragma unroll
             for (int q = 0; q < KB; ++q) z[q] -= t[q];
             __syncwarp();
@@ -1249,14 +1357,14 @@ __device__ bool trsm_workers(const Args<T> &A, unsigned char *smem)
         // Dinv_b staged into a free tile slot, Zf_b into the P row buffer
         stage_dense(base, A.Dinv + (size_t)b * kB * kB, lane);
         cp_commit();
-        row_store<T, KB>(Pr, lane, z);
+        share_store<T, KB>(Pr, lane, z);
         cp_wait<0>();
         __syncwarp();
-        lane_mv<T, KB>(base, Pr, z, lane);
+        share_mv<T, KB>(base, Pr, z, lane);
         __syncwarp();
-        long long *zt = A.Ztag + ((size_t)b * kB + lane) * KB * TW;
+        long long *zt = A.Ztag + (size_t)b * kB * KB * TW;
 #pragma unroll
-        for (int q = 0; q < KB; ++q) put_tag(zt + q * TW, z[q], ep64);
+        for (int e = 0; e < KB; ++e) put_tag(zt + (Sh::row(lane, e) * KB + Sh::col(lane, e)) * TW, z[e], ep64);
         if (A.trace && lane == 0) A.trace[(size_t)b * 16 + 9] = global_ns();
         if (A.fused) {
             // every tile of the far part read: the sweep's segments of this column may go
