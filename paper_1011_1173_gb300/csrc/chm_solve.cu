@@ -18,7 +18,7 @@
 // whatever the number of resident blocks.
 //
 // A step sums the tiles whose y is already published, staged through shared
-// memory (a lane reads down its column), the third and fourth tiles back
+// memory (a lane reads down its column; tile_sum), the third and fourth tiles back
 // split over the four warps, and multiplies by U; between one block's result and the next
 // block's there is one 32 x 32 product (eight FMAs per warp and right-hand
 // side), one barrier and a four-way sum.  With the two nearest tiles
@@ -94,7 +94,7 @@ union SolveSmem {
     PrepSmem prep;
     struct {
         T tile[kWarps][2][kW * pass::Stride<T>::value];
-        double y[kWarps][R][kW];
+        alignas(16) double y[kWarps][R][kW][sizeof(T) == 4 ? 2 : 1];  // a tile's values (in float, as three floats)
         double part[2][kWarps][R][kW];
     };
     __device__ SolveSmem() {}
@@ -221,9 +221,9 @@ __device__ void preph_task(const SolveArgs<T> &a, const SyncArgs &sy, int b, Pre
     publish(a.hflag + b, sy.epoch);
 }
 
-// t[j] = L[row j, column lane] of a staged tile, in double.
+// t[j] = L[row j, column lane] of a staged tile.
 template <typename T>
-__device__ __forceinline__ void tile_column(const T *tl, double (&t)[kW])
+__device__ __forceinline__ void tile_column(const T *tl, T (&t)[kW])
 {
     constexpr int E = 16 / (int)sizeof(T);
     using V16 = typename pass::Vec16<T>::type;
@@ -231,21 +231,80 @@ __device__ __forceinline__ void tile_column(const T *tl, double (&t)[kW])
     for (int j = 0; j < kW; j += E) {
         const V16 x = *reinterpret_cast<const V16 *>(tl + j);
 #pragma unroll
-        for (int e = 0; e < E; ++e) t[j + e] = (double)pass::vget<T>(x, e);
+        for (int e = 0; e < E; ++e) t[j + e] = pass::vget<T>(x, e);
     }
 }
-// acc[r] += sum over the tile's 32 entries of t[j] y[r][j].
+// acc[r] += sum over a tile's 32 entries of t[j] v_j[r], lane j holding v_j;
+// y is the warp's space for them.
 template <int R>
-__device__ __forceinline__ void tile_sum(const double (&t)[kW], const double (*y)[kW], double (&acc)[R])
+__device__ __forceinline__ void tile_sum(const double (&t)[kW], const double (&v)[R], double (*y)[kW][1], int lane,
+                                         double (&acc)[R])
 {
+#pragma unroll
+    for (int r = 0; r < R; ++r) y[r][lane][0] = v[r];
+    __syncwarp();
 #pragma unroll
     for (int j = 0; j < kW; j += 2)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const double2 u = *reinterpret_cast<const double2 *>(&y[r][j]);
+            const double2 u = *reinterpret_cast<const double2 *>(y[r][j]);
             acc[r] = fma(t[j], u.x, acc[r]);
             acc[r] = fma(t[j + 1], u.y, acc[r]);
         }
+    __syncwarp();
+}
+// For a factor in float: a conversion is as slow as an FMA in double (64
+// cycles a warp instruction), and together they bound every solve but the
+// smallest.  The values are scaled by a power of two to below 2^-5 (whatever
+// their range, no product with the factor's entries overflows) and split into
+// three floats that hold all of their 53 bits; the products are split exactly,
+// and the tile's sum is kept in three floats, two of them added to exactly
+// (two-sum): to about 2^-70 of the sum of its terms' sizes, against 2^-50 in double.  The
+// tiles' sums are added up in double.  A tile costs 1060 FP32 and 15 FP64
+// instructions a right-hand side instead of 64 FP64 ones: n = 16384, 1 / 5 / 8
+// right-hand sides 1.65 / 2.75 / 3.92 ms against 2.18 / 5.96 / 8.96.
+__device__ __forceinline__ void two_sum(float &s, float x, float &err)
+{
+    const float u = __fadd_rn(s, x), b = __fsub_rn(u, s);
+    err = __fadd_rn(__fsub_rn(s, __fsub_rn(u, b)), __fsub_rn(x, b));
+    s = u;
+}
+template <int R>
+__device__ __forceinline__ void tile_sum(const float (&t)[kW], const double (&v)[R], double (*y)[kW][2], int lane,
+                                         double (&acc)[R])
+{
+    double up[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        // the largest value's exponent, kept where both powers of two are finite
+        const unsigned top = __reduce_max_sync(kFull, (unsigned)__double2hiint(v[r]) & 0x7fffffffu) >> 20;
+        const int ex = min(max((int)top, 64), 2000);
+        up[r] = __hiloint2double((ex + 6) << 20, 0);
+        double x = v[r] * __hiloint2double((2040 - ex) << 20, 0);
+        const float h = (float)x;
+        x -= (double)h;
+        const float m = (float)x;
+        *reinterpret_cast<float4 *>(y[r][lane]) = make_float4(h, m, (float)(x - (double)m), 0.0f);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float s = 0.0f, e = 0.0f, l = 0.0f;
+#pragma unroll
+        for (int j = 0; j < kW; ++j) {
+            const float4 u = *reinterpret_cast<const float4 *>(y[r][j]);
+            const float p = __fmul_rn(t[j], u.x), d = fmaf(t[j], u.x, -p);
+            const float q = __fmul_rn(t[j], u.y), g = fmaf(t[j], u.z, fmaf(t[j], u.y, -q));
+            float e0, e1, e2, e3;
+            two_sum(s, p, e0);
+            two_sum(e, d, e1);
+            two_sum(e, q, e2);
+            two_sum(e, e0, e3);
+            l = __fadd_rn(l, __fadd_rn(__fadd_rn(g, e1), __fadd_rn(e2, e3)));
+        }
+        acc[r] = fma((double)s + ((double)e + (double)l), up[r], acc[r]);
+    }
+    __syncwarp();
 }
 
 // Chain c's step at block b, forward.
@@ -293,20 +352,16 @@ __device__ void forward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lon
     int slot = 0;
     for (int p = warp; p < far; p += kWarps) {
         stage(p + kWarps, slot ^ 1);
-        // (the tile's column in registers, and in double, before y is waited for)
+        // (the tile's column in registers before y is waited for)
         pass::cp_wait<1>();
         __syncwarp();
-        double t[kW];
+        T t[kW];
         tile_column<T>(S.tile[warp][slot] + lane * SD, t);
         const long long *w = ytag + tag_at<R>(p, 0, 0);
         double y[R];
         // (a warp's last tile is waited for as closely as the chain's next steps)
         wait_vals<R>(sy, w + tag_at<R>(0, lane, 0), p + kWarps < far ? w + tag_at<R>(1, 0, 0) - 1 : nullptr, ep64, b, y);
-#pragma unroll
-        for (int r = 0; r < R; ++r) S.y[warp][r][lane] = y[r];
-        __syncwarp();
-        tile_sum<R>(t, S.y[warp], acc);
-        __syncwarp();
+        tile_sum<R>(t, y, S.y[warp], lane, acc);
         slot ^= 1;
     }
     pass::cp_wait<0>();
@@ -408,18 +463,14 @@ __device__ void backward_task(const SolveArgs<T> &a, const SyncArgs &sy, long lo
     for (int q = nb - 1 - warp; q >= b + 5; q -= kWarps) {
         const long long q0 = (long long)q * kW;
         const int ncq = (int)min((long long)kW, n - q0);
-        double t[kW];
+        T t[kW];
 #pragma unroll
         for (int i = 0; i < kW; ++i)
-            t[i] = (active && i < ncq && CHK_TRI(sy, rowo + (q0 + i) * ld, n, ld)) ? (double)__ldg(row + (q0 + i) * ld) : 0.0;
+            t[i] = (active && i < ncq && CHK_TRI(sy, rowo + (q0 + i) * ld, n, ld)) ? __ldg(row + (q0 + i) * ld) : T(0);
         const long long *w = xtag + tag_at<R>(q, 0, 0);
         double x[R];
         wait_vals<R>(sy, w + tag_at<R>(0, lane, 0), q - kWarps >= b + 5 ? w + tag_at<R>(1, 0, 0) - 1 : nullptr, ep64, b, x);
-#pragma unroll
-        for (int r = 0; r < R; ++r) S.y[warp][r][lane] = x[r];
-        __syncwarp();
-        tile_sum<R>(t, S.y[warp], acc);
-        __syncwarp();
+        tile_sum<R>(t, x, S.y[warp], lane, acc);
     }
     // y_b: this chain's forward result, or the caller's
     double yv[R];
