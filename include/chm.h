@@ -245,7 +245,8 @@ int chm_batch_plan_destroy(void *plan);
  * launch formed from requests that arrived while another was running
  * overlaps it on the device.  Requests on one factor run one after another
  * in submission order, each in its own launch; a factor's result is
- * bit-identical to applying the same requests alone with chm_modify_ex.
+ * bit-identical to applying the same requests alone with chm_modify_ex
+ * where that runs the team kernel too (chm_config_set).
  *
  * chm_server_create
  *   hbm_budget_bytes  device memory the server may hold: factors (n^2
@@ -313,7 +314,8 @@ int chm_server_destroy(void *srv);
  *          left unchanged
  *   nrhs   number of right-hand sides, nrhs >= 0 (0 is a no-op)
  *   dtype  CHM_F64: double L and B, double arithmetic.  CHM_F32_MIXED: float
- *          L and B, every product and sum in double, X rounded to float once
+ *          L and B, every product and sum in double or (the sums of a 32 x 32
+ *          tile, kept in three floats) closer, X rounded to float once
  * Stream-ordered like chm_update (enqueue it after a modification on the
  * same stream to solve with the modified factor).  Each 32 x 32 diagonal
  * block is applied through its explicit inverse.  If some L_ii <= 0 or is
@@ -449,7 +451,7 @@ int chm_microbench(int which, double *out, int nout);
  *         factor once for the whole block of vectors.
  * The automatic rule takes the pass kernels when the factor's upper
  * triangle is at least 32 MB in float (with 8 or more vectors above order
- * 6500 only) or 256 MB in double (with one vector; two above order 12000, up
+ * 5500 only) or 256 MB in double (with one vector; two above order 12000, up
  * to 8 above 16384), and for a factor of order >= 64 in page-locked host
  * memory modified by two or more vectors (it then crosses the CPU-GPU link
  * three times per pass of up to 16 vectors; the wave kernel twice per

@@ -105,9 +105,9 @@ int path_setting()
 
 // The built-in rule: the pass path once the factor is larger than about a
 // third of L2 (where path 1's kernels start to re-stream it), but
-// - in float not for eight or more vectors up to order 6500 (n = 5000, pass /
+// - in float not for eight or more vectors up to order 5500 (n = 5000, pass /
 //   team kernel: k = 4 0.31 / 0.33 ms, k = 8 0.50 / 0.41, k = 16 0.99 / 0.72;
-//   n = 8192: k = 16 1.42 / 1.49);
+//   n = 6001: k = 8 0.73 / 0.80, k = 16 1.47 / 1.43; n = 8192: k = 16 1.42 / 1.49);
 // - in double only up to 8 vectors: beyond that the paths run at the FP64 rate
 //   (n = 32768: 25.0 against 25.9 ms at k = 8, 50.1 against 50.1 at k = 16, the
 //   wave kernel ahead at k = 64), and of those with fewer the larger ones
@@ -122,7 +122,7 @@ static bool rule_pass(long long n, long long k, int dtype, bool host_factor)
     if (host_factor) return n >= 64 && k >= 2;
     const double bytes = (double)(dtype == CHM_F64 ? 8 : 4) * n * n / 2;
     if (dtype == CHM_F64) return bytes >= 256e6 && (k <= 1 || (k <= 2 && n > 12000) || (k <= 8 && n > 16384));
-    return bytes >= 32e6 && (k < 8 || n > 6500);
+    return bytes >= 32e6 && (k < 8 || n > 5500);
 }
 
 PassChoice builtin_choice(long long n, long long k, int dtype, bool host_factor)
