@@ -77,6 +77,8 @@ int launch_wave(int dtype, const Prob *single, const Prob *d_probs, const int *d
 // memory, with `tasks` tasks in all.  cfg.groups is the number of teams.
 // `trace` is null or a device array of k * nb * kTracePoints words.
 ScratchNeed team_need(const ProbShape *shapes, int count);
+// Scratch that serves one problem of any order up to sh.n with up to sh.k vectors.
+ScratchNeed team_need_cap(const ProbShape &sh);
 void team_carve(const ProbShape *shapes, int count, int dtype, const Scratch &sc, Prob *problems);
 int team_occupancy(int dtype, int dev, int *ctas_per_sm);
 int launch_team(int dtype, const Prob *single, const Prob *d_probs, int nprobs, long long tasks, const Scratch &sc,

@@ -251,17 +251,44 @@ int check_reachable(const void *p)
 // k = 16 1.69 / 1.98, k = 64 6.2 / 6.6; n = 8192 k = 8 2.1 / 2.9, k = 16 3.9 /
 // 4.0, k = 64 14.5 / 13.8; n = 12000 k = 8 4.35 / 4.48; n = 16384 k = 4 4.3
 // (the pass kernels 4.8), k = 6 6.6 / 6.2, k = 8 7.7 / 7.4; float: n = 2000
-// k = 1 0.13 / 0.41, k = 16 0.27 / 0.65; n = 8192 k = 64 5.5 / 8.6.
+// k = 1 0.13 / 0.41, k = 16 0.27 / 0.65; n = 8192 k = 64 5.5 / 8.6.  Each
+// range: orders up to n with up to k vectors a launch.
+struct TeamRange {
+    long long n;
+    int k;
+};
+static const TeamRange kTeamF64[] = {{6144, kMaxWaves}, {8192, 16}, {12288, 8}, {16384, 4}};
+static const TeamRange kTeamF32[] = {{8192, kMaxWaves}};
+static const TeamRange *team_ranges(int dtype, int *count)
+{
+    *count = dtype == CHM_F64 ? 4 : 1;
+    return dtype == CHM_F64 ? kTeamF64 : kTeamF32;
+}
 bool use_team(long long n, long long k, int dtype)
 {
-    if (dtype != CHM_F64) return n <= 8192;
-    return n <= 6144 || (n <= 8192 && k <= 16) || (n <= 12288 && k <= 8) || (n <= 16384 && k <= 4);
+    int count = 0;
+    const TeamRange *r = team_ranges(dtype, &count);
+    for (int i = 0; i < count; ++i)
+        if (n <= r[i].n && std::min<long long>(k, kMaxWaves) <= r[i].k) return true;
+    return false;
 }
 
-// The scratch of path 1 for one launch.
+// The scratch of path 1 for launches of up to sh.k vectors: what this shape
+// takes and what any call of the same or a smaller size does (so that a
+// stream's workspace is never outgrown by one), whichever kernel it runs on.
 static ScratchNeed single_need(const ProbShape &sh, int dtype)
 {
-    return use_team(sh.n, sh.k, dtype) ? team_need(&sh, 1) : scratch_need(&sh, 1);
+    ScratchNeed need;
+    if (!use_team(sh.n, sh.k, dtype)) need = scratch_need(&sh, 1);
+    int count = 0;
+    const TeamRange *r = team_ranges(dtype, &count);
+    for (int i = 0; i < count; ++i) {
+        const ScratchNeed t = team_need_cap(ProbShape{std::min(sh.n, r[i].n), std::min(sh.k, r[i].k)});
+        need.iflags = std::max(need.iflags, t.iflags);
+        need.progress = std::max(need.progress, t.progress);
+        need.data = std::max(need.data, t.data);
+    }
+    return need;
 }
 
 size_t single_workspace_bytes(long long n, long long k, int dtype)
@@ -412,7 +439,7 @@ static unsigned long long down_mask(const int8_t *sigma, int sign, long long q0,
 }
 
 // Enqueue the launches of one modification, at most kw_max waves each, on
-// scratch `sc` (already large enough for kw_max waves).
+// scratch `sc` (already large enough for launches of kw_max and of what is left).
 static int enqueue_single(void *L, long long n, long long ld, const void *V, long long ldv, long long k,
                           const int8_t *sigma, int sign, int dtype, cudaStream_t stream, long long *d_info,
                           const Scratch &sc, int kw_max, bool allow_trace, bool team)
@@ -650,18 +677,22 @@ static int noalloc_setup(int dev, NoAllocState **out)
     return CHM_OK;
 }
 
-// Vectors per launch that fit the array, of the k asked for (0: none).  The
+// Vectors per launch that fit the array, of the `left` asked for (0: none); the
+// last launch, of what is left, has to fit as well (fewer vectors can take more).  The
 // team kernel's launches hold whole passes, so that the passes, and with
 // them the result, are those of one launch.
-static int noalloc_vectors(long long n, int k, bool team)
+static int noalloc_vectors(long long n, long long left, bool team)
 {
-    for (int kw = k; kw >= 1; --kw) {
+    const int k = (int)std::min<long long>(left, kMaxWaves);
+    auto fits = [&](int kw) {
         const ProbShape sh{n, kw};
         const ScratchNeed need = team ? team_need(&sh, 1) : scratch_need(&sh, 1);
+        return need.iflags <= kNoAllocIflags && need.progress <= kNoAllocProgress &&
+               need.data <= kNoAllocBytes - kNoAllocDataOff;
+    };
+    for (int kw = k; kw >= 1; --kw) {
         if (team && kw < k && kw % team::kTeamKb != 0) continue;
-        if (need.iflags <= kNoAllocIflags && need.progress <= kNoAllocProgress &&
-            need.data <= kNoAllocBytes - kNoAllocDataOff)
-            return kw;
+        if (fits(kw) && (left % kw == 0 || fits((int)(left % kw)))) return kw;
     }
     return 0;
 }
@@ -678,9 +709,8 @@ static int modify_noalloc(void *L, long long n, long long ld, const void *V, lon
     if (n > kNoAllocMaxN) return CHM_ERR_BUDGET;
     if (n == 0 || k == 0) return info_init(d_info, 1, stream);
     if ((rc = check_reachable(L)) != CHM_OK || (rc = check_reachable(V)) != CHM_OK) return rc;
-    const int kw = (int)std::min<long long>(k, kMaxWaves);
-    const bool team = use_team(n, kw, dtype);
-    const int kw_max = noalloc_vectors(n, kw, team);
+    const bool team = use_team(n, k, dtype);
+    const int kw_max = noalloc_vectors(n, k, team);
     if (kw_max < 1) return CHM_ERR_BUDGET;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return CHM_ERR_CUDA;

@@ -24,6 +24,16 @@ ScratchNeed team_need(const ProbShape *shapes, int count)
     return r;
 }
 
+ScratchNeed team_need_cap(const ProbShape &sh)
+{
+    ScratchNeed r;
+    const int nb = (int)((sh.n + kW - 1) / kW);
+    r.iflags = team::prob_flags(nb, sh.k);
+    r.progress = team::prob_tags(nb, sh.k);
+    r.data = team::prob_data_cap(nb, sh.k);
+    return r;
+}
+
 void team_carve(const ProbShape *shapes, int count, int dtype, const Scratch &sc, Prob *problems)
 {
     size_t fi = 0, fp = 0, fd = 0;

@@ -89,6 +89,29 @@ CHM_HD inline size_t prob_dcar(int nb, int k)
     return pass_data_off(nb, np - 1) + pass_rec(nb, k - (np - 1) * kTeamKb).bytes;
 }
 CHM_HD inline size_t prob_data(int nb, int k) { return align256(prob_dcar(nb, k) + (size_t)nb * kW * 8); }
+// A problem's data region is not the larger the larger n or k: a last pass of
+// two vectors can keep more segment starts than one of eight, and the segments
+// grow in steps with n.  A workspace that serves more than the one shape it was
+// sized for (a modification's launches of 64 vectors and of what is left, a
+// stream's later, smaller calls) is therefore sized by bounds that never
+// fall: at least the segment starts of every order up to this one,
+CHM_HD inline size_t bounds_cap(int nb, int KB)
+{
+    const int x = KB <= 2 ? nb / 2 : nb / 4, most = KB <= 2 ? 64 : 12;
+    return (size_t)(x < most ? x : most);
+}
+// and at least the data region of every problem of up to nb blocks and k vectors.
+CHM_HD inline size_t prob_data_cap(int nb, int k)
+{
+    const size_t rows = (size_t)nb * kW;
+    size_t pass = 0;
+    for (int KB = 1; KB <= kb_inst(k < kTeamKb ? k : kTeamKb); KB *= 2) {
+        const size_t snap = bounds_cap(nb, KB) * (rows * KB + KB * (KB + 1) / 2) * 8;
+        const size_t b = align256(rows * (3 * kW + 2 * KB + 2) * 8 + snap);
+        if (b > pass) pass = b;
+    }
+    return align256((size_t)passes_of(k) * pass + rows * 8);
+}
 // Int flags: per pass, U, G1, G2 and the coefficients published ([nb] each).
 CHM_HD inline size_t prob_flags(int nb, int k) { return ((size_t)passes_of(k) * 4 * nb + 63) & ~(size_t)63; }
 // Epoch-tagged 64-bit words: per pass P ([kb][nb][kW][2]) and the prefix
