@@ -320,7 +320,9 @@ int chm_server_destroy(void *srv);
  * same stream to solve with the modified factor).  Each 32 x 32 diagonal
  * block is applied through its explicit inverse.  If some L_ii <= 0 or is
  * not finite, the stream's status word records CHM_ERR_NOT_PD with that row
- * and X is unspecified.  Uses the stream's workspace (O(n) bytes).
+ * and X is unspecified.  Uses the stream's workspace: about 1.3 KB per row of L
+ * and 64 bytes per row and right-hand side of a launch (at most 64, above
+ * order 8192 at most 16), and at least what any smaller solve takes.
  * Returns CHM_OK, CHM_ERR_ARG, CHM_ERR_NOMEM or CHM_ERR_CUDA.
  */
 int chm_solve(const void *L, int64_t n, int64_t ld, void *B, int64_t ldb, int64_t nrhs, int dtype,

@@ -656,7 +656,8 @@ __global__ void __launch_bounds__(kThreads, R == 1 ? 3 : 2) solve_kernel(SolveAr
 // Right-hand sides of one launch, at most: 64 (their tagged words take
 // 2 KB per row block and right-hand side), 16 above order 8192, where 16
 // chains of one already keep the FP64 pipes busy.
-int solve_group(long long n) { return n > 8192 ? kSolveChains : kSolveChains * kSolveRhs; }
+constexpr long long kSolveWide = 8192;
+int solve_group(long long n) { return n > kSolveWide ? kSolveChains : kSolveChains * kSolveRhs; }
 // Right-hand sides per chain: one while the chains suffice for all (a step
 // is shortest then), else as few as do.
 int solve_rhs(int nr) { return nr <= kSolveChains ? 1 : nr <= 2 * kSolveChains ? 2 : kSolveRhs; }
@@ -734,14 +735,21 @@ int solve_all(const void *L, long long n, long long ld, void *B, long long ldb, 
 
 }  // namespace
 
+// What this solve takes or, where more, what a smaller one does: up to order
+// 8192 a launch holds four times the right-hand sides, so that the tagged words
+// of an order above it can be fewer (a stream's workspace, once it served a
+// solve, serves every smaller one without growing).
 ScratchNeed solve_need(long long n, long long nrhs)
 {
     const size_t nb = (size_t)((n + kW - 1) / kW);
-    const size_t nr = (size_t)std::min<long long>(std::max(1ll, nrhs), solve_group(n));
-    const size_t R = (size_t)solve_rhs((int)nr), cols = (nr + R - 1) / R * R;
+    auto tags = [&](long long m) {
+        const size_t nr = (size_t)std::min<long long>(std::max(1ll, nrhs), solve_group(m));
+        const size_t R = (size_t)solve_rhs((int)nr), cols = (nr + R - 1) / R * R;
+        return 2 * (size_t)((m + kW - 1) / kW) * kW * cols * 2;
+    };
     ScratchNeed need;
     need.iflags = (4 * nb + 63) & ~(size_t)63;
-    need.progress = 2 * nb * kW * cols * 2;
+    need.progress = std::max(tags(n), tags(std::min(n, kSolveWide)));
     need.data = nb * kPrepMats * kW * kW * sizeof(double);
     return need;
 }
