@@ -18,8 +18,9 @@
 //             The tiles above are summed as their p arrive, and what is left
 //             of v at the start of every sweep segment is kept.  After
 //             p_{b-1} there is one 32 x 32 product, eight FMAs a warp.
-//   COEF(b)   the prefix Grams of row block b's rows, their LDL^T and the
-//             rows' sweep coefficients
+//   COEF(b)   the prefix Grams of row block b's rows, their LDL^T (where that
+//             would cancel, factors carried from row to row) and the rows'
+//             sweep coefficients
 //   SWEEP(b, s) segments of column block b (`seg` row blocks each): the
 //             carries restart from the kept residual, and every tile is
 //             read, rotated and written once per pass
@@ -90,7 +91,8 @@ struct View {
     double *rst;         // [nbound][KB (KB + 1) / 2]: packed unit lower factor, 1 / |D_q| on the diagonal
     double *dcar;        // [nb * kW]: the diagonal, carried in double from pass to pass
     long long *ptag;     // [kb][nb][kW][2]
-    long long *htag;     // [nb][KB (KB + 1) / 2][2]
+    long long *htag;     // [nb][KB (KB + 1) / 2][2]: the Gram before block b + 1
+    long long *ftag;     // [nb][KB (KB + 1) / 2][2]: its factor, where the Gram is ill-conditioned (else infinity)
     int *uflag, *gflag, *g2flag, *cflag;  // [nb] each: U, G1, G2, coefficients published (== epoch)
     long long *sdone;    // [nb]: sweep tasks of a column finished, all passes (epoch-tagged count)
     SyncArgs sync;
@@ -120,6 +122,12 @@ struct CoefSmem {
     double g[8][ne];        // the Grams of the threads' shares of the rows
     double p[kW][kTeamKb + 1];
     double z[kW][kTeamKb + 1];
+    double p0[kW][kTeamKb + 1];  // p again (p becomes z = L^{-1} p)
+    double size[kTeamKb];        // the sizes of the Gram's diagonal behind the block
+    double l0[ne];               // the factor handed on by the block before, |D_q| on its diagonal
+    unsigned ill[kWarps];        // per warp: four bits a row, set where its Gram is ill-conditioned
+    double M[ne];                // from l0 on: the Gram behind the block, then its factor, |D_q| on the diagonal
+    int have;                    // a factor was handed on
 };
 // A sweep task's segments: NV warps pass a tile on, so NV + 1 tiles are in
 // flight per segment.
@@ -471,31 +479,204 @@ __device__ __forceinline__ double wait_one(const SyncArgs &sy, const long long *
     return x;
 }
 
+// Signs and comparisons on the integer pipe: an FP64 instruction takes its own
+// for 64 cycles.
+__device__ __forceinline__ double signed_by(double x, unsigned down) { return __hiloint2double(__double2hiint(x) ^ (int)(down << 31), __double2loint(x)); }
+__device__ __forceinline__ bool positive_finite(double x)
+{
+    const long long u = __double_as_longlong(x);
+    return u > 0 && u < 0x7ff0000000000000ll;
+}
+
+// A Gram is ill-conditioned if a pivot |D_q| is below this fraction of the
+// sums that it is left of, 1 + sum_i p_iq^2: subtracting costs the pivot that
+// factor in relative accuracy, so that three bits may go in double; in float,
+// whose coefficients are rounded to 24 bits, twenty of the Gram's 53.
+// Compared by the numbers' high words; a NaN is not found here, but as a row
+// that has failed.
+template <typename T>
+__device__ __forceinline__ bool ill_pivot(double ad, double size)
+{
+    constexpr int bits = sizeof(T) == 8 ? 3 : 20;
+    return __double2hiint(ad) < __double2hiint(size) - (bits << 20);
+}
+
+// The factor of an ill-conditioned Gram is not taken from the Gram, whose small
+// pivots are rounding errors (a factor 1e-4 I and eight vectors of size 1: the
+// result off by 1e-8).  A block whose first Gram is ill-conditioned starts
+// from the factor L0 D0 L0^T that the block before hands on, and sums the
+// Grams of L0^{-1} p on top of D0: only what these rows add counts there, so
+// that vectors which are large and alike all the way cost a chain of 2 to 9 us
+// a block (n = 5000, 2 / 8 vectors 0.79 / 1.94 ms instead of 0.44 / 0.95).
+// Where rows are still ill-conditioned (the first ones of an estimator that
+// starts from a small multiple of the identity) the factor is carried from row
+// to row, L D L^T + p p^T:
+//   z = L^{-1} p,  D~_q = D_q Dc_q / Dc_{q-1},  L~_iq = L_iq + sigma_q b_q w_iq,
+// w_iq what is left of p_i behind z_q.  These are the rotations that the sweep
+// applies, with the coefficients that it applies, so that the factor and the
+// carries stay consistent, as they do where vector after vector is rotated
+// (and as they do not with a Gram of more bits).  A serial chain of up to 40 FP64
+// instructions and two dozen shuffles a row, 2.9 us with eight vectors.
+// Lane i (one of eight; the others repeat them) holds row i.
+struct Carried {
+    double l[kTeamKb], ad;  // L_iq, |D_i|
+};
+__device__ __forceinline__ Carried carried_at(const CoefSmem &S, int row, int kb, unsigned down_mask)
+{
+    const int i = threadIdx.x & (kTeamKb - 1);
+    Carried c;
+    c.ad = 1.0;
+#pragma unroll
+    for (int q = 0; q < kTeamKb; ++q) c.l[q] = (i < kb && q < i) ? S.H[row][tri(i, q)] : 0.0;
+    if (i < kb) c.ad = signed_by(S.H[row][tri(i, i)], (down_mask >> i) & 1u);
+    return c;
+}
+// `c` is row `row`'s factor: its z and the terms of its Dc to S, and (`store`) itself; then the next row's.
+__device__ __forceinline__ void carry_row(CoefSmem &S, Carried &c, int row, int kb, unsigned down_mask, bool store)
+{
+    const int lane = threadIdx.x & 31, i = lane & (kTeamKb - 1);
+    const unsigned down = (down_mask >> i) & 1u;
+    double w = i < kb ? S.p0[row][i] : 0.0, wq[kTeamKb];
+#pragma unroll
+    for (int q = 0; q < kTeamKb; ++q) {
+        if (q < kb) {
+            const double zq = __shfl_sync(kFull, w, q);
+            if (q < i) w = fma(-zq, c.l[q], w);
+        }
+        wq[q] = w;
+    }
+    const double term = signed_by(w * w, down) * rcp_refined(c.ad);
+    double Dc = 1.0, before = 1.0;
+#pragma unroll
+    for (int q = 0; q < kTeamKb; ++q) {
+        if (q < kb) {
+            const double t = __shfl_sync(kFull, term, q);
+            if (q == i) before = Dc;
+            if (q <= i) Dc += t;
+        }
+    }
+    if (store && lane < kb) {
+#pragma unroll
+        for (int q = 0; q < kTeamKb; ++q)
+            if (q < i) S.H[row][tri(i, q)] = c.l[q];
+        S.H[row][tri(i, i)] = signed_by(c.ad, down);
+        S.p[row][i] = w;
+        S.z[row][i] = term;
+    }
+    const double b = signed_by(w * rcp_refined(c.ad * Dc), down);
+#pragma unroll
+    for (int q = 0; q < kTeamKb; ++q) {
+        if (q < kb) {
+            const double bq = __shfl_sync(kFull, b, q);
+            if (q < i) c.l[q] = fma(bq, wq[q], c.l[q]);
+        }
+    }
+    c.ad = c.ad * Dc * rcp_refined(before);
+}
+
+// One warp: rows first .. last are carried from row first's Gram on.
+__device__ __noinline__ void carry_rows(CoefSmem &S, int first, int last, int kb, unsigned down_mask)
+{
+    Carried c = carried_at(S, first, kb, down_mask);
+    __syncwarp();
+    for (int m = first; m <= last; ++m) carry_row(S, c, m, kb, down_mask, true);
+}
+// One warp: S.M becomes the factor behind the block, one row on from the last.
+__device__ __noinline__ void carry_end(CoefSmem &S, int kb, unsigned down_mask)
+{
+    const int lane = threadIdx.x & 31;
+    Carried c = carried_at(S, kW - 1, kb, down_mask);
+    carry_row(S, c, kW - 1, kb, down_mask, false);
+    if (lane < kb) {
+#pragma unroll
+        for (int q = 0; q < kTeamKb; ++q)
+            if (q < lane) S.M[tri(lane, q)] = c.l[q];
+        S.M[tri(lane, lane)] = c.ad;
+    }
+    __syncwarp();
+}
+// One warp: S.M, the Gram behind the block on top of D0, becomes its factor;
+// false if that is ill-conditioned.  Lane i (one of eight) holds row i.
+template <typename T>
+__device__ __noinline__ bool factor_end(CoefSmem &S, int kb, unsigned down_mask)
+{
+    const int lane = threadIdx.x & 31, i = lane & (kTeamKb - 1);
+    const unsigned down = (down_mask >> i) & 1u;
+    double a[kTeamKb];
+#pragma unroll
+    for (int m = 0; m < kTeamKb; ++m) a[m] = (i < kb && m <= i) ? S.M[tri(i, m)] : 0.0;
+    const double size = i < kb ? S.M[tri(i, i)] + (down ? 2.0 * S.l0[tri(i, i)] : 0.0) : 0.0;
+    double ad = 1.0;
+#pragma unroll
+    for (int j = 0; j < kTeamKb; ++j) {
+        if (j >= kb) continue;
+        if (i == j) ad = signed_by(a[j], down);
+        const double l = a[j] * rcp_refined(__shfl_sync(kFull, a[j], j));
+#pragma unroll
+        for (int m = j + 1; m < kTeamKb; ++m) {
+            if (m >= kb) continue;
+            const double x = __shfl_sync(kFull, a[j], m);
+            if (m <= i) a[m] = fma(-l, x, a[m]);
+        }
+        if (i > j) a[j] = l;
+    }
+    const bool ok = __all_sync(kFull, i >= kb || !ill_pivot<T>(ad, size)) != 0;
+    if (lane < kb) {
+#pragma unroll
+        for (int m = 0; m < kTeamKb; ++m)
+            if (m < i) S.M[tri(i, m)] = a[m];
+        S.M[tri(i, i)] = ad;
+    }
+    __syncwarp();
+    return ok;
+}
+// One warp: the factor L0 M (`handed`) or M to the next block.
+__device__ __noinline__ void put_factor(const CoefSmem &S, long long *w, int kb, int ne, bool handed, long long ep64)
+{
+    for (int e = threadIdx.x & 31; e < ne; e += 32) {
+        int i = 0;
+        while ((i + 1) * (i + 2) / 2 <= e) ++i;
+        const int j = e - i * (i + 1) / 2;
+        double f = i < kb ? S.M[e] : 0.0;
+        if (handed && j < i && i < kb) {
+            f += S.l0[e];
+            for (int m = j + 1; m < i; ++m) f = fma(S.l0[tri(i, m)], S.M[tri(m, j)], f);
+        }
+        put_tagged(w + 2 * e, f, ep64);
+    }
+}
+
 // Row r of the block: H_r = H_b + sum_{i<r} p_i p_i^T = L D L^T, z = L^{-1} p_r and,
 // with |D_q| = sigma_q D_q,
 //   Dc_q = 1 + sum_{q'<=q} sigma_q' z_q'^2 / |D_q'|,  a_q = sigma_q z_q,
 //   b_q = z_q / (|D_q| Dc_q),  e = Dc_kb^{-1/2},  the diagonal factor Dc_kb^{1/2}.
 // The Grams of the blocks form a chain (H_{b+1} = H_b + the block's Gram)
-// that is handed on before the factors are formed.  Four lanes share a row:
+// that is handed on before the factors are formed; where H_{b+1} is
+// ill-conditioned, its factor is handed on too (see Carried).  Four lanes share a row:
 // its factor's rows are dealt to them, so that a block of eight vectors
 // takes about 60 FP64 instructions a warp and step group instead of 250.
 template <typename T>
 __device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem &S)
 {
     const SyncArgs &sy = v.sync;
-    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long ep64 = (long long)sy.epoch << 32;
     const int kb = v.kb, KB = v.KB, ne = KB * (KB + 1) / 2;
     const long long r0 = (long long)b * kW;
     const int rows = (int)min((long long)kW, v.n - r0);
     for (int x = threadIdx.x; x < kW * kb; x += kThreads) {
         const int q = x / kW, i = x & (kW - 1);
-        S.p[i][q] = wait_one(sy, v.ptag + (((size_t)q * v.nb + b) * kW + i) * 2, ep64, b, false);
+        const double p = wait_one(sy, v.ptag + (((size_t)q * v.nb + b) * kW + i) * 2, ep64, b, false);
+        S.p[i][q] = p;
+        S.p0[i][q] = p;
     }
     __syncthreads();
     TEAM_TRACE(0, b, 5);
-    // the prefix Grams, entry x of the packed triangle: each of `ng` threads
-    // sums its share of the rows, then adds what comes before it
+    // rows threadIdx.x / 4; the four lanes of a row take the factor's rows i = sub, sub + 4, ...;
+    // row kb of the elimination is p itself, which becomes z
+    const int row = threadIdx.x >> 2, sub = threadIdx.x & 3;
+    double *h = S.H[row], *t = S.p[row];
+    // entry x of the packed triangle: each of `ng` threads sums its share of the rows
     const int ng = KB <= 4 ? 8 : 2, nr = kW / ng;
     const int x = threadIdx.x % ne, part = threadIdx.x / ne, i0 = part * nr;
     const bool mine = part < ng;
@@ -503,84 +684,155 @@ __device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem 
     while ((q + 1) * (q + 2) / 2 <= x) ++q;
     const int r = x - q * (q + 1) / 2;
     const bool in = mine && q < kb;
-    double acc = 0.0;
-    if (mine) {
+    bool handed = false;  // the block starts from a factor handed on, S.l0
+    bool early = false;   // (last warp) the next block has its factor
+    for (;;) {
+        // the prefix Grams: each thread's share, then what comes before it
+        double acc = 0.0;
+        if (mine) {
 #pragma unroll 4
-        for (int i = i0; i < i0 + nr; ++i) {
-            S.H[i][x] = acc;
-            if (in) acc = fma(S.p[i][q], S.p[i][r], acc);
+            for (int i = i0; i < i0 + nr; ++i) {
+                S.H[i][x] = acc;
+                if (in) acc = fma(S.p[i][q], S.p[i][r], acc);
+            }
+            S.g[part][x] = acc;
         }
-        S.g[part][x] = acc;
-    }
-    __syncthreads();
-    if (mine) {
-        double before = 0.0, all = 0.0;
-        for (int m = 0; m < ng; ++m) {
-            if (m == part) before = all;
-            all += S.g[m][x];
-        }
-        double h = (q == r) ? ((v.down_mask >> q) & 1u ? -1.0 : 1.0) : 0.0;
-        if (b > 0 && in) h = wait_one(sy, v.htag + ((size_t)(b - 1) * ne + x) * 2, ep64, b, true);
-        if (in && part == 0 && b + 1 < v.nb) put_tagged(v.htag + ((size_t)b * ne + x) * 2, h + all, ep64);
-        h += before;
-#pragma unroll 4
-        for (int i = i0; i < i0 + nr; ++i) S.H[i][x] += h;
-    }
-    __syncthreads();
-    // rows threadIdx.x / 4; the four lanes of a row take the factor's rows i = sub, sub + 4, ...;
-    // row kb of the elimination is p itself, which becomes z
-    const int row = threadIdx.x >> 2, sub = threadIdx.x & 3;
-    double *h = S.H[row], *t = S.p[row];
-    for (int j = 0; j < kb; ++j) {
-        const double id = rcp_refined(h[tri(j, j)]);
-        for (int i = sub; i <= kb; i += 4) {
-            if (i <= j) continue;
-            const double lij = (i == kb ? t[j] : h[tri(i, j)]) * id;
-            if (i == kb) {
-                for (int m = j + 1; m < kb; ++m) t[m] = fma(-lij, h[tri(m, j)], t[m]);
+        __syncthreads();
+        if (mine) {
+            double before = 0.0, all = 0.0;
+            for (int m = 0; m < ng; ++m) {
+                if (m == part) before = all;
+                all += S.g[m][x];
+            }
+            const bool down = (v.down_mask >> q) & 1u;
+            double h = (q == r) ? (down ? -1.0 : 1.0) : 0.0;
+            if (handed) {
+                if (in) h *= S.l0[x];
+                if (part == 0) S.M[x] = h + all;
             } else {
-                for (int m = j + 1; m <= i; ++m) h[tri(i, m)] = fma(-lij, h[tri(m, j)], h[tri(i, m)]);
+                if (b > 0 && in) h = wait_one(sy, v.htag + ((size_t)(b - 1) * ne + x) * 2, ep64, b, true);
+                if (in && part == 0 && b + 1 < v.nb) put_tagged(v.htag + ((size_t)b * ne + x) * 2, h + all, ep64);
+                if (in && part == 0 && q == r) S.size[q] = h + all + (down ? 2.0 : 0.0);
+            }
+            h += before;
+#pragma unroll 4
+            for (int i = i0; i < i0 + nr; ++i) S.H[i][x] += h;
+        }
+        __syncthreads();
+        // where the blocks' factors form a chain, the next block's goes first
+        if (handed && warp == kWarps - 1 && b + 1 < v.nb && factor_end<T>(S, kb, v.down_mask)) {
+            put_factor(S, v.ftag + (size_t)b * ne * 2, kb, ne, true, ep64);
+            early = true;
+        }
+        // the sizes of the diagonal's sums (the elimination's pivots q are this lane's own rows)
+        double size[kTeamKb / 4];
+#pragma unroll
+        for (int u = 0; u < kTeamKb / 4; ++u) {
+            const int q = sub + 4 * u;
+            size[u] = 0.0;
+            if (q < kb) size[u] = h[tri(q, q)] + ((v.down_mask >> q) & 1u ? 2.0 * (handed ? S.l0[tri(q, q)] : 1.0) : 0.0);
+        }
+        for (int j = 0; j < kb; ++j) {
+            const double id = rcp_refined(h[tri(j, j)]);
+            for (int i = sub; i <= kb; i += 4) {
+                if (i <= j) continue;
+                const double lij = (i == kb ? t[j] : h[tri(i, j)]) * id;
+                if (i == kb) {
+                    for (int m = j + 1; m < kb; ++m) t[m] = fma(-lij, h[tri(m, j)], t[m]);
+                } else {
+                    for (int m = j + 1; m <= i; ++m) h[tri(i, m)] = fma(-lij, h[tri(m, j)], h[tri(i, m)]);
+                }
+            }
+            __syncwarp();
+            for (int i = sub; i < kb; i += 4)
+                if (i > j) h[tri(i, j)] *= id;
+            __syncwarp();
+        }
+        // the terms of Dc, and which rows' Grams are ill-conditioned
+        bool ill = false;
+#pragma unroll
+        for (int u = 0; u < kTeamKb / 4; ++u) {
+            const int q = sub + 4 * u;
+            if (q >= kb) continue;
+            const unsigned down = (v.down_mask >> q) & 1u;
+            const double ad = signed_by(h[tri(q, q)], down);
+            ill = ill || ill_pivot<T>(ad, size[u]);
+            S.z[row][q] = signed_by(t[q] * t[q], down) * rcp_refined(ad);
+        }
+        const unsigned illm = __ballot_sync(kFull, ill && row < rows);
+        if (lane == 0) S.ill[warp] = illm;
+        __syncthreads();
+        if (handed || b == 0 || (S.ill[0] & 0xfu) == 0u) break;
+        if (warp == 0) {
+            // NaN: a row of the block before has failed, the rest is unspecified;
+            // infinity: it found its last pivots just large enough, so take the Gram
+            bool nan = false, inf = false;
+            for (int e = lane; e < ne; e += 32) {
+                const double f = wait_one(sy, v.ftag + ((size_t)(b - 1) * ne + e) * 2, ep64, b, true);
+                S.l0[e] = f;
+                nan = nan || f != f;
+                inf = inf || fabs(f) > DBL_MAX;
+            }
+            nan = __any_sync(kFull, nan);
+            inf = __any_sync(kFull, inf);
+            if (lane == 0) {
+                S.have = !nan && !inf;
+                if (inf && !nan) S.ill[0] &= ~0xfu;
             }
         }
-        __syncwarp();
-        for (int i = sub; i < kb; i += 4)
-            if (i > j) h[tri(i, j)] *= id;
-        __syncwarp();
-    }
-    // the terms of Dc and the inverses, then its prefix sums
-    bool bad = false;
-    for (int q = sub; q < kb; q += 4) {
-        const double sg = (v.down_mask >> q) & 1u ? -1.0 : 1.0;
-        const double ad = sg * h[tri(q, q)];
-        bad = bad || !(ad > 0.0 && ad <= DBL_MAX);
-        const double iad = rcp_refined(ad);
-        S.z[row][q] = sg * t[q] * t[q] * iad;
-        const int start = seg_at(b, v.seg);
-        if (row == 0 && start > 0 && start <= v.nbound) {
-            // a segment starts at this block: the factor of H_b for its carries
-            double *dst = v.rst + (size_t)(start - 1) * ne;
-            for (int m = 0; m < q; ++m) __stcg(dst + tri(q, m), h[tri(q, m)]);
-            __stcg(dst + tri(q, q), iad);
+        __syncthreads();
+        if (!S.have) break;
+        // p becomes L0^{-1} p
+        double *y = S.p0[row];
+        for (int j = 0; j + 1 < kb; ++j) {
+            for (int i = sub; i < kb; i += 4)
+                if (i > j) y[i] = fma(-S.l0[tri(i, j)], y[j], y[i]);
+            __syncwarp();
         }
+        for (int i = sub; i < kb; i += 4) t[i] = y[i];
+        handed = true;
+        __syncthreads();
     }
-    __syncwarp();
+    int first = kW, last = -1;
+#pragma unroll
+    for (int m = kWarps - 1; m >= 0; --m) {
+        if (!S.ill[m]) continue;
+        first = m * 8 + ((__ffs(S.ill[m]) - 1) >> 2);
+        last = max(last, m * 8 + ((31 - __clz(S.ill[m])) >> 2));
+    }
+    if (first > 0 && last >= 0) {
+        // (row 0 is ill-conditioned only behind a row that has failed)
+        if (warp == 0) carry_rows(S, first - 1, last, kb, v.down_mask);
+        __syncthreads();
+    }
+    // the prefix sums and the coefficients
+    bool bad = false, next = false;
+    const int start = seg_at(b, v.seg);
     double Dc = 1.0;
     T *cf = v.coef + (size_t)(r0 + row) * 2 * KB;
     for (int q = 0; q < KB; ++q) {
+        const double before = Dc;
         if (q < kb) {
             Dc += S.z[row][q];
-            bad = bad || !(Dc > 0.0 && Dc <= DBL_MAX);
+            bad = bad || !positive_finite(Dc);
         }
-        if ((q & 3) == sub && row < rows) {
-            if (q < kb) {
-                const double sg = (v.down_mask >> q) & 1u ? -1.0 : 1.0;
-                const double ad = sg * h[tri(q, q)];
-                cf[2 * q] = (T)(sg * t[q]);
-                cf[2 * q + 1] = (T)(t[q] * rcp_refined(ad * Dc));
-            } else {
-                cf[2 * q] = T(0);
-                cf[2 * q + 1] = T(0);
+        if ((q & 3) != sub || row >= rows) continue;
+        if (q < kb) {
+            const unsigned down = (v.down_mask >> q) & 1u;
+            const double ad = signed_by(h[tri(q, q)], down);
+            bad = bad || !positive_finite(ad);
+            cf[2 * q] = (T)signed_by(t[q], down);
+            cf[2 * q + 1] = (T)(t[q] * rcp_refined(ad * Dc));
+            next = next || (row == kW - 1 && ill_pivot<T>(ad * Dc, S.size[q] * before));
+            if (row == 0 && start > 0 && start <= v.nbound) {
+                // a segment starts at this block: the factor of H_b for its carries
+                double *dst = v.rst + (size_t)(start - 1) * ne;
+                for (int m = 0; m < q; ++m) __stcg(dst + tri(q, m), handed ? S.l0[tri(q, m)] : h[tri(q, m)]);
+                __stcg(dst + tri(q, q), rcp_refined(ad));
             }
+        } else {
+            cf[2 * q] = T(0);
+            cf[2 * q + 1] = T(0);
         }
     }
     if (sub == 0 && row < rows) {
@@ -591,9 +843,21 @@ __device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem 
     const unsigned badm = __ballot_sync(kFull, bad && row < rows);
     if (badm && lane == 0) record_error(sy, kStatusNotPD, r0 + ((threadIdx.x + __ffs(badm) - 1) >> 2));
     __threadfence();
-    __syncthreads();
+    const bool failed = __syncthreads_or(badm != 0u) != 0;
     if (threadIdx.x == 0) st_release_gpu(v.cflag + b, sy.epoch);
     TEAM_TRACE(0, b, 6);
+    if (warp == kWarps - 1 && b + 1 < v.nb && !early) {
+        // the next block's factor, if its Gram is ill-conditioned, else
+        // infinity, or NaN where a row has failed
+        long long *w = v.ftag + (size_t)b * ne * 2;
+        if (!failed && __any_sync(kFull, next)) {
+            carry_end(S, kb, v.down_mask);
+            put_factor(S, w, kb, ne, handed, ep64);
+        } else {
+            const double none = __longlong_as_double(failed ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
+            for (int e = lane; e < ne; e += 32) put_tagged(w + 2 * e, none, ep64);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- SWEEP
@@ -900,6 +1164,7 @@ __device__ bool set_view(const Launch<T> &P, int i, int s, int epoch, View<T> &v
     v.dcar = reinterpret_cast<double *>(pr.data + prob_dcar(nb, pr.k));
     v.ptag = pr.progress + pass_tag_off(nb, s);
     v.htag = v.ptag + (size_t)kb * nb * kW * 2;
+    v.ftag = v.htag + (size_t)nb * KB * (KB + 1);
     v.uflag = pr.iflags + (size_t)s * 4 * nb;
     v.gflag = v.uflag + nb;
     v.g2flag = v.gflag + nb;
@@ -918,8 +1183,8 @@ __device__ bool set_view(const Launch<T> &P, int i, int s, int epoch, View<T> &v
                       P.ws_progress_n * sizeof(long long)) &&
            CHK_REGION(v.sync, d, rc.bytes, pr.data, prob_data(nb, pr.k)) &&
            CHK_REGION(v.sync, v.dcar, (size_t)nb * kW * sizeof(double), pr.data, prob_data(nb, pr.k)) &&
-           CHK_REGION(v.sync, v.ptag, ((size_t)kb * nb * kW * 2 + (size_t)nb * KB * (KB + 1)) * sizeof(long long),
-                      pr.progress, prob_tags(nb, pr.k) * sizeof(long long)) &&
+           CHK_REGION(v.sync, v.ptag, pass_tags(nb, kb) * sizeof(long long), pr.progress,
+                      prob_tags(nb, pr.k) * sizeof(long long)) &&
            CHK_RECT(v.sync, (long long)s, (long long)passes_of(pr.k), 1, 1 << 30);
 #else
     return true;

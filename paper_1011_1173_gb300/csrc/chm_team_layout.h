@@ -114,14 +114,14 @@ CHM_HD inline size_t prob_data_cap(int nb, int k)
 }
 // Int flags: per pass, U, G1, G2 and the coefficients published ([nb] each).
 CHM_HD inline size_t prob_flags(int nb, int k) { return ((size_t)passes_of(k) * 4 * nb + 63) & ~(size_t)63; }
-// Epoch-tagged 64-bit words: per pass P ([kb][nb][kW][2]) and the prefix
-// Grams ([nb][KB (KB + 1) / 2][2]) as tagged doubles; then the problem's
-// ticket word and, per column block, the count of its segments swept
-// ((epoch << 32) + count each).
+// Epoch-tagged 64-bit words: per pass P ([kb][nb][kW][2]), the prefix Grams
+// and the factors handed on in their place ([nb][KB (KB + 1) / 2][2] each) as
+// tagged doubles; then the problem's ticket word and, per column block, the
+// count of its segments swept ((epoch << 32) + count each).
 CHM_HD inline size_t pass_tags(int nb, int kb)
 {
     const int KB = kb_inst(kb);
-    return (size_t)kb * nb * kW * 2 + (size_t)nb * KB * (KB + 1);
+    return (size_t)kb * nb * kW * 2 + 2 * (size_t)nb * KB * (KB + 1);
 }
 CHM_HD inline size_t pass_tag_off(int nb, int s) { return (size_t)s * pass_tags(nb, kTeamKb); }
 CHM_HD inline size_t prob_ticket(int nb, int k)
