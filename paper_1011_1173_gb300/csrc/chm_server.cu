@@ -324,7 +324,7 @@ int create(size_t budget, int dtype, int max_inflight, Server **out)
     for (int i = 0; i < s->nslots && rc == CHM_OK; ++i) {
         Slot &sl = s->slots[i];
         // flag and tagged-word regions in proportion to the data region: per
-        // 32 columns and pass of 8 vectors, 20 KB of data or more against 2
+        // 32 columns and pass of 8 vectors, 20 KB of data or more against 5
         // int flags and 656 tagged words
         const size_t iflags = per / 4096, progress = per / 40;
         const size_t data = per - iflags * sizeof(int) - progress * sizeof(long long);

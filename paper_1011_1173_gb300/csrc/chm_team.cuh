@@ -11,7 +11,9 @@
 // waits only on tasks before it, so that a launch of any number of resident
 // blocks progresses.  Blocks take a factor's tasks from its ticket word; a
 // factor is worked on by a team of blocks, and the launch holds G teams.
-//   PREP(b)   U_b = D_b^{-1} and G1_b = U_b^T F_{b-1,b}^T of diagonal block b
+//   PREP(b)   U_b = D_b^{-1} and G1_b = U_b^T F_{b-1,b}^T of diagonal block b,
+//             and whether D_b is so ill-conditioned that SUB substitutes
+//             through it instead (see is_hard)
 //   PREP2(b)  G2_b = U_b^T F_{b-2,b}^T
 //   SUB(c, b) step b of the forward substitution of vector c:
 //               p_b = U_b^T (v_b - sum_{r<=b-3} F_{r,b}^T p_r) - G2_b p_{b-2} - G1_b p_{b-1}.
@@ -94,6 +96,7 @@ struct View {
     long long *htag;     // [nb][KB (KB + 1) / 2][2]: the Gram before block b + 1
     long long *ftag;     // [nb][KB (KB + 1) / 2][2]: its factor, where the Gram is ill-conditioned (else infinity)
     int *uflag, *gflag, *g2flag, *cflag;  // [nb] each: U, G1, G2, coefficients published (== epoch)
+    int *hflag;          // [nb]: whether block b is multiplied by U (epoch) or substituted (-epoch)
     long long *sdone;    // [nb]: sweep tasks of a column finished, all passes (epoch-tagged count)
     SyncArgs sync;
 };
@@ -191,7 +194,42 @@ __device__ __forceinline__ void load_above(const View<T> &v, int b, int up, Prep
         S.F[i][j] = (j < nc && CHK_TRI(v.sync, o, v.n, v.ld)) ? (double)__ldcg(v.L + o) : 0.0;
     }
 }
-// U_b and G1_b.
+// The size of x in units of 2^e, e the exponent in the high word e0 (`inverse`:
+// of 2^-e), to 20 bits on the integer pipe; beyond float's range 0 or its largest.
+__device__ __forceinline__ float coarse(double x, int e0, bool inverse)
+{
+    const int e = e0 & 0x7ff00000, h = __double2hiint(x) & 0x7fffffff;
+    const int u = inverse ? min(h - 0x77f00000, 0x000fffff) + e : min(h - e, 0x10000000) + 0x07f00000;
+    return __int_as_float(min(max(u, 0), 0x0fefffff) << 3);
+}
+// Whether p = U^T r would be less accurate than substituting through D: the
+// product's residual D^T p - r is up to kappa = max_i sum_l (|D^T| |U^T|)_il
+// roundings of |D^T| |p|, the substitution's one or two whatever D is.  kappa
+// is 3 to 50 for the blocks of well-conditioned factors, where both leave the
+// same error; from about 100 on the factor's error grows with it (smooth rows
+// over a diagonal of 1e-4: kappa 900, 2e-13 instead of 9e-15).  Uses S.M.
+__device__ __forceinline__ bool is_hard(PrepSmem &S)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float(*part)[kW] = reinterpret_cast<float(*)[kW]>(&S.M[0][0]);
+    const int e0 = __double2hiint(S.D[0][0]);
+    float s = 0.0f;
+#pragma unroll
+    for (int m = 0; m < kPer; ++m) s += coarse(S.U[warp * kPer + m][lane], e0, true);
+    part[warp][lane] = s;
+    __syncthreads();
+    const float g = (part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]);
+    s = 0.0f;
+#pragma unroll
+    for (int m = 0; m < kPer; ++m)
+        s = fmaf(coarse(S.D[warp * kPer + m][lane], e0, false), __shfl_sync(kFull, g, warp * kPer + m), s);
+    part[kWarps + warp][lane] = s;
+    __syncthreads();
+    const float kappa = (part[4][lane] + part[5][lane]) + (part[6][lane] + part[7][lane]);
+    return __any_sync(kFull, !(kappa <= 64.0f)) != 0;
+}
+// U_b and G1_b, then the block's kind, which nothing waits for before its far
+// tiles are summed.
 template <typename T>
 __device__ void prep_task(const Launch<T> &P, const View<T> &v, int b, PrepSmem &S)
 {
@@ -237,6 +275,8 @@ __device__ void prep_task(const Launch<T> &P, const View<T> &v, int b, PrepSmem 
         form_g(S, ug + kW * kW);
         publish(v.gflag + b, sy.epoch);
     }
+    const bool hard = is_hard(S);
+    if (tid == 0) st_release_gpu(v.hflag + b, hard ? -sy.epoch : sy.epoch);
 }
 
 // G2_b, from PREP(b)'s U_b.
@@ -301,6 +341,77 @@ __device__ __forceinline__ void put_y(double *y, double x, float)
     *reinterpret_cast<float2 *>(y) = make_float2(hi, (float)(x - (double)hi));
 }
 
+// What is left of SUB(c, b) where block b is substituted; false if it turns
+// out not to be (`kind`: an early look at hflag, which is waited for here).
+// `rv` is what the far tiles left of v: the two tiles next to the block come
+// off it as they are, then D^T p = rv goes one row at a time.  32 FMAs in a
+// row instead of eight, and nothing taken beforehand: n = 5000 with every block
+// like this, one vector 0.77 instead of 0.38 ms, 16 vectors 1.90 instead of 1.69.
+template <typename T>
+__device__ __noinline__ bool sub_hard(const Launch<T> &P, const View<T> &v, int c, int b, double rv, int kind, SubSmem<T> &S)
+{
+    const SyncArgs &sy = v.sync;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long n = v.n, ld = v.ld, c0 = (long long)b * kW;
+    const int nc = (int)min((long long)kW, n - c0);
+    const long long ep64 = (long long)sy.epoch << 32;
+    long long *ptag = v.ptag + (size_t)c * v.nb * kW * 2;
+    const long long t0 = global_ns();
+    for (unsigned it = 1; !__all_sync(kFull, kind == sy.epoch || kind == -sy.epoch); ++it) {
+        if ((it & 31u) == 0u) {
+            const bool late = global_ns() - t0 > sy.timeout_ns || it > (1u << 28);
+            if (__any_sync(kFull, late || aborted(sy))) {
+                if (lane == 0 && late) record_error(sy, kStatusTimeout, b);
+                break;
+            }
+        }
+        kind = ld_relaxed_gpu(v.hflag + b);
+    }
+    // (every warp decides the same, but for one that gave up, whose way has as many barriers)
+    if (!__any_sync(kFull, kind == -sy.epoch)) return false;
+    // dr[i kW + j] = D_ij / D_ii above the diagonal, 1 / D_ii on it (the tiles are done with)
+    double *const dr = reinterpret_cast<double *>(&S.tile[1][0][0]);
+    const long long o = c0 + lane + c0 * ld;
+    double d = 1.0;
+    if (lane < nc && v.pass > 0) d = __ldcg(v.dcar + c0 + lane);
+    else if (lane < nc && CHK_TRI(sy, o + lane * ld, n, ld)) d = (double)__ldcg(v.L + o + lane * ld);
+    const double rd = rcp_refined(d);
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+        const int j = warp + x * kWarps;
+        double f = lane == j ? rd : 0.0;
+        if (lane < j && j < nc && CHK_TRI(sy, o + j * ld, n, ld)) f = (double)__ldcg(v.L + o + j * ld) * rd;
+        dr[lane * kW + j] = f;
+    }
+    // this warp's rows of the two tiles
+    double x = warp == 0 ? rv : 0.0;
+    for (int up = 2; up >= 1; --up) {
+        if (b < up) continue;
+        const long long r0 = c0 - up * kW + warp * kPer + (c0 + lane) * ld;
+        double f[kPer];
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj)
+            f[jj] = (lane < nc && CHK_TRI(sy, r0 + jj, n, ld)) ? (double)__ldcg(v.L + r0 + jj) : 0.0;
+        const double y = wait_p(sy, ptag + ((size_t)(b - up) * kW + warp * kPer + (lane & (kPer - 1))) * 2, nullptr, ep64, b);
+#pragma unroll
+        for (int jj = 0; jj < kPer; ++jj) x = fma(-f[jj], __shfl_sync(kFull, y, jj), x);
+    }
+    double(*sum)[kW] = reinterpret_cast<double(*)[kW]>(&S.tile[0][0][0]);
+    sum[warp][lane] = x;
+    __syncthreads();
+    if (warp == 0 && !(c == 0 && b == P.skip_publish)) {
+        x = (sum[0][lane] + sum[1][lane]) + (sum[2][lane] + sum[3][lane]);
+#pragma unroll 4
+        for (int i = 0; i < kW; ++i) {
+            const double xi = __shfl_sync(kFull, x, i);
+            if (lane > i) x = fma(-dr[i * kW + lane], xi, x);
+        }
+        x *= dr[lane * kW + lane];
+        put_tagged(ptag + ((size_t)b * kW + lane) * 2, lane < nc ? x : 0.0, ep64);
+    }
+    return true;
+}
+
 template <typename T>
 __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, SubSmem<T> &S)
 {
@@ -336,6 +447,7 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
     wait_flags(sy, v.uflag, b, b, b);
     if (b >= 1) wait_flags(sy, v.gflag, b, b, b);
     if (b >= 2) wait_flags(sy, v.g2flag, b, b, b);
+    int kind = ld_relaxed_gpu(v.hflag + b);
     double g1[kPer], g2[kPer];
 #pragma unroll
     for (int jj = 0; jj < kPer; ++jj) {
@@ -443,6 +555,7 @@ __device__ void sub_task(const Launch<T> &P, const View<T> &v, int c, int b, Sub
         __stcg(v.snap + ((size_t)(next - 1) * v.nb * kW + c0 + lane) * v.KB + c, (T)rv);
         __threadfence();
     }
+    if (!__all_sync(kFull, kind == sy.epoch) && sub_hard(P, v, c, b, rv, kind, S)) return;
     if (b >= 2) {
         if (!__all_sync(kFull, have2)) y2 = wait_p(sy, tag_of(2), nullptr, ep64, b);
 #pragma unroll
@@ -1165,10 +1278,11 @@ __device__ bool set_view(const Launch<T> &P, int i, int s, int epoch, View<T> &v
     v.ptag = pr.progress + pass_tag_off(nb, s);
     v.htag = v.ptag + (size_t)kb * nb * kW * 2;
     v.ftag = v.htag + (size_t)nb * KB * (KB + 1);
-    v.uflag = pr.iflags + (size_t)s * 4 * nb;
+    v.uflag = pr.iflags + (size_t)s * kPassFlags * nb;
     v.gflag = v.uflag + nb;
     v.g2flag = v.gflag + nb;
     v.cflag = v.g2flag + nb;
+    v.hflag = v.cflag + nb;
     v.sdone = pr.progress + prob_ticket(nb, pr.k) + 1;
     v.sync.abort_flag = P.ctl + kCtlAbort;
     v.sync.status = P.status;

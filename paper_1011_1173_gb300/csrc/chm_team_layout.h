@@ -112,8 +112,9 @@ CHM_HD inline size_t prob_data_cap(int nb, int k)
     }
     return align256((size_t)passes_of(k) * pass + rows * 8);
 }
-// Int flags: per pass, U, G1, G2 and the coefficients published ([nb] each).
-CHM_HD inline size_t prob_flags(int nb, int k) { return ((size_t)passes_of(k) * 4 * nb + 63) & ~(size_t)63; }
+// Int flags: per pass, U, G1, G2, a block's kind and the coefficients published ([nb] each).
+constexpr int kPassFlags = 5;
+CHM_HD inline size_t prob_flags(int nb, int k) { return ((size_t)passes_of(k) * kPassFlags * nb + 63) & ~(size_t)63; }
 // Epoch-tagged 64-bit words: per pass P ([kb][nb][kW][2]), the prefix Grams
 // and the factors handed on in their place ([nb][KB (KB + 1) / 2][2] each) as
 // tagged doubles; then the problem's ticket word and, per column block, the
