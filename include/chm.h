@@ -315,13 +315,14 @@ int chm_server_destroy(void *srv);
  *   nrhs   number of right-hand sides, nrhs >= 0 (0 is a no-op)
  *   dtype  CHM_F64: double L and B, double arithmetic.  CHM_F32_MIXED: float
  *          L and B, every product and sum in double or (the sums of a 32 x 32
- *          tile, kept in three floats) closer, X rounded to float once
+ *          tile, in three floats where their range holds all that counts) closer,
+ *          X rounded to float once
  * Stream-ordered like chm_update (enqueue it after a modification on the
  * same stream to solve with the modified factor).  Each 32 x 32 diagonal
  * block is applied through its explicit inverse.  If some L_ii <= 0 or is
  * not finite, the stream's status word records CHM_ERR_NOT_PD with that row
  * and X is unspecified.  Uses the stream's workspace: about 1.3 KB per row of L
- * and 64 bytes per row and right-hand side of a launch (at most 64, above
+ * and 32 bytes per row and right-hand side of a launch (at most 64, above
  * order 8192 at most 16), and at least what any smaller solve takes.
  * Returns CHM_OK, CHM_ERR_ARG, CHM_ERR_NOMEM or CHM_ERR_CUDA.
  */

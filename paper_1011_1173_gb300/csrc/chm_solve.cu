@@ -255,14 +255,24 @@ __device__ __forceinline__ void tile_sum(const double (&t)[kW], const double (&v
 }
 // For a factor in float: a conversion is as slow as an FMA in double (64
 // cycles a warp instruction), and together they bound every solve but the
-// smallest.  The values are scaled by a power of two to below 2^-5 (whatever
-// their range, no product with the factor's entries overflows) and split into
-// three floats that hold all of their 53 bits; the products are split exactly,
-// and the tile's sum is kept in three floats, two of them added to exactly
+// smallest.  The values are scaled by a power of two to below 2^-5 (so that
+// no sum of products with the factor's entries overflows) and split into three
+// floats that hold all of their 53 bits; the products are split exactly, and
+// the tile's sum is kept in three floats, two of them added to exactly
 // (two-sum): to about 2^-70 of the sum of its terms' sizes, against 2^-50 in double.  The
-// tiles' sums are added up in double.  A tile costs 1060 FP32 and 15 FP64
-// instructions a right-hand side instead of 64 FP64 ones: n = 16384, 1 / 5 / 8
-// right-hand sides 1.65 / 2.75 / 3.92 ms against 2.18 / 5.96 / 8.96.
+// tiles' sums are added up in double.  A tile costs 1090 FP32 and 15 FP64
+// instructions a right-hand side instead of 64 FP64 ones: n = 16384, 1 / 8
+// right-hand sides 1.70 / 4.11 ms against 2.18 / 8.96.
+//
+// What a float cannot hold is lost below 2^-150: of each value, so 2^-145 max
+// |t| of the sum, and of each product's parts, 2^-143.  A double sum is off by
+// 2^-53 of its largest term or more, which is at least the smallest value
+// (that is not zero) times max |t| (over those).  Where that is not above
+// 2^-88 or the smallest value not above 2^-90 (values or entries that differ by
+// tens of orders of magnitude, entries next to a float's smallest), and where a
+// value is not finite, the warp sums the tile in double (n = 16384 with columns
+// between 1e-18 and 1e18: 1.88 / 6.78 ms).  The test costs 3 to 5 % where the
+// FP32 rate binds.
 __device__ __forceinline__ void two_sum(float &s, float x, float &err)
 {
     const float u = __fadd_rn(s, x), b = __fsub_rn(u, s);
@@ -274,19 +284,46 @@ __device__ __forceinline__ void tile_sum(const float (&t)[kW], const double (&v)
                                          double (&acc)[R])
 {
     double up[R];
+    bool plain = false;  // the tile is summed in double
+    // (four entries are large enough nearly always)
+    const float four = fmaxf(fmaxf(fabsf(t[0]), fabsf(t[9])), fmaxf(fabsf(t[18]), fabsf(t[27])));
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        // the largest value's exponent, kept where both powers of two are finite
-        const unsigned top = __reduce_max_sync(kFull, (unsigned)__double2hiint(v[r]) & 0x7fffffffu) >> 20;
-        const int ex = min(max((int)top, 64), 2000);
+        // the largest value's exponent, kept where both powers of two are finite, and the smallest's
+        const unsigned hi = (unsigned)__double2hiint(v[r]) & 0x7fffffffu;
+        const bool some = (hi | (unsigned)__double2loint(v[r])) != 0u;
+        const int top = (int)(__reduce_max_sync(kFull, hi) >> 20), ex = min(max(top, 64), 2000);
+        const int low = (int)(__reduce_min_sync(kFull, some ? hi : 0x7fffffffu) >> 20) - ex - 6;
+        auto above = [&](float m) { return low >= -90 && (__float_as_int(m) >> 23) - 127 + low >= -88; };
+        const unsigned which = __ballot_sync(kFull, some);
+        if (top == 0x7ff || which != kFull || !__all_sync(kFull, above(four))) {
+            float m = 0.0f;
+#pragma unroll
+            for (int j = 0; j < kW; ++j)
+                if (which >> j & 1u) m = fmaxf(m, fabsf(t[j]));
+            if (top == 0x7ff || !__all_sync(kFull, m == 0.0f || above(m))) plain = true;
+        }
         up[r] = __hiloint2double((ex + 6) << 20, 0);
         double x = v[r] * __hiloint2double((2040 - ex) << 20, 0);
         const float h = (float)x;
         x -= (double)h;
-        const float m = (float)x;
-        *reinterpret_cast<float4 *>(y[r][lane]) = make_float4(h, m, (float)(x - (double)m), 0.0f);
+        const float l = (float)x;
+        *reinterpret_cast<float4 *>(y[r][lane]) = make_float4(h, l, (float)(x - (double)l), 0.0f);
     }
     __syncwarp();
+    if (plain) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) y[r][lane][0] = v[r];
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < kW; ++j) {
+            const double f = (double)t[j];
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = fma(f, y[r][j][0], acc[r]);
+        }
+        __syncwarp();
+        return;
+    }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         float s = 0.0f, e = 0.0f, l = 0.0f;
