@@ -27,28 +27,33 @@ struct PrepSmem {
 // Stage the 32 x 32 tile at row r0, column c0 into dst[column][Stride], read
 // through L2 (an earlier pass of the launch may have written it on another
 // SM): 16-byte asynchronous copies if `vec`, else loads of one element,
-// eight in flight per lane (a 4-byte cp.async would go through L1).  `diag`:
-// the diagonal tile, rows <= column only; the rest is zero.
-template <typename T>
-__device__ __forceinline__ void stage_tile(const SyncArgs &sy, T *dst, const T *L, long long ld, long long r0,
-                                           long long c0, long long n, bool vec, bool diag, int lane)
+// sixteen in flight per lane (a 4- or 8-byte cp.async would go through L1; with
+// eight a substitution step's tiles take 5 % longer).  `diag`: the diagonal
+// tile, rows <= column only; the rest is zero.  stage_columns: the columns
+// first .. last - 1, N loads in flight.
+template <int N, typename T>
+__device__ __forceinline__ void stage_columns(const SyncArgs &sy, T *dst, const T *L, long long ld, long long r0,
+                                              long long c0, long long n, bool diag, int lane, int first, int last)
 {
     constexpr int SD = pass::Stride<T>::value;
-    if (vec) {
-        pass::stage_tile(sy, dst, L, ld, r0, c0, n, kW, true, lane);
-        return;
-    }
 #pragma unroll 1
-    for (int c = 0; c < kW; c += 8) {
-        T x[8];
+    for (int c = first; c < last; c += N) {
+        T x[N];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < N; ++i) {
             const long long o = (r0 + lane) + (c0 + c + i) * ld;
             x[i] = (c0 + c + i < n && (!diag || lane <= c + i) && CHK_TRI(sy, o, n, ld)) ? __ldcg(L + o) : T(0);
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) dst[(c + i) * SD + lane] = x[i];
+        for (int i = 0; i < N; ++i) dst[(c + i) * SD + lane] = x[i];
     }
+}
+template <typename T>
+__device__ __forceinline__ void stage_tile(const SyncArgs &sy, T *dst, const T *L, long long ld, long long r0,
+                                           long long c0, long long n, bool vec, bool diag, int lane)
+{
+    if (vec) pass::stage_tile(sy, dst, L, ld, r0, c0, n, kW, true, lane);
+    else stage_columns<16>(sy, dst, L, ld, r0, c0, n, diag, lane, 0, kW);
 }
 
 // S.U = S.D^{-1}, upper triangular, with `d` the diagonal to use (lane = row,

@@ -1070,8 +1070,8 @@ __device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task
                     for (int w = 0; w < E; ++w) d[w] = T(0);
                 }
             }
-        } else if (part == 0) {
-            stage_tile(sy, tl, v.L, ld, r0, c0, n, false, r == j, lane);
+        } else {
+            stage_columns<8>(sy, tl, v.L, ld, r0, c0, n, r == j, lane, part * (kW / NV), (part + 1) * (kW / NV));
         }
         const T *cf = v.coef + (size_t)r0 * 2 * KB;
         for (int x = part * 32 + lane; x < kW * 2 * KB / E; x += NV * 32) pass::cp16(U.cf[slot] + x * E, cf + x * E);
@@ -1202,16 +1202,28 @@ __device__ void sweep_task(const Launch<T> &P, const View<T> &v, int j, int task
                                 __stcg(v.L + r0 + i0 + w + (c0 + lane) * ld,
                                        tl[lane * SD + i0 + w] * (scale && i0 + w < lane ? er[i0 + w] : T(1)));
                     }
-                } else {
-#pragma unroll 8
-                    for (int cc = 0; cc < kW; ++cc)
-                        if (c0 + cc < n && (!diag || lane <= cc) && CHK_TRI(sy, (r0 + lane) + (c0 + cc) * ld, n, ld))
-                            __stcg(v.L + (r0 + lane) + (c0 + cc) * ld,
-                                   tl[cc * SD + lane] * (scale && (!diag || lane < cc) ? er[lane] : T(1)));
                 }
             }
         }
         unit_sync<NV>(unit);  // the next step's copies may take the slot of the tile that left
+        const int left = i - (NV - 1);
+        if (!v.vec && left >= 0) {
+            // (or, where columns do not start on 16 bytes, the segment's warps
+            // store it first, each its share, as they fetched it: one warp for
+            // either kept the others waiting, n = 6001 with 64 vectors 10.3 ms
+            // instead of 9.05, n = 511 1.20 instead of 1.03)
+            const int r = rb + left, slot = left % NS;
+            const bool diag = r == j;
+            const long long r0 = (long long)r * kW;
+            const T *tl = U.tile[slot], e = NR < NV ? U.e[slot][lane] : T(1);
+#pragma unroll
+            for (int x = 0; x < kW / NV; ++x) {
+                const int cc = part * (kW / NV) + x;
+                if (c0 + cc < n && (!diag || lane <= cc) && CHK_TRI(sy, (r0 + lane) + (c0 + cc) * ld, n, ld))
+                    __stcg(v.L + (r0 + lane) + (c0 + cc) * ld, tl[cc * SD + lane] * (diag && lane == cc ? T(1) : e));
+            }
+            unit_sync<NV>(unit);
+        }
     }
     pass::cp_wait<0>();
     if (P.trace && last && part == 0 && lane == 0)
