@@ -1,4 +1,4 @@
-// Batched up/downdate: many independent factors in one launch of the wave
+// Batched up/downdate: many independent factors in one launch of the team
 // kernel, replayed from a CUDA graph, with a launch configuration chosen by
 // an autotuner that times candidate configurations on synthetic factors of
 // the plan's shapes.
@@ -29,6 +29,7 @@ struct Plan {
     // problems with work, in launch order: order[p] = caller's factor index
     std::vector<int> order;
     bool lpt = true;  // launch order: largest work first (else caller's order)
+    bool wave = false;  // the one problem runs on the wave kernel
     long long ntasks = 0;
     std::vector<Prob> tmpl;  // carved records without L and V
     Scratch sc;
@@ -45,6 +46,22 @@ struct Plan {
 };
 
 size_t elt_size(int dtype) { return dtype == CHM_F64 ? 8 : 4; }
+
+// A plan of one factor in double that a single modification would give to the
+// wave kernel goes there too (batch of one, team / wave: n = 8192 k = 64 14.7 /
+// 13.9 ms, n = 12000 k = 16 7.9 / 7.7, n = 16384 k = 64 54.9 / 49.0).  From two
+// factors on the team kernel is ahead everywhere (n = 8192 k = 64, four factors
+// 52.7 / 59.1; n = 12000 k = 16, three 20.8 / 24.7; n = 20000 k = 16, two 37.7 /
+// 42.9), and in float with one as well (n = 8200 k = 1 0.48 / 1.54; n = 16384
+// k = 64 19.2 / 29.5).
+bool wave_plan(const std::vector<ProbShape> &shapes, int dtype)
+{
+    return dtype == CHM_F64 && shapes.size() == 1 && !use_team(shapes[0].n, shapes[0].k, dtype);
+}
+int plan_occupancy(const Plan *p, int *occ)
+{
+    return p->wave ? wave_occupancy(p->dtype, p->device, occ) : team_occupancy(p->dtype, p->device, occ);
+}
 
 // Launch order and carved records for the plan's current ordering.
 int relayout(Plan *p)
@@ -64,7 +81,8 @@ int relayout(Plan *p)
     p->tmpl.assign(act.size(), Prob());
     for (Prob &pr : p->tmpl) memset(&pr, 0, sizeof(pr));
     if (act.empty()) return CHM_OK;
-    team_carve(shapes.data(), (int)shapes.size(), p->dtype, p->sc, p->tmpl.data());
+    if (p->wave) carve(shapes.data(), 1, p->sc, p->tmpl.data());
+    else team_carve(shapes.data(), (int)shapes.size(), p->dtype, p->sc, p->tmpl.data());
     for (size_t q = 0; q < act.size(); ++q) {
         const int i = act[q];
         Prob &pr = p->tmpl[q];
@@ -124,7 +142,10 @@ int capture(Plan *p, int s)
     if (cudaMemcpyAsync(p->d_probs, p->h_probs[s], np * sizeof(Prob), cudaMemcpyHostToDevice, cs) != cudaSuccess)
         rc = CHM_ERR_CUDA;
     if (rc == CHM_OK) rc = info_init(p->d_info, p->count, cs);
-    if (rc == CHM_OK)
+    if (rc == CHM_OK && p->wave)
+        rc = launch_wave(p->dtype, nullptr, p->d_probs, nullptr, 1, p->tmpl[0].k + 1, p->tmpl[0].nb, p->sc, p->cfg,
+                         nullptr, cs);
+    else if (rc == CHM_OK)
         rc = launch_team(p->dtype, nullptr, p->d_probs, (int)np, p->ntasks, p->sc, p->cfg, nullptr, cs);
     const cudaError_t ec = cudaStreamEndCapture(cs, &g);
     if (rc == CHM_OK && ec != cudaSuccess) rc = CHM_ERR_CUDA;
@@ -259,11 +280,13 @@ int autotune(Plan *p, cudaStream_t stream)
     if (rc != CHM_OK) return rc;
     const int nsm = sm_count(p->device);
     int occ = 0;
-    rc = team_occupancy(p->dtype, p->device, &occ);
+    rc = plan_occupancy(p, &occ);
     if (rc != CHM_OK) return rc;
     std::vector<int> groups;
     for (int d : {24, 16, 12, 8, 6, 4, 3, 2, 1}) {
-        const int g = std::max(1, std::min(std::min((int)p->order.size(), kMaxTeams), nsm * occ / d));
+        // (the wave kernel: SM groups, each a wave at a time; else teams of blocks)
+        const int g = p->wave ? std::max(1, std::min(std::min(p->tmpl[0].k + 1, kMaxGroups), nsm / std::max(2, d)))
+                              : std::max(1, std::min(std::min((int)p->order.size(), kMaxTeams), nsm * occ / d));
         if (std::find(groups.begin(), groups.end(), g) == groups.end()) groups.push_back(g);
     }
     const LaunchCfg keep = p->cfg;
@@ -334,7 +357,9 @@ int chm_batch_plan_create(int count, const int64_t *n, const int64_t *ld, const 
         p->sign[i] = sigma ? sigma[i] : 1;
         if (n[i] > 0 && k[i] > 0) shapes.push_back(ProbShape{n[i], (int)k[i]});
     }
-    const ScratchNeed need = team_need(shapes.data(), (int)shapes.size());
+    p->wave = wave_plan(shapes, dtype);
+    const ScratchNeed need =
+        p->wave ? scratch_need(shapes.data(), 1) : team_need(shapes.data(), (int)shapes.size());
     int rc = CHM_OK;
     if (cudaMalloc(&p->d_info, 2 * sizeof(long long) * std::max(1, count)) != cudaSuccess) rc = CHM_ERR_NOMEM;
     if (rc == CHM_OK && cudaMalloc(&p->d_probs, sizeof(Prob) * std::max<size_t>(1, shapes.size())) != cudaSuccess)
@@ -350,7 +375,7 @@ int chm_batch_plan_create(int count, const int64_t *n, const int64_t *ld, const 
     if (rc == CHM_OK) rc = relayout(p);
     // the kernel's one-time set-up happens here, outside any stream capture
     int occ = 0;
-    if (rc == CHM_OK) rc = team_occupancy(dtype, p->device, &occ);
+    if (rc == CHM_OK) rc = plan_occupancy(p, &occ);
     if (rc == CHM_OK) rc = info_init(p->d_info, count, nullptr);
     if (rc == CHM_OK && cudaDeviceSynchronize() != cudaSuccess) rc = CHM_ERR_CUDA;
     if (rc != CHM_OK) {

@@ -1,7 +1,7 @@
 """The wave kernel where the rules send work to it: double factors above the
 team kernel's range (here with a ragged order, an odd leading dimension and both
-signs, in the bounds-checked build too and with a wait that runs out) and float factors
-above its range where path 1 is asked for.
+signs, in the bounds-checked build too and with a wait that runs out), plans of one
+such factor, and float factors above its range where path 1 is asked for.
 
 Tolerances as in tests/common.py: float64 column-scaled 1e-11 against the
 oracle's CholeskyModifyB, float the derived bound against its mixed emulation."""
@@ -77,6 +77,22 @@ def test_ragged_padded_mixed_signs(n, k, pad, dtype):
         assert torch.all(torch.isnan(L[:, n:]))
         assert torch.equal(L[:, :n][low], L0[:, :n][low])
         assert colscaled_err(L[:, :n].cpu().numpy(), ref) <= tol
+
+
+def test_plan_of_one_factor_equals_the_call():
+    n, k = 6200, 17
+    L, V, _ = problem(n, k, 0)
+    solo = L.clone()
+    assert chm.modify(solo, V, 1) == chm.CHM_OK
+    plan = chm.BatchPlan([n], [n], [k])
+    assert plan.execute([L], [V]) == chm.CHM_OK
+    assert plan.status() == (chm.CHM_OK, [(chm.CHM_OK, -1)])
+    assert torch.equal(L, solo)
+    before = L.clone()
+    assert plan.autotune() == chm.CHM_OK and torch.equal(L, before)
+    assert plan.execute([L], [V]) == chm.CHM_OK and chm.modify(solo, V, 1) == chm.CHM_OK
+    assert plan.status()[0] == chm.CHM_OK and torch.equal(L, solo)
+    plan.close()
 
 
 CHILD = textwrap.dedent("""
