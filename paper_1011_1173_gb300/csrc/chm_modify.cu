@@ -273,21 +273,35 @@ bool use_team(long long n, long long k, int dtype)
     return false;
 }
 
+// One vector into a large double factor in page-locked host memory, which the
+// automatic rule brings to path 1, takes the wave kernel: the team kernel reads
+// the factor once for the substitution and once for the sweep, and what has left
+// L2 in between crosses the CPU-GPU link again (team / wave: n = 5000 1.74 / 1.82 ms,
+// 8000 4.4 / 4.0, 12000 9.7 / 8.0).  From the order on from which a factor on the device
+// takes the pass kernels, so that below it, and wherever path 1 is asked
+// for, a result does not depend on where the factor lies.
+static bool host_takes_wave(long long n, long long k, int dtype)
+{
+    return dtype == CHM_F64 && k == 1 && n >= 8000;
+}
+
 // The scratch of path 1 for launches of up to sh.k vectors: what this shape
 // takes and what any call of the same or a smaller size does (so that a
 // stream's workspace is never outgrown by one), whichever kernel it runs on.
 static ScratchNeed single_need(const ProbShape &sh, int dtype)
 {
     ScratchNeed need;
-    if (!use_team(sh.n, sh.k, dtype)) need = scratch_need(&sh, 1);
-    int count = 0;
-    const TeamRange *r = team_ranges(dtype, &count);
-    for (int i = 0; i < count; ++i) {
-        const ScratchNeed t = team_need_cap(ProbShape{std::min(sh.n, r[i].n), std::min(sh.k, r[i].k)});
+    auto cover = [&](const ScratchNeed &t) {
         need.iflags = std::max(need.iflags, t.iflags);
         need.progress = std::max(need.progress, t.progress);
         need.data = std::max(need.data, t.data);
-    }
+    };
+    const ProbShape one{sh.n, 1};
+    if (!use_team(sh.n, sh.k, dtype)) cover(scratch_need(&sh, 1));
+    if (host_takes_wave(sh.n, 1, dtype)) cover(scratch_need(&one, 1));
+    int count = 0;
+    const TeamRange *r = team_ranges(dtype, &count);
+    for (int i = 0; i < count; ++i) cover(team_need_cap(ProbShape{std::min(sh.n, r[i].n), std::min(sh.k, r[i].k)}));
     return need;
 }
 
@@ -513,7 +527,8 @@ static int modify_dispatch(void *L, long long n, long long ld, const void *V, lo
     if (rc != CHM_OK) return rc;
     if (n == 0 || k == 0) return info_init(d_info, 1, stream);
     if ((rc = check_reachable(L)) != CHM_OK || (rc = check_reachable(V)) != CHM_OK) return rc;
-    const PassChoice ch = choose_path(n, k, dtype, is_host_memory(L));
+    const bool host = is_host_memory(L);
+    const PassChoice ch = choose_path(n, k, dtype, host);
     if (ch.path == 2) {
         return with_pass_workspace(stream, pass_workspace_bytes(n, dtype, ch.seg), n, dtype,
                                    [&](const Scratch &sc, PassSpace &ps) {
@@ -523,9 +538,9 @@ static int modify_dispatch(void *L, long long n, long long ld, const void *V, lo
     }
     const int kw_max = (int)std::min<long long>(k, kMaxWaves);
     const ProbShape sh{n, kw_max};
+    const bool team = use_team(n, kw_max, dtype) && !(host && path_setting() == 0 && host_takes_wave(n, k, dtype));
     return with_stream_scratch(stream, single_need(sh, dtype), [&](const Scratch &sc) {
-        return enqueue_single(L, n, ld, V, ldv, k, sigma, sign, dtype, stream, d_info, sc, kw_max, true,
-                              use_team(n, kw_max, dtype));
+        return enqueue_single(L, n, ld, V, ldv, k, sigma, sign, dtype, stream, d_info, sc, kw_max, true, team);
     });
 }
 

@@ -1,7 +1,8 @@
 """The wave kernel where the rules send work to it: double factors above the
 team kernel's range (here with a ragged order, an odd leading dimension and both
 signs, in the bounds-checked build too and with a wait that runs out), plans of one
-such factor, and float factors above its range where path 1 is asked for.
+such factor, float factors above its range where path 1 is asked for, and one
+vector into a large double factor in page-locked host memory.
 
 Tolerances as in tests/common.py: float64 column-scaled 1e-11 against the
 oracle's CholeskyModifyB, float the derived bound against its mixed emulation."""
@@ -93,6 +94,16 @@ def test_plan_of_one_factor_equals_the_call():
     assert plan.execute([L], [V]) == chm.CHM_OK and chm.modify(solo, V, 1) == chm.CHM_OK
     assert plan.status()[0] == chm.CHM_OK and torch.equal(L, solo)
     plan.close()
+
+
+def test_one_vector_into_a_host_factor():
+    n = 8001
+    L, V, sig = problem(n, 1, 1)
+    ref, tol = expected(L, V, sig, n)
+    host = torch.empty(L.shape, dtype=L.dtype, pin_memory=True).copy_(L)
+    assert chm.modify(host, V, sig.tolist(), n=n) == chm.CHM_OK
+    assert chm.status_sync() == (chm.CHM_OK, -1)
+    assert colscaled_err(host[:, :n].numpy(), ref) <= tol
 
 
 CHILD = textwrap.dedent("""
