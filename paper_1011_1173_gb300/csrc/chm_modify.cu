@@ -694,8 +694,9 @@ static int noalloc_setup(int dev, NoAllocState **out)
 
 // Vectors per launch that fit the array, of the `left` asked for (0: none); the
 // last launch, of what is left, has to fit as well (fewer vectors can take more).  The
-// team kernel's launches hold whole passes, so that the passes, and with
-// them the result, are those of one launch.
+// team kernel's launches hold whole passes, so that the passes are those of one
+// launch, and with them in double the result's bits.  (In float each launch
+// rounds the diagonal that it carries in double.)
 static int noalloc_vectors(long long n, long long left, bool team)
 {
     const int k = (int)std::min<long long>(left, kMaxWaves);
