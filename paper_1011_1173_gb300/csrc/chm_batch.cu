@@ -81,7 +81,7 @@ int relayout(Plan *p)
     p->tmpl.assign(act.size(), Prob());
     for (Prob &pr : p->tmpl) memset(&pr, 0, sizeof(pr));
     if (act.empty()) return CHM_OK;
-    if (p->wave) carve(shapes.data(), 1, p->sc, p->tmpl.data());
+    if (p->wave) carve(shapes[0], p->sc, p->tmpl.data());
     else team_carve(shapes.data(), (int)shapes.size(), p->dtype, p->sc, p->tmpl.data());
     for (size_t q = 0; q < act.size(); ++q) {
         const int i = act[q];
@@ -143,8 +143,7 @@ int capture(Plan *p, int s)
         rc = CHM_ERR_CUDA;
     if (rc == CHM_OK) rc = info_init(p->d_info, p->count, cs);
     if (rc == CHM_OK && p->wave)
-        rc = launch_wave(p->dtype, nullptr, p->d_probs, nullptr, 1, p->tmpl[0].k + 1, p->tmpl[0].nb, p->sc, p->cfg,
-                         nullptr, cs);
+        rc = launch_wave(p->dtype, nullptr, p->d_probs, p->tmpl[0].k, p->sc, p->cfg, nullptr, cs);
     else if (rc == CHM_OK)
         rc = launch_team(p->dtype, nullptr, p->d_probs, (int)np, p->ntasks, p->sc, p->cfg, nullptr, cs);
     const cudaError_t ec = cudaStreamEndCapture(cs, &g);
@@ -359,7 +358,7 @@ int chm_batch_plan_create(int count, const int64_t *n, const int64_t *ld, const 
     }
     p->wave = wave_plan(shapes, dtype);
     const ScratchNeed need =
-        p->wave ? scratch_need(shapes.data(), 1) : team_need(shapes.data(), (int)shapes.size());
+        p->wave ? scratch_need(shapes[0]) : team_need(shapes.data(), (int)shapes.size());
     int rc = CHM_OK;
     if (cudaMalloc(&p->d_info, 2 * sizeof(long long) * std::max(1, count)) != cudaSuccess) rc = CHM_ERR_NOMEM;
     if (rc == CHM_OK && cudaMalloc(&p->d_probs, sizeof(Prob) * std::max<size_t>(1, shapes.size())) != cudaSuccess)

@@ -34,17 +34,15 @@ struct ProbShape {
     int k;  // waves in the launch (1 .. kMaxWaves)
 };
 
-// Scratch needed by a list of problems laid out one after another.
+// Scratch that a launch takes.
 struct ScratchNeed {
     size_t iflags = 0, progress = 0, data = 0;
-    int npairs = 0, nbmax = 0;
 };
-ScratchNeed scratch_need(const ProbShape *shapes, int count);
-
-// Fill the scratch pointers, nb, k and pair0 of problems[0..count) for the
-// layout of scratch_need(); the caller sets L, V, n, ld, ldv, down_mask and
-// info.  Returns the pair -> problem map.
-std::vector<int> carve(const ProbShape *shapes, int count, const Scratch &sc, Prob *problems);
+// A launch of the wave kernel (one problem), and the problem's scratch
+// pointers, nb and k for that layout; the caller sets L, V, n, ld, ldv,
+// down_mask and info.
+ScratchNeed scratch_need(const ProbShape &shape);
+void carve(const ProbShape &shape, const Scratch &sc, Prob *problem);
 
 // Launch configuration.
 struct LaunchCfg {
@@ -60,14 +58,11 @@ struct LaunchCfg {
 int sm_count(int dev);
 int wave_occupancy(int dtype, int dev, int *ctas_per_sm);
 long long timeout_ns();
-int default_groups(int npairs, int nsm, int nprobs);
 
-// Enqueue one launch of the wave kernel on `stream`.  Either one problem
-// (`single`, no device tables) or `nprobs` problems whose records are in
-// device memory `d_probs` with pair map `d_pair_prob`.  `trace` is null or
-// a device array of 2 * npairs * nbmax * kTracePoints words.
-int launch_wave(int dtype, const Prob *single, const Prob *d_probs, const int *d_pair_prob,
-                int nprobs, int npairs, int nbmax, const Scratch &sc, const LaunchCfg &cfg,
+// Enqueue one launch of the wave kernel on `stream`: of one problem with k
+// vectors, by value (`single`) or with its record in device memory (`d_prob`).
+// `trace` is null or a device array of 2 * (k + 1) * nb * kTracePoints words.
+int launch_wave(int dtype, const Prob *single, const Prob *d_prob, int k, const Scratch &sc, const LaunchCfg &cfg,
                 long long *trace, cudaStream_t stream);
 
 // The team kernel (chm_team.cu): scratch needed by a list of problems laid

@@ -1,5 +1,5 @@
 // Scratch layout of the wave kernel, shared by the device code and the host
-// side that carves scratch memory for one or many problems: the per-pair
+// side that carves scratch memory for a problem: the per-pair
 // data records, the flag words, the problem record and the launch control
 // words.  Plain C++ usable from host and device translation units.
 #pragma once
@@ -93,7 +93,6 @@ struct Prob {
     long long n, ld, ldv;
     int k;                         // waves of this problem in the launch (<= kMaxWaves)
     int nb;                        // column blocks of kW columns
-    int pair0;                     // index of its first pair (k waves, then the final pass)
     int ntasks;                    // team kernel: its tasks
     unsigned long long down_mask;  // bit q set: wave q is a downdate
     char *data;                    // prob_data_bytes(nb, k), 256-byte aligned

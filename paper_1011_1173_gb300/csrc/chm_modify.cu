@@ -20,43 +20,23 @@ namespace chm {
 
 // ---------------------------------------------------------------- scratch carving
 
-ScratchNeed scratch_need(const ProbShape *shapes, int count)
+ScratchNeed scratch_need(const ProbShape &shape)
 {
+    const int nb = (int)((shape.n + kW - 1) / kW), k = shape.k;
     ScratchNeed r;
-    for (int i = 0; i < count; ++i) {
-        const int nb = (int)((shapes[i].n + kW - 1) / kW);
-        const int k = shapes[i].k;
-        r.iflags += prob_iflags(nb, k);
-        r.progress += prob_progress(nb, k);
-        r.data += prob_data_bytes(nb, k);
-        r.npairs += k + 1;  // its waves and the final pass
-        r.nbmax = std::max(r.nbmax, nb);
-    }
+    r.iflags = prob_iflags(nb, k);
+    r.progress = prob_progress(nb, k);
+    r.data = prob_data_bytes(nb, k);
     return r;
 }
 
-std::vector<int> carve(const ProbShape *shapes, int count, const Scratch &sc, Prob *problems)
+void carve(const ProbShape &shape, const Scratch &sc, Prob *problem)
 {
-    std::vector<int> pair_prob;
-    size_t fi = 0, fp = 0, fd = 0;
-    int pair = 0;
-    for (int i = 0; i < count; ++i) {
-        const int nb = (int)((shapes[i].n + kW - 1) / kW);
-        const int k = shapes[i].k;
-        Prob &p = problems[i];
-        p.nb = nb;
-        p.k = k;
-        p.pair0 = pair;
-        p.iflags = sc.iflags + fi;
-        p.progress = sc.progress + fp;
-        p.data = sc.data + fd;
-        fi += prob_iflags(nb, k);
-        fp += prob_progress(nb, k);
-        fd += prob_data_bytes(nb, k);
-        pair_prob.insert(pair_prob.end(), (size_t)k + 1, i);
-        pair += k + 1;
-    }
-    return pair_prob;
+    problem->nb = (int)((shape.n + kW - 1) / kW);
+    problem->k = shape.k;
+    problem->iflags = sc.iflags;
+    problem->progress = sc.progress;
+    problem->data = sc.data;
 }
 
 // ---------------------------------------------------------------- device facts
@@ -115,28 +95,25 @@ int wave_occupancy(int dtype, int dev, int *ctas_per_sm)
     return dtype == CHM_F64 ? occupancy<double>(dev, ctas_per_sm) : occupancy<float>(dev, ctas_per_sm);
 }
 
-// Groups: one per concurrently running wave.  One problem: about seven sweep
-// SMs per group (its waves share the sweep work of one factor), and up to
-// nsm / 8 groups, so that a rank-16 modification runs all its waves and its
-// final pass at once (measured at n = 5000, k = 16: 17 groups 1.88 ms, 16
-// groups 1.99 ms, 12 groups 2.43 ms); many independent problems: two sweep
-// SMs per group, since more chains in flight matter more than sweep
-// capacity per chain (measured on the batched workload: 50 groups 31 ms,
-// 16 groups 59 ms).
-int default_groups(int npairs, int nsm, int nprobs)
+// Groups: one per concurrently running wave.  About seven sweep SMs per group
+// (its waves share the sweep work of the factor), and up to nsm / 8 groups, so
+// that a rank-16 modification runs all its waves and its final pass at once
+// (measured at n = 5000, k = 16: 17 groups 1.88 ms, 16 groups 1.99 ms, 12
+// groups 2.43 ms).
+static int default_groups(int npairs, int nsm)
 {
     int g = env_int("CHM_GROUPS");
-    if (g <= 0) g = std::max(1, nprobs > 1 ? nsm / 3 : nsm / 8);
+    if (g <= 0) g = std::max(1, nsm / 8);
     return std::max(1, std::min(std::min(g, npairs), std::min(kMaxGroups, nsm / 2)));
 }
 
 // ---------------------------------------------------------------- launch
 
 template <typename T>
-static int launch_t(const Prob *single, const Prob *d_probs, const int *d_pair_prob, int nprobs,
-                    int npairs, int nbmax, const Scratch &sc, const LaunchCfg &cfg, long long *trace,
-                    cudaStream_t stream)
+static int launch_t(const Prob *single, const Prob *d_prob, int k, const Scratch &sc, const LaunchCfg &cfg,
+                    long long *trace, cudaStream_t stream)
 {
+    const int npairs = k + 1;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return CHM_ERR_CUDA;
     int bps = 0;
@@ -144,21 +121,18 @@ static int launch_t(const Prob *single, const Prob *d_probs, const int *d_pair_p
     if (rc != CHM_OK) return rc;
     if (cfg.ctas_per_sm > 0) bps = std::min(bps, cfg.ctas_per_sm);
     const int nsm = sm_count(dev);
-    if (nsm < 2 || nsm > kMaxSm || npairs < 1) return CHM_ERR_ARG;
+    if (nsm < 2 || nsm > kMaxSm || k < 1) return CHM_ERR_ARG;
     const int grid = cfg.grid > 0 ? std::max(2, std::min(cfg.grid, nsm * bps)) : nsm * bps;
     // SMs the launch can hold at the occupancy limit
     const int nsm_eff = std::max(2, std::min(nsm, grid / bps));
-    int G = cfg.groups > 0 ? cfg.groups : default_groups(npairs, nsm_eff, nprobs);
+    int G = cfg.groups > 0 ? cfg.groups : default_groups(npairs, nsm_eff);
     G = std::max(1, std::min(std::min(G, npairs), std::min(kMaxGroups, nsm_eff / 2)));
     Launch<T> P;
     memset(&P, 0, sizeof(P));
-    P.probs = d_probs;
+    P.prob = d_prob;
     if (single) P.prob0 = *single;
-    P.pair_prob = d_pair_prob;
-    P.nprobs = nprobs;
     P.npairs = npairs;
     P.ngroups = G;
-    P.nbmax = nbmax;
     P.ctl = sc.ctl;
     P.status = sc.status;
     P.trace = trace;
@@ -175,13 +149,11 @@ static int launch_t(const Prob *single, const Prob *d_probs, const int *d_pair_p
     return cudaGetLastError() == cudaSuccess ? CHM_OK : CHM_ERR_CUDA;
 }
 
-int launch_wave(int dtype, const Prob *single, const Prob *d_probs, const int *d_pair_prob, int nprobs,
-                int npairs, int nbmax, const Scratch &sc, const LaunchCfg &cfg, long long *trace,
-                cudaStream_t stream)
+int launch_wave(int dtype, const Prob *single, const Prob *d_prob, int k, const Scratch &sc, const LaunchCfg &cfg,
+                long long *trace, cudaStream_t stream)
 {
-    if (dtype == CHM_F64)
-        return launch_t<double>(single, d_probs, d_pair_prob, nprobs, npairs, nbmax, sc, cfg, trace, stream);
-    return launch_t<float>(single, d_probs, d_pair_prob, nprobs, npairs, nbmax, sc, cfg, trace, stream);
+    return dtype == CHM_F64 ? launch_t<double>(single, d_prob, k, sc, cfg, trace, stream)
+                            : launch_t<float>(single, d_prob, k, sc, cfg, trace, stream);
 }
 
 __global__ void info_init_kernel(long long *info, int count)
@@ -297,8 +269,8 @@ static ScratchNeed single_need(const ProbShape &sh, int dtype)
         need.data = std::max(need.data, t.data);
     };
     const ProbShape one{sh.n, 1};
-    if (!use_team(sh.n, sh.k, dtype)) cover(scratch_need(&sh, 1));
-    if (host_takes_wave(sh.n, 1, dtype)) cover(scratch_need(&one, 1));
+    if (!use_team(sh.n, sh.k, dtype)) cover(scratch_need(sh));
+    if (host_takes_wave(sh.n, 1, dtype)) cover(scratch_need(one));
     int count = 0;
     const TeamRange *r = team_ranges(dtype, &count);
     for (int i = 0; i < count; ++i) cover(team_need_cap(ProbShape{std::min(sh.n, r[i].n), std::min(sh.k, r[i].k)}));
@@ -468,7 +440,7 @@ static int enqueue_single(void *L, long long n, long long ld, const void *V, lon
         memset(&pr, 0, sizeof(pr));
         const ProbShape sh{n, kw};
         if (team) team_carve(&sh, 1, dtype, sc, &pr);
-        else carve(&sh, 1, sc, &pr);
+        else carve(sh, sc, &pr);
         pr.L = L;
         pr.V = static_cast<const char *>(V) + (size_t)q0 * ldv * elt;
         pr.n = n;
@@ -494,7 +466,7 @@ static int enqueue_single(void *L, long long n, long long ld, const void *V, lon
         LaunchCfg cfg;
         cfg.skip_publish = take_test_skip();
         rc = team ? launch_team(dtype, &pr, nullptr, 1, pr.ntasks, sc, cfg, trace, stream)
-                  : launch_wave(dtype, &pr, nullptr, nullptr, 1, kw + 1, nb, sc, cfg, trace, stream);
+                  : launch_wave(dtype, &pr, nullptr, kw, sc, cfg, trace, stream);
         if (rc != CHM_OK) return rc;
     }
     return CHM_OK;
@@ -702,7 +674,7 @@ static int noalloc_vectors(long long n, long long left, bool team)
     const int k = (int)std::min<long long>(left, kMaxWaves);
     auto fits = [&](int kw) {
         const ProbShape sh{n, kw};
-        const ScratchNeed need = team ? team_need(&sh, 1) : scratch_need(&sh, 1);
+        const ScratchNeed need = team ? team_need(&sh, 1) : scratch_need(sh);
         return need.iflags <= kNoAllocIflags && need.progress <= kNoAllocProgress &&
                need.data <= kNoAllocBytes - kNoAllocDataOff;
     };

@@ -1,12 +1,11 @@
 // Wave-pipelined rank-k up/downdate kernel (Walder 2010, Algorithm 1, with
-// the CPU/GPU panelling of Sec. 4 replaced by one device-resident launch
-// that may carry many independent factors).
+// the CPU/GPU panelling of Sec. 4 replaced by one device-resident launch).
 //
 // A rank-k modification is k waves: wave q is the rank-1 modification of the
 // factor left by waves < q by column q of V (Sec. 4.1 processes columns in
 // order; any dependency-respecting order gives the same factor).  A launch
-// holds one or more problems (factor, V, signs); a (problem, wave) pair is
-// the unit of scheduling.
+// holds one problem (factor, V, signs); the unit of scheduling is a pair, one
+// of its waves or its final pass.
 //
 // Per wave, with F the current factor and v the vector (sign sigma):
 //   chain:  p = F^{-T} v (forward substitution), T_0 = 1, T_{i+1} = T_i + sigma p_i^2,
@@ -39,12 +38,12 @@
 //     held in registers.  It also publishes what the wave block needs: the
 //     carry z for the block, the carry u_hat at the diagonal, and the next
 //     wave's dot-product matrix.
-// A pair waits only on itself and on the previous wave of its problem, which
+// A pair waits only on itself and on the previous wave, which
 // was taken from the counter earlier and is running or done, so the launch
 // always progresses.  Every wait is bounded (%globaltimer).
 //
 // Storage between waves of one launch: the diagonal holds true values, an
-// off-diagonal L_ij is held as S_ij = L_ij / e_i.  Each problem's last pair
+// off-diagonal L_ij is held as S_ij = L_ij / e_i.  The problem's last pair
 // is a final pass that multiplies the last wave's scales back in, trailing
 // that wave tile by tile.
 #pragma once
@@ -56,13 +55,12 @@ namespace chm {
 
 template <typename T>
 struct Launch {
-    const Prob *probs;      // device array [nprobs]; null: the one problem is prob0
+    const Prob *prob;       // the problem in device memory; null: it is prob0
     Prob prob0;
-    const int *pair_prob;   // device array [npairs]: problem of each pair; null: all 0
-    int nprobs, npairs, ngroups, nbmax;
+    int npairs, ngroups;    // pairs: the problem's waves and its final pass
     int *ctl;               // kCtlInts control words
     long long *status;      // sticky {status, row} of the scratch owner
-    long long *trace;       // optional timestamps, [2][npairs][nbmax][kTracePoints]
+    long long *trace;       // optional timestamps, [2][npairs][nb][kTracePoints]
     long long timeout_ns;
     int skip_publish;       // test hook: wave blocks never release this block's panel (-1: none)
     // the workspace allocations the problems' regions are carved from (bounds-checked builds)
@@ -106,10 +104,9 @@ struct Wave {
 template <typename T>
 __device__ Wave<T> make_wave(const Launch<T> &P, int j)
 {
-    const int i = P.pair_prob ? __ldg(P.pair_prob + j) : 0;
-    const Prob pr = P.probs ? P.probs[i] : P.prob0;
+    const Prob pr = P.prob ? *P.prob : P.prob0;
     Wave<T> w;
-    const int q = j - pr.pair0, nb = pr.nb;
+    const int q = j, nb = pr.nb;
     const PairRec rc = pair_rec(nb);
     char *d = pr.data + (size_t)q * rc.bytes;
     w.L = static_cast<T *>(pr.L);
@@ -142,9 +139,9 @@ __device__ Wave<T> make_wave(const Launch<T> &P, int j)
     w.ctag = pr.progress + (size_t)pr.k * nb * (1 + kW * 2) + (size_t)q * nb * kW * 2;
     w.final_done = pr.progress + prob_final_done(nb, pr.k);
     if (P.trace) {
-        const size_t row = (size_t)j * P.nbmax * kTracePoints;
+        const size_t row = (size_t)j * nb * kTracePoints;
         w.trace_sweep = P.trace + row;
-        w.trace_wave = P.trace + (size_t)P.npairs * P.nbmax * kTracePoints + row;
+        w.trace_wave = P.trace + (size_t)P.npairs * nb * kTracePoints + row;
     } else {
         w.trace_sweep = w.trace_wave = nullptr;
     }
@@ -887,11 +884,10 @@ __device__ __forceinline__ int role_code(int role, int group) { return role | (g
 template <typename T>
 __device__ __forceinline__ unsigned long long *task_range(const Launch<T> &P, int j, int *first, int *nb)
 {
-    const int i = P.pair_prob ? __ldg(P.pair_prob + j) : 0;
-    const Prob *pr = P.probs ? P.probs + i : &P.prob0;
-    *first = j > pr->pair0 ? 1 : 0;  // block 0 of a later wave has no off-diagonal tile
+    const Prob *pr = P.prob ? P.prob : &P.prob0;
+    *first = j > 0 ? 1 : 0;  // block 0 of a later wave has no off-diagonal tile
     *nb = pr->nb;
-    return reinterpret_cast<unsigned long long *>(pr->progress + prob_ticket(pr->nb, pr->k, j - pr->pair0));
+    return reinterpret_cast<unsigned long long *>(pr->progress + prob_ticket(pr->nb, pr->k, j));
 }
 // Take one sweep task: from the own group's current pair first, then, when
 // it has no task left, from another group's pair that is lower than the own
@@ -956,7 +952,7 @@ template <typename T>
 __global__ void __launch_bounds__(128, 3) wave_kernel(Launch<T> P)
 {
     extern __shared__ __align__(16) unsigned char chm_smem[];
-    __shared__ int s_role, s_pair, s_last, s_abort;
+    __shared__ int s_role, s_pair, s_last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int *ctl = P.ctl;
     SyncArgs sy;  // launch-level waits
@@ -1089,16 +1085,11 @@ __global__ void __launch_bounds__(128, 3) wave_kernel(Launch<T> P)
     __syncthreads();
     if (s_last) {
         __threadfence();
-        // A wait that ran out aborted the whole launch: every problem that
-        // recorded nothing stopped unfinished, so it is marked too (info -5:
-        // stopped by another problem's failure) and none reads as complete.
-        if (threadIdx.x == 0) s_abort = ld_relaxed_gpu(ctl + kCtlAbort);
-        __syncthreads();
-        if (s_abort) {
-            for (int i = threadIdx.x; i < P.nprobs; i += blockDim.x) {
-                long long *info = P.probs ? P.probs[i].info : P.prob0.info;
-                if (info) record_one(info, kStatusTimeout, -5);
-            }
+        // A wait that ran out aborted the launch: the problem is marked
+        // unfinished (info -5) if the wait did not say so itself.
+        if (threadIdx.x == 0 && ld_relaxed_gpu(ctl + kCtlAbort) != 0) {
+            long long *info = P.prob ? P.prob->info : P.prob0.info;
+            if (info) record_one(info, kStatusTimeout, -5);
         }
         __syncthreads();
         for (int i = threadIdx.x; i < kCtlInts; i += blockDim.x)
