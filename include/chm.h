@@ -69,7 +69,7 @@
  *     says which build is loaded (1 checked, 0 not).
  *   - Memory.  The library keeps a workspace per (device, stream): per
  *     vector of a launch (at most 64 per launch) coefficients, residuals,
- *     matrices and flags of at most about 42 KB per 32 rows, and the status
+ *     matrices and flags of at most about 43 KB per 32 rows, and the status
  *     word
  *     (chm_workspace_bytes gives the total).  It is allocated on the first
  *     call that needs a larger one; later calls of the same or smaller size
@@ -181,7 +181,8 @@ int chm_modify_noalloc(void *L, int64_t n, int64_t ld, const void *V, int64_t ld
  * Batched up/downdate of many independent factors (a systems form of the
  * method; Sec. 4.1's rank-k blocking applied to each factor).  A plan fixes
  * the shapes; each execution takes the factors' and update blocks' device
- * addresses and runs every factor in ONE launch of the team kernel, replayed
+ * addresses and runs every factor in ONE launch (of the team kernel; a plan of
+ * one factor in double on the kernel that a single call takes), replayed
  * from a CUDA graph captured by the plan (a copy of the problem table from
  * pinned host memory, a reset of the per-factor status words, the launch).
  *
@@ -195,13 +196,13 @@ int chm_modify_noalloc(void *L, int64_t n, int64_t ld, const void *V, int64_t ld
  *   plan    receives the plan
  * Factors with n_i == 0 or k_i == 0 are no-ops.  V_i is n_i x k_i
  * column-major with leading dimension n_i.  The plan owns all device scratch
- * (at most about 42 KB per vector and 32 rows of every factor) and pinned staging memory;
+ * (at most about 43 KB per vector and 32 rows of every factor) and pinned staging memory;
  * nothing is allocated by chm_batch_execute.  The current device at creation
  * is the plan's device.  Returns CHM_OK, CHM_ERR_ARG, CHM_ERR_NOMEM or
  * CHM_ERR_CUDA.
  *
  * chm_batch_autotune: times candidate launch configurations (teams of thread
- * blocks that share a factor, blocks per SM, largest-work-first or caller order) on synthetic factors of
+ * blocks that share a factor, on the wave kernel SM groups; blocks per SM, largest-work-first or caller order) on synthetic factors of
  * the plan's shapes (L = I, V = 1e-3, allocated for the duration of the call)
  * and keeps the fastest.  Synchronises `stream`.  The plan's status words
  * are reset.  Returns CHM_OK, CHM_ERR_NOMEM (no room for the synthetic
@@ -245,8 +246,9 @@ int chm_batch_plan_destroy(void *plan);
  * launch formed from requests that arrived while another was running
  * overlaps it on the device.  Requests on one factor run one after another
  * in submission order, each in its own launch; a factor's result is
- * bit-identical to applying the same requests alone with chm_modify_ex
- * where that runs the team kernel too (chm_config_set).
+ * bit-identical to applying the same requests alone with chm_modify_ex on
+ * path 1 where that runs the team kernel too: orders up to 8192, in double with
+ * more than 16 vectors up to 6144 (chm_config_set).
  *
  * chm_server_create
  *   hbm_budget_bytes  device memory the server may hold: factors (n^2
@@ -457,8 +459,13 @@ int chm_microbench(int which, double *out, int nout);
  * 5500 only) or 256 MB in double (with one vector; two above order 12000, up
  * to 8 above 16384), and for a factor of order >= 64 in page-locked host
  * memory modified by two or more vectors (it then crosses the CPU-GPU link
- * three times per pass of up to 16 vectors; the wave kernel twice per
- * vector).
+ * three times per pass of up to 16 vectors; on path 1 about once per vector
+ * and twice per eight).  One vector into a double factor of order 8000 or more
+ * in page-locked host memory takes the wave kernel where the path is automatic.
+ * Accuracy: path 1 is backward stable like Algorithm 1 itself.  The pass
+ * kernels' coefficients come from prefix Grams: in double with two or more
+ * vectors their backward error grows as 2^-53 times the squared size of
+ * F^{-T} V (F = 1e-2 I and vectors of size 1: 1e-12).
  * chm_config_get also answers "pass_d_f32", "pass_d_f64", "pass_kb_f32"
  * and "pass_kb_f64" (the values in effect, tuning cache aside) and
  * "checked" (1 in the bounds-checked build).  The bounds-checked

@@ -114,9 +114,10 @@ int path_setting()
 //   (pass / team kernel, n = 8192: k = 1 1.08 / 0.78 ms, k = 2 1.6 / 1.0, k = 8 5.6 /
 //   2.1; n = 16384: k = 1 1.8 / 2.4, k = 2 2.8 / 3.3, k = 4 4.8 / 4.3, k = 8 9.5 / 7.4 on the wave kernel;
 //   n = 32768: k = 4 12.6 / 16.0);
-// and for a factor in page-locked host memory with two or more vectors (the
-// pass crosses the CPU-GPU link three times per block of vectors, the wave
-// kernel twice per vector).
+// and for a factor in page-locked host memory with two or more vectors (a
+// pass crosses the CPU-GPU link three times per block of up to 16 vectors; of
+// path 1's kernels the team kernel once per vector and twice per eight, the
+// wave kernel twice per vector, once the factor has left L2).
 static bool rule_pass(long long n, long long k, int dtype, bool host_factor)
 {
     if (host_factor) return n >= 64 && k >= 2;

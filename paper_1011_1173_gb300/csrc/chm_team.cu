@@ -84,9 +84,9 @@ int occupancy(int dev, int *bps_out)
 
 // Teams: one for a single problem; for many, about fourteen blocks each, so
 // that the largest problems, which start first, end with the rest (512
-// factors of order 64 to 4096 in double, two executions: 75.1 ms with 14
-// blocks a team against 76.2 with 28 and 76.9 with four; 96 float factors
-// up to order 2048: 4.7 against 4.7 and 5.5 ms).
+// factors of order 64 to 4096 in double, two executions: 54.0 ms with 14
+// blocks a team against 54.3 with 28 and 55.0 with four; 96 float factors
+// up to order 2048, 608 blocks: 4.1 ms with 14, 3.9 with 38 and 4.5 with four).
 int default_teams(int nprobs, int grid)
 {
     const char *e = getenv("CHM_GROUPS");

@@ -37,14 +37,15 @@
 // chain: the sweep trails it by one segment, whatever the number of vectors.
 // With many vectors or factors the FP64 rate binds (three FMAs per element
 // and vector: one in the substitution, two in the sweep).  n = 5000 in double,
-// one call: k = 1 0.37 ms (the wave kernel 1.08), k = 16 1.68 ms (1.97), of
+// one call: k = 1 0.38 ms (the wave kernel 1.04), k = 16 1.69 ms (1.93), of
 // which the FMAs are 0.05 and 1.1 ms.
 //
-// Precision: CHM_F64 is double throughout.  CHM_F32_MIXED substitutes in
-// double (P, U, G) with the far sums in pairs of floats (48 bits), forms the
-// coefficients in double, and sweeps in float; the diagonal is carried in
-// double through all passes of the launch and rounded to float at the end of
-// each.
+// Precision: CHM_F64 is double throughout; what the identities would lose
+// where Grams or diagonal blocks are ill-conditioned is avoided (Carried,
+// is_hard).  CHM_F32_MIXED substitutes in double (P, U, G) with the far sums in
+// pairs of floats (48 bits), forms the coefficients in double, and sweeps in
+// float; the diagonal is carried in double through all passes of the launch and
+// rounded to float at the end of each.
 #pragma once
 
 #include "chm_sub.cuh"
