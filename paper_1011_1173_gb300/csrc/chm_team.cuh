@@ -131,7 +131,7 @@ struct CoefSmem {
     double l0[ne];               // the factor handed on by the block before, |D_q| on its diagonal
     unsigned ill[kWarps];        // per warp: four bits a row, set where its Gram is ill-conditioned
     double M[ne];                // from l0 on: the Gram behind the block, then its factor, |D_q| on the diagonal
-    int have;                    // a factor was handed on
+    int have;                    // what the block before has handed on
 };
 // A sweep task's segments: NV warps pass a tile on, so NV + 1 tiles are in
 // flight per segment.
@@ -798,6 +798,8 @@ __device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem 
     while ((q + 1) * (q + 2) / 2 <= x) ++q;
     const int r = x - q * (q + 1) / 2;
     const bool in = mine && q < kb;
+    enum { kHanded, kTakeGram, kFailed };
+    int from = kHanded;
     bool handed = false;  // the block starts from a factor handed on, S.l0
     bool early = false;   // (last warp) the next block has its factor
     for (;;) {
@@ -889,13 +891,11 @@ __device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem 
             }
             nan = __any_sync(kFull, nan);
             inf = __any_sync(kFull, inf);
-            if (lane == 0) {
-                S.have = !nan && !inf;
-                if (inf && !nan) S.ill[0] &= ~0xfu;
-            }
+            if (lane == 0) S.have = nan ? kFailed : inf ? kTakeGram : kHanded;
         }
         __syncthreads();
-        if (!S.have) break;
+        from = S.have;
+        if (from != kHanded) break;
         // p becomes L0^{-1} p
         double *y = S.p0[row];
         for (int j = 0; j + 1 < kb; ++j) {
@@ -910,9 +910,10 @@ __device__ void coef_task(const Launch<T> &P, const View<T> &v, int b, CoefSmem 
     int first = kW, last = -1;
 #pragma unroll
     for (int m = kWarps - 1; m >= 0; --m) {
-        if (!S.ill[m]) continue;
-        first = m * 8 + ((__ffs(S.ill[m]) - 1) >> 2);
-        last = max(last, m * 8 + ((31 - __clz(S.ill[m])) >> 2));
+        const unsigned rowm = S.ill[m] & (m == 0 && from == kTakeGram ? ~0xfu : ~0u);
+        if (!rowm) continue;
+        first = m * 8 + ((__ffs(rowm) - 1) >> 2);
+        last = max(last, m * 8 + ((31 - __clz(rowm)) >> 2));
     }
     if (first > 0 && last >= 0) {
         // (row 0 is ill-conditioned only behind a row that has failed)
